@@ -2,12 +2,11 @@
 // grouped launches, CUDA-graph replay and the schedule autotuner.
 //
 // Every pattern gets an ordinary transform plan (exact SNF and tables, the
-// same device code as pfft_forward) restricted to the generic shared-memory
-// kernels, whose tables are sub-allocated from one arena.  A schedule turns
+// same device code as pfft_forward) restricted to the mixed-radix tiles of
+// fft_mixed.cuh, whose tables are sub-allocated from one arena.  A schedule turns
 // the plans into grouped launches: for each pass, the patterns are grouped by
-// the shared-memory footprint of their tile into at most kMaxBuckets
-// launches (so that small tiles are not held to the occupancy of the largest
-// one), those launches run concurrently on forked streams, and inside a
+// the threads of their tile into at most kMaxBuckets launches (so that small
+// tiles are not held to the occupancy of the largest one), those launches run concurrently on forked streams, and inside a
 // launch the CTAs of the costliest tiles come first.  The split level of every
 // pattern is one more grouped launch.  The autotuner times candidate tile
 // budgets and orders on the real batch and keeps the fastest.
@@ -26,12 +25,14 @@
 using namespace pfft;
 
 namespace {
-constexpr int kMaxBuckets = 5;
-// upper ends of the shared-memory classes of a grouped pass launch (bytes)
-constexpr int kSmemClass[kMaxBuckets] = {24 * 1024, 48 * 1024, 72 * 1024, 112 * 1024, kGroupedMaxDynSmem};
+constexpr int kMaxBuckets = 6;
+// Upper ends of the thread classes of a grouped pass launch: every CTA of a
+// launch has the threads of its largest tile, and a tile's idle warps hold
+// registers and wait at its barriers.
+constexpr int kThreadClass[kMaxBuckets] = {128, 256, 384, 512, 768, 1024};
 
 struct Bucket {
-  int cols = 0, n = 0, nctas = 0, threads = 0, smem = 0;
+  int n = 0, nctas = 0, threads = 0, smem = 0;
   size_t items_off = 0, cta0_off = 0;  // byte offsets into the schedule buffer
 };
 }  // namespace
@@ -53,7 +54,7 @@ struct pfft_batch_s {
   void* ws = nullptr;
   void* sched = nullptr;  // device: items and first-CTA tables of all launches
   std::vector<Bucket> rows, cols, splits, primes;
-  int row_budget = 8192, col_budget = 8192, order = 1, max2 = 16;
+  int row_budget = 4096, col_budget = 4096, order = 1, max2 = 16;
   std::vector<int> ident;  // patterns with m = 1 (the transform is a copy)
   cudaStream_t cap = nullptr;
   std::vector<cudaStream_t> streams;
@@ -63,7 +64,7 @@ struct pfft_batch_s {
   // single launch (PFFT_BATCH_ONE_LAUNCH): the queue's tables in the schedule
   // buffer (pointers filled per call), its counters and status word
   QueueArgs q{};
-  int q_units = 0, q_smem = 0;
+  int q_units = 0, q_threads = 0, q_smem = 0;
   size_t q_off[14] = {};
   int* qmem = nullptr;  // [0] status, then the counters of QueueArgs
   unsigned spin_limit = kSpinLimit;
@@ -86,28 +87,28 @@ size_t ebytes(int dtype) { return dtype == PFFT_C64 ? 8 : 16; }
 
 // Relative cost of one CTA of a pass: its elements times the per-element work
 // of its stages (direct prime stages cost about R / 4 radix-2 butterflies).
-double tile_cost(const PassArgs& a) {
+double tile_cost(const MixDesc& a) {
   double w = 0;
   for (int i = 0; i < a.nstages; ++i) {
     const int R = a.st[i].R;
-    w += R >= kMinDirectRadix ? R / 4.0 : std::log2(double(R));
+    w += R >= kMixMinDirect ? R / 4.0 : std::log2(double(R));
   }
   return double(a.T) * a.L * (w + 2.0);
 }
 
 struct Item {
-  PassArgs a;
+  MixDesc a;
   int pattern;
   double cost;
 };
 
-// Group items into launches by shared-memory class; order each launch.
-void make_buckets(std::vector<Item>& items, int cols, int order, std::vector<Bucket>& out,
+// Group items into launches by thread class; order each launch.
+void make_buckets(std::vector<Item>& items, int order, std::vector<Bucket>& out,
                   std::vector<std::vector<Item>>& groups) {
   std::vector<std::vector<Item>> g(kMaxBuckets);
   for (auto& it : items) {
     int c = 0;
-    while (c + 1 < kMaxBuckets && it.a.smem_bytes > kSmemClass[c]) ++c;
+    while (c + 1 < kMaxBuckets && it.a.nthreads > kThreadClass[c]) ++c;
     g[c].push_back(it);
   }
   for (auto& v : g) {
@@ -115,7 +116,6 @@ void make_buckets(std::vector<Item>& items, int cols, int order, std::vector<Buc
     if (order == 1)
       std::stable_sort(v.begin(), v.end(), [](const Item& x, const Item& y) { return x.cost > y.cost; });
     Bucket b;
-    b.cols = cols;
     b.n = int(v.size());
     int tmax = 1;
     for (auto& it : v) {
@@ -124,9 +124,9 @@ void make_buckets(std::vector<Item>& items, int cols, int order, std::vector<Buc
       b.smem = std::max(b.smem, it.a.smem_bytes);
       tmax = std::max(tmax, it.a.T);
     }
-    // a column pass keeps one column per thread: the block size must be a
-    // multiple of every item's T (powers of two up to 512)
-    if (cols && b.threads % tmax) b.threads = (b.threads + tmax - 1) / tmax * tmax;
+    // a thread keeps one pencil of a tile that holds them side by side: the
+    // block size must be a multiple of every item's T (powers of two up to 64)
+    if (b.threads % tmax) b.threads = (b.threads + tmax - 1) / tmax * tmax;
     out.push_back(b);
     groups.push_back(std::move(v));
   }
@@ -142,29 +142,21 @@ pfft_status build_schedule(pfft_batch_s& B) {
     if (st != PFFT_OK) return st;
     const double scale = 1.0 / std::sqrt(double(P->m));
     const uintptr_t boff = uintptr_t(B.off[i]) * eb;
-    PassArgs r = P->rowp;
-    r.batch = 1;
+    // one tile per signal, or the row pass and the column pass
+    const bool whole = P->mixed[MIX_WHOLE], single = whole || P->pen.empty();
+    MixDesc r = P->mix[whole ? MIX_WHOLE : MIX_ROW];
     r.load_mode = MAP_BOX_H;
-    r.conj_in = r.conj_out = 0;
+    r.store_mode = single ? MAP_BOX_G : MAP_WS;
+    r.scale = single ? scale : 1.0;
     r.in_sel = 0;
+    r.out_sel = single ? 2 : 1;
     r.in = reinterpret_cast<const void*>(boff);
     r.out = reinterpret_cast<void*>(boff);
-    if (P->pen.empty()) {
-      r.store_mode = MAP_BOX_G;
-      r.scale = scale;
-      r.out_sel = 2;
-    } else {
-      r.store_mode = MAP_WS;
-      r.scale = 1.0;
-      r.out_sel = 1;
-    }
     rows.push_back({r, i, tile_cost(r)});
-    if (!P->pen.empty()) {
-      PassArgs c = P->colp;
-      c.batch = 1;
+    if (!single) {
+      MixDesc c = P->mix[MIX_COL];
       c.load_mode = MAP_WS;
       c.store_mode = MAP_BOX_G;
-      c.conj_in = c.conj_out = 0;
       c.scale = scale;
       c.in_sel = 1;
       c.out_sel = 2;
@@ -175,8 +167,8 @@ pfft_status build_schedule(pfft_batch_s& B) {
   }
   std::vector<Bucket> rb, cb, sb;
   std::vector<std::vector<Item>> rg, cg;
-  make_buckets(rows, 0, B.order, rb, rg);
-  make_buckets(cols, 1, B.order, cb, cg);
+  make_buckets(rows, B.order, rb, rg);
+  make_buckets(cols, B.order, cb, cg);
   // split launch: one item per pattern, costliest first
   std::vector<int> sorder;
   for (int i = 0; i < int(B.sitems.size()); ++i) sorder.push_back(i);
@@ -204,13 +196,13 @@ pfft_status build_schedule(pfft_batch_s& B) {
     return c0;
   };
   auto put_group = [&](Bucket& b, const std::vector<Item>& v) {
-    std::vector<PassArgs> a(v.size());
+    std::vector<MixDesc> a(v.size());
     std::vector<int> c0(v.size() + 1, 0);
     for (size_t k = 0; k < v.size(); ++k) {
       a[k] = v[k].a;
       c0[k + 1] = c0[k] + v[k].a.groups;
     }
-    b.items_off = put(a.data(), a.size() * sizeof(PassArgs));
+    b.items_off = put(a.data(), a.size() * sizeof(MixDesc));
     const std::vector<int> t = with_map(c0);
     b.cta0_off = put(t.data(), t.size() * sizeof(int));
   };
@@ -259,9 +251,9 @@ pfft_status build_schedule(pfft_batch_s& B) {
   // list in the buckets' order, with first units, patterns and the patterns'
   // tile counts
   if (B.flags & PFFT_BATCH_ONE_LAUNCH) {
-    std::vector<PassArgs> qa;
+    std::vector<MixDesc> qa;
     std::vector<int> u0(1, 0), pat, need_r(B.n, 0), need_c(B.n, 0);
-    int smem = 0;
+    int smem = 0, threads = kMaxThreads;
     auto pass_list = [&](const std::vector<std::vector<Item>>& groups, std::vector<int>& need, size_t* o) {
       qa.clear();
       u0.assign(1, 0);
@@ -273,8 +265,9 @@ pfft_status build_schedule(pfft_batch_s& B) {
           pat.push_back(it.pattern);
           need[it.pattern] += it.a.groups;
           smem = std::max(smem, it.a.smem_bytes);
+          threads = std::max(threads, it.a.nthreads);
         }
-      o[0] = qa.empty() ? 0 : put(qa.data(), qa.size() * sizeof(PassArgs));
+      o[0] = qa.empty() ? 0 : put(qa.data(), qa.size() * sizeof(MixDesc));
       o[1] = put(u0.data(), u0.size() * sizeof(int));
       o[2] = pat.empty() ? 0 : put(pat.data(), pat.size() * sizeof(int));
       return std::make_pair(int(qa.size()), u0.back());
@@ -322,6 +315,7 @@ pfft_status build_schedule(pfft_batch_s& B) {
     B.q_off[13] = put(need_c.data(), need_c.size() * sizeof(int));
     B.q.npat = B.n;
     B.q_smem = smem;
+    B.q_threads = (threads + 63) / 64 * 64;  // a multiple of every column tile's T
     B.q_units = B.q.u_rows + B.q.u_cols + B.q.u_splits + B.q.u_primes;
   }
   void* dev = nullptr;
@@ -356,10 +350,10 @@ pfft_status enqueue(pfft_batch_s& B, const void* in, void* chat, void* sc, void*
   if (B.flags & PFFT_BATCH_ONE_LAUNCH) {
     QueueArgs q = B.q;
     auto at = [&](int i) { return static_cast<const void*>(sched + B.q_off[i]); };
-    q.rows = static_cast<const PassArgs*>(at(0));
+    q.rows = static_cast<const MixDesc*>(at(0));
     q.row_u0 = static_cast<const int*>(at(1));
     q.row_pat = static_cast<const int*>(at(2));
-    q.cols = static_cast<const PassArgs*>(at(3));
+    q.cols = static_cast<const MixDesc*>(at(3));
     q.col_u0 = static_cast<const int*>(at(4));
     q.col_pat = static_cast<const int*>(at(5));
     q.splits = static_cast<const SplitItem*>(at(6));
@@ -381,18 +375,18 @@ pfft_status enqueue(pfft_batch_s& B, const void* in, void* chat, void* sc, void*
     if (!(sc && wv)) q.u_splits = q.u_primes = 0;
     const int units = q.u_rows + q.u_cols + q.u_splits + q.u_primes;
     if (cudaMemsetAsync(q.counters, 0, sizeof(int) * size_t(2 + 2 * B.n), s) != cudaSuccess) return PFFT_ERR_CUDA;
-    return launch_batch_queue(q, B.dtype, units, B.q_smem, s) == 0 ? PFFT_OK : PFFT_ERR_CUDA;
+    return launch_batch_queue(q, B.dtype, units, B.q_threads, B.q_smem, s) == 0 ? PFFT_OK : PFFT_ERR_CUDA;
   }
   auto phase = [&](const std::vector<Bucket>& bs) -> pfft_status {
     auto launch = [&](const Bucket& b, cudaStream_t st) {
       GroupArgs g;
-      g.items = reinterpret_cast<const PassArgs*>(sched + b.items_off);
+      g.items = reinterpret_cast<const MixDesc*>(sched + b.items_off);
       g.cta0 = reinterpret_cast<const int*>(sched + b.cta0_off);
       g.n = b.n;
       g.base[0] = in;
       g.base[1] = B.ws;
       g.base[2] = chat;
-      return launch_grouped_pass(g, b.cols, B.dtype, b.nctas, b.threads, b.smem, st);
+      return launch_grouped_pass(g, B.dtype, b.nctas, b.threads, b.smem, st);
     };
     if (bs.empty()) return PFFT_OK;
     if (bs.size() == 1) return launch(bs[0], s) == 0 ? PFFT_OK : PFFT_ERR_CUDA;
@@ -566,9 +560,6 @@ extern "C" pfft_status pfft_batch_create(pfft_batch* out, int n, const int* d, c
     P->arena = &B->arena;
     P->generic_only = true;
     P->own_workspace = false;
-    // grouped kernels: 16 complex64 points per thread (64 registers, two
-    // 512-thread CTAs per SM) to hide the latency of the table-driven passes
-    P->ept_c64 = kGroupedEptC64;
     pfft_status st;
     try {
       st = plan_host(*P, d[i], M + mo);
@@ -581,7 +572,7 @@ extern "C" pfft_status pfft_batch_create(pfft_batch* out, int n, const int* d, c
     B->off.push_back(B->total);
     B->total += P->m;
     if (P->D == 0) B->ident.push_back(i);
-    if (!P->pen.empty()) need_ws = true;
+    if (!P->pen.empty() && !P->mixed[MIX_WHOLE]) need_ws = true;
     if (J) {
       i64 pdet = 0;
       try {

@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "fft_mixed.hpp"
 #include "fft_plan.hpp"
 #include "split_prime.cuh"
 #include "wavelet_kernels.cuh"
@@ -10,11 +11,7 @@
 namespace pfft {
 
 constexpr int kSplitThreads = 256;
-constexpr int kGroupedEptC64 = 16;  // complex64 points per thread of the grouped pass kernels
 constexpr int kSplitPerThread = 4;  // fibres per thread of a grouped split CTA
-// Dynamic shared memory of a grouped pass CTA: the 227 KB per CTA less room
-// for the static copy of its pass descriptor.
-constexpr int kGroupedMaxDynSmem = 227 * 1024 - 4096;
 
 // One grouped pass launch: items[k] is the descriptor of the k-th pattern of
 // the launch, whose tiles are CTAs cta0[k] .. cta0[k+1]-1; after the n + 1
@@ -22,7 +19,7 @@ constexpr int kGroupedMaxDynSmem = 227 * 1024 - 4096;
 // CTA.  The in / out fields of an item hold byte offsets into base[in_sel] /
 // base[out_sel].
 struct GroupArgs {
-  const PassArgs* items;
+  const MixDesc* items;
   const int* cta0;
   int n;
   const void* base[3];  // 0: the caller's input, 1: the batch workspace, 2: the caller's output
@@ -56,11 +53,11 @@ struct alignas(16) PrimeItem {
 // (|det J| > 2).
 constexpr int kQueueSplitFibres = kMaxThreads * kSplitPerThread;
 struct QueueArgs {
-  const PassArgs* rows;          // row-pass items, costliest first
+  const MixDesc* rows;           // row-pass (and whole-signal) items, costliest first
   const int* row_u0;             // first unit of each row item (prefix, n + 1 entries)
   const int* row_pat;            // pattern of each row item
   int nrow;
-  const PassArgs* cols;
+  const MixDesc* cols;
   const int* col_u0;
   const int* col_pat;
   int ncol;
@@ -86,13 +83,13 @@ struct QueueArgs {
 // Raise the shared-memory limit of the queue kernel (once per process; call
 // before any stream capture).
 int prepare_queue(int dtype);
-int launch_batch_queue(const QueueArgs& g, int dtype, int nunits, int smem, cudaStream_t s);
+// threads: the largest item's (at least kMaxThreads, which the split units use).
+int launch_batch_queue(const QueueArgs& g, int dtype, int nunits, int threads, int smem, cudaStream_t s);
 
 // Raise the dynamic shared-memory limit of the grouped kernels (once per
 // process; call before any stream capture).
 int prepare_grouped(int dtype);
-int launch_grouped_pass(const GroupArgs& g, int cols, int dtype, int nctas, int threads, int smem,
-                        cudaStream_t s);
+int launch_grouped_pass(const GroupArgs& g, int dtype, int nctas, int threads, int smem, cudaStream_t s);
 // The split levels of the patterns with |det J| = 2 (cta0 and the CTA map as
 // in GroupArgs).
 int launch_grouped_split(const SplitItem* items, const int* cta0, int n, int nctas, const void* chat, void* sc,

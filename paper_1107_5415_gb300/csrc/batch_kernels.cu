@@ -2,13 +2,13 @@
 // patterns of different size.  Each CTA reads its pattern and tile from a
 // per-CTA map stored after the launch's prefix table of first-CTA indices,
 // copies that pattern's pass descriptor into shared memory and runs the
-// generic (shared-memory Stockham) pass body of fft_kernels.cuh or the split
+// mixed-radix tile body of fft_mixed.cuh or the split
 // butterfly of wavelet_kernels.cuh on its tile.  The single-launch queue
 // kernel finds the pattern of a work unit by a search of its prefix table.
 #include <cuda_runtime.h>
 
 #include "batch.hpp"
-#include "fft_kernels.cuh"
+#include "fft_mixed.cuh"
 #include "wavelet_kernels.cuh"
 
 namespace pfft {
@@ -41,31 +41,22 @@ __device__ __forceinline__ void copy_to_smem(T* dst, const T* src) {
   for (int i = threadIdx.x; i < int(sizeof(T) / 16); i += blockDim.x) d[i] = __ldg(s + i);
 }
 
-template <typename C, int EPT, bool COLS, int MINB>
-__global__ void __launch_bounds__(kMaxThreads, MINB) grouped_pass_kernel(GroupArgs g) {
-  __shared__ PassArgs a;
+// Byte offsets of a descriptor into the launch's buffers -> addresses (one thread).
+__device__ __forceinline__ void resolve_buffers(MixDesc& a, const void* const* base) {
+  a.in = static_cast<const char*>(base[a.in_sel]) + reinterpret_cast<uintptr_t>(a.in);
+  a.out = static_cast<char*>(const_cast<void*>(base[a.out_sel])) + reinterpret_cast<uintptr_t>(a.out);
+}
+
+template <typename C>
+__global__ void __launch_bounds__(kMixThreads<C>, 1) grouped_pass_kernel(GroupArgs g) {
+  __shared__ MixDesc a;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int2 kt = cta_item(g.cta0, g.n, blockIdx.x);
   copy_to_smem(&a, g.items + kt.x);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    a.in = static_cast<const char*>(g.base[a.in_sel]) + reinterpret_cast<uintptr_t>(a.in);
-    a.out = static_cast<char*>(const_cast<void*>(g.base[a.out_sel])) + reinterpret_cast<uintptr_t>(a.out);
-  }
+  if (threadIdx.x == 0) resolve_buffers(a, g.base);
   __syncthreads();
-  const int tile = kt.y;
-  C* sm = reinterpret_cast<C*>(smem_raw);
-  if constexpr (COLS) {
-    if (a.pad)
-      col_pass_body<C, EPT, false, true, false>(a, tile, 0, sm);
-    else
-      col_pass_body<C, EPT, false, false, false>(a, tile, 0, sm);
-  } else {
-    if (a.pad)
-      row_pass_body<C, EPT, false, true, false>(a, tile, 0, sm);
-    else
-      row_pass_body<C, EPT, false, false, false>(a, tile, 0, sm);
-  }
+  mixed_body<C, false>(a, kt.y, 0, reinterpret_cast<C*>(smem_raw));
 }
 
 template <typename C>
@@ -128,22 +119,7 @@ __device__ __forceinline__ int queue_wait(const int* done, int need, const int* 
   }
 }
 
-// The units of the single-launch queue.
-template <typename C, int EPT>
-__device__ __forceinline__ void queue_row(const PassArgs& a, int tile, C* sm) {
-  if (a.pad)
-    row_pass_body<C, EPT, false, true, false>(a, tile, 0, sm);
-  else
-    row_pass_body<C, EPT, false, false, false>(a, tile, 0, sm);
-}
-// the workspace was written by other CTAs of the launch: coherent loads
-template <typename C, int EPT>
-__device__ __forceinline__ void queue_col(const PassArgs& a, int tile, C* sm) {
-  if (a.pad)
-    col_pass_body<C, EPT, false, true, false, true>(a, tile, 0, sm);
-  else
-    col_pass_body<C, EPT, false, false, false, true>(a, tile, 0, sm);
-}
+// The split units of the single-launch queue.
 template <typename C>
 __device__ __noinline__ void queue_split(const SplitItem& si, int local, const QueueArgs& g) {
   const C* cin = static_cast<const C*>(g.base[2]) + si.in_off;
@@ -163,7 +139,7 @@ template <typename C>
 __device__ __noinline__ void queue_prime(const PrimeItem& pi, int local, const QueueArgs& g) {
   const long long w = (long long)local * kMaxThreads + threadIdx.x;
   const long long mN = pi.P.mN;
-  if (w >= mN * pi.P.nch) return;
+  if (threadIdx.x >= kMaxThreads || w >= mN * pi.P.nch) return;
   const int ch = int(w / mN), gs = int(w - ch * mN);
   prime_split_item<C, 0, true>(pi.P, gs, ch * kPrimeChunk, static_cast<const C*>(g.base[2]) + pi.in_off, nullptr,
                                nullptr, nullptr, static_cast<C*>(g.sc) + pi.sc_off + gs,
@@ -172,9 +148,9 @@ __device__ __noinline__ void queue_prime(const PrimeItem& pi, int local, const Q
 
 // One unit of the launch: find its item, wait (bounded) for its dependency,
 // run it and, for a pass tile, count it done.
-template <typename C, int EPT>
+template <typename C>
 __device__ __forceinline__ void queue_unit(const QueueArgs& g, int u, C* sm) {
-  __shared__ PassArgs it_a;
+  __shared__ MixDesc it_a;
   __shared__ SplitItem it_s;
   __shared__ PrimeItem it_p;
   __shared__ int s_ok;
@@ -231,15 +207,10 @@ __device__ __forceinline__ void queue_unit(const QueueArgs& g, int u, C* sm) {
   __syncthreads();
   if (!s_ok) return;  // block-uniform
   if (u < U2) {
-    if (threadIdx.x == 0) {
-      it_a.in = static_cast<const char*>(g.base[it_a.in_sel]) + reinterpret_cast<uintptr_t>(it_a.in);
-      it_a.out = static_cast<char*>(const_cast<void*>(g.base[it_a.out_sel])) + reinterpret_cast<uintptr_t>(it_a.out);
-    }
+    if (threadIdx.x == 0) resolve_buffers(it_a, g.base);
     __syncthreads();
-    if (u < U1)
-      queue_row<C, EPT>(it_a, local, sm);
-    else
-      queue_col<C, EPT>(it_a, local, sm);
+    // the workspace was written by other CTAs of the launch: coherent loads
+    mixed_body<C, true>(it_a, local, 0, sm);
     __syncthreads();  // every output of the tile is written
     if (threadIdx.x == 0) {
       __threadfence();
@@ -257,8 +228,8 @@ __device__ __forceinline__ void queue_unit(const QueueArgs& g, int u, C* sm) {
 // that started earlier and run to completion).  One unit per CTA: a loop of
 // units around the generic pass bodies made the compiler keep their per-thread
 // values live across iterations (kilobytes of spills per thread).
-template <typename C, int EPT, int MINB>
-__global__ void __launch_bounds__(kMaxThreads, MINB) batch_queue_kernel(QueueArgs g) {
+template <typename C>
+__global__ void __launch_bounds__(kMixThreads<C>, 1) batch_queue_kernel(QueueArgs g) {
   __shared__ int s_unit;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* sm = reinterpret_cast<C*>(smem_raw);
@@ -267,7 +238,7 @@ __global__ void __launch_bounds__(kMaxThreads, MINB) batch_queue_kernel(QueueArg
   const int u = s_unit;
   if (u >= g.u_rows + g.u_cols + g.u_splits + g.u_primes) return;
   if (*reinterpret_cast<volatile int*>(g.counters + 1)) return;  // aborted after a timed-out wait
-  queue_unit<C, EPT>(g, u, reinterpret_cast<C*>(sm));
+  queue_unit<C>(g, u, reinterpret_cast<C*>(sm));
 }
 
 namespace {
@@ -275,7 +246,7 @@ template <typename K>
 int allow_smem(K* k) {
   // the static descriptor copy shares the 227 KB with the dynamic tile
   return cudaFuncSetAttribute(reinterpret_cast<const void*>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kGroupedMaxDynSmem) == cudaSuccess
+                              kMixGroupedSmem) == cudaSuccess
              ? 0
              : -1;
 }
@@ -283,30 +254,20 @@ int allow_smem(K* k) {
 
 int prepare_grouped(int dtype) {
   if (dtype == 0) {
-    static const int ok = allow_smem(grouped_pass_kernel<float2, kGroupedEptC64, false, 2>) |
-                          allow_smem(grouped_pass_kernel<float2, kGroupedEptC64, true, 2>);
+    static const int ok = allow_smem(grouped_pass_kernel<float2>);
     return ok;
   }
-  static const int ok = allow_smem(grouped_pass_kernel<double2, 16, false, 1>) |
-                        allow_smem(grouped_pass_kernel<double2, 16, true, 1>);
+  static const int ok = allow_smem(grouped_pass_kernel<double2>);
   return ok;
 }
 
-int launch_grouped_pass(const GroupArgs& g, int cols, int dtype, int nctas, int threads, int smem,
-                        cudaStream_t s) {
+int launch_grouped_pass(const GroupArgs& g, int dtype, int nctas, int threads, int smem, cudaStream_t s) {
   if (nctas <= 0) return 0;
-  if (smem > kGroupedMaxDynSmem || threads > kMaxThreads) return -1;
-  if (dtype == 0) {
-    if (cols)
-      grouped_pass_kernel<float2, kGroupedEptC64, true, 2><<<nctas, threads, smem, s>>>(g);
-    else
-      grouped_pass_kernel<float2, kGroupedEptC64, false, 2><<<nctas, threads, smem, s>>>(g);
-  } else {
-    if (cols)
-      grouped_pass_kernel<double2, 16, true, 1><<<nctas, threads, smem, s>>>(g);
-    else
-      grouped_pass_kernel<double2, 16, false, 1><<<nctas, threads, smem, s>>>(g);
-  }
+  if (smem > kMixGroupedSmem || threads > (dtype == 0 ? kMixThreadsC64 : kMixThreadsC128)) return -1;
+  if (dtype == 0)
+    grouped_pass_kernel<float2><<<nctas, threads, smem, s>>>(g);
+  else
+    grouped_pass_kernel<double2><<<nctas, threads, smem, s>>>(g);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -341,20 +302,21 @@ int launch_grouped_prime_split(const PrimeItem* items, const int* cta0, int n, i
 namespace pfft {
 int prepare_queue(int dtype) {
   if (dtype == 0) {
-    static const int ok = allow_smem(batch_queue_kernel<float2, kGroupedEptC64, 2>);
+    static const int ok = allow_smem(batch_queue_kernel<float2>);
     return ok;
   }
-  static const int ok = allow_smem(batch_queue_kernel<double2, 16, 1>);
+  static const int ok = allow_smem(batch_queue_kernel<double2>);
   return ok;
 }
 
-int launch_batch_queue(const QueueArgs& g, int dtype, int nunits, int smem, cudaStream_t s) {
+int launch_batch_queue(const QueueArgs& g, int dtype, int nunits, int threads, int smem, cudaStream_t s) {
   if (nunits <= 0) return 0;
-  if (smem > kGroupedMaxDynSmem) return -1;
+  if (smem > kMixGroupedSmem || threads < kMaxThreads || threads > (dtype == 0 ? kMixThreadsC64 : kMixThreadsC128))
+    return -1;
   if (dtype == 0)
-    batch_queue_kernel<float2, kGroupedEptC64, 2><<<nunits, kMaxThreads, smem, s>>>(g);
+    batch_queue_kernel<float2><<<nunits, threads, smem, s>>>(g);
   else
-    batch_queue_kernel<double2, 16, 1><<<nunits, kMaxThreads, smem, s>>>(g);
+    batch_queue_kernel<double2><<<nunits, threads, smem, s>>>(g);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 }  // namespace pfft

@@ -41,6 +41,25 @@ template <typename C>
 __device__ __forceinline__ C cadd(C a, C b) { return cmake<C>(a.x + b.x, a.y + b.y); }
 template <typename C>
 __device__ __forceinline__ C csub(C a, C b) { return cmake<C>(a.x - b.x, a.y - b.y); }
+// Sums of the butterflies.  PK: one packed instruction per complex64 sum (the
+// same two IEEE sums), for the kernels bound by instruction issue (M = [[512,
+// 128], [0, 512]] x 16 there and back: 0.1024 -> 0.0977 ms); the pipelined passes,
+// bound by their memory phases, keep the plain ones, which the compiler may
+// contract with a preceding product (2.185 against 2.197 ms for the 2^24 x 8 step).
+template <bool PK, typename C>
+__device__ __forceinline__ C bsum(C a, C b) {
+  if constexpr (PK && sizeof(C) == 8)
+    return __fadd2_rn(a, b);
+  else
+    return cadd(a, b);
+}
+template <bool PK, typename C>
+__device__ __forceinline__ C bdiff(C a, C b) {
+  if constexpr (PK && sizeof(C) == 8)
+    return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+  else
+    return csub(a, b);
+}
 template <typename C>
 __device__ __forceinline__ C cmul(C a, C b) {
   return cmake<C>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -179,20 +198,20 @@ __device__ __forceinline__ void load_point(const int* __restrict__ tab, int idx,
 
 // ------------------------------------------------------------- butterflies
 // In-register forward DFTs, X[k] = sum_n x[n] exp(-2 pi i n k / R).
-template <typename C>
+template <typename C, bool PK = true>
 __device__ __forceinline__ void dft2(C& a, C& b) {
   C t = a;
-  a = cadd(t, b);
-  b = csub(t, b);
+  a = bsum<PK>(t, b);
+  b = bdiff<PK>(t, b);
 }
 
-template <typename C>
+template <typename C, bool PK = true>
 __device__ __forceinline__ void dft4(C& x0, C& x1, C& x2, C& x3) {
-  C a = cadd(x0, x2), b = csub(x0, x2), c = cadd(x1, x3), d = cmul_mi(csub(x1, x3));
-  x0 = cadd(a, c);
-  x2 = csub(a, c);
-  x1 = cadd(b, d);
-  x3 = csub(b, d);
+  C a = bsum<PK>(x0, x2), b = bdiff<PK>(x0, x2), c = bsum<PK>(x1, x3), d = cmul_mi(bdiff<PK>(x1, x3));
+  x0 = bsum<PK>(a, c);
+  x2 = bdiff<PK>(a, c);
+  x1 = bsum<PK>(b, d);
+  x3 = bdiff<PK>(b, d);
 }
 
 // exp(-2 pi i q / 16) for q = 0..15 (exact constants of cos/sin(pi/8 multiples)).
@@ -222,29 +241,29 @@ __device__ __forceinline__ C w16(int q) {
 }
 
 // Length 8 as 4 x 2: n = 2 n1 + n2, k = k1 + 4 k2.
-template <typename C>
+template <typename C, bool PK = true>
 __device__ __forceinline__ void dft8(C* x) {
   C e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6];
   C o0 = x[1], o1 = x[3], o2 = x[5], o3 = x[7];
-  dft4(e0, e1, e2, e3);
-  dft4(o0, o1, o2, o3);
+  dft4<C, PK>(e0, e1, e2, e3);
+  dft4<C, PK>(o0, o1, o2, o3);
   o1 = cmul(o1, w16<C>(2));
   o2 = cmul_mi(o2);
   o3 = cmul(o3, w16<C>(6));
-  x[0] = cadd(e0, o0); x[4] = csub(e0, o0);
-  x[1] = cadd(e1, o1); x[5] = csub(e1, o1);
-  x[2] = cadd(e2, o2); x[6] = csub(e2, o2);
-  x[3] = cadd(e3, o3); x[7] = csub(e3, o3);
+  x[0] = bsum<PK>(e0, o0); x[4] = bdiff<PK>(e0, o0);
+  x[1] = bsum<PK>(e1, o1); x[5] = bdiff<PK>(e1, o1);
+  x[2] = bsum<PK>(e2, o2); x[6] = bdiff<PK>(e2, o2);
+  x[3] = bsum<PK>(e3, o3); x[7] = bdiff<PK>(e3, o3);
 }
 
 // Length 16 as 4 x 4: n = 4 n1 + n2, k = k1 + 4 k2.
-template <typename C>
+template <typename C, bool PK = true>
 __device__ __forceinline__ void dft16(C* x) {
   C y[16];
 #pragma unroll
   for (int n2 = 0; n2 < 4; ++n2) {
     C a = x[n2], b = x[4 + n2], c = x[8 + n2], d = x[12 + n2];
-    dft4(a, b, c, d);  // over n1 -> k1
+    dft4<C, PK>(a, b, c, d);  // over n1 -> k1
     y[n2 * 4 + 0] = a;
     y[n2 * 4 + 1] = (n2 == 0) ? b : cmul(b, w16<C>(n2));
     y[n2 * 4 + 2] = (n2 == 0) ? c : cmul(c, w16<C>(2 * n2));
@@ -253,7 +272,7 @@ __device__ __forceinline__ void dft16(C* x) {
 #pragma unroll
   for (int k1 = 0; k1 < 4; ++k1) {
     C a = y[k1], b = y[4 + k1], c = y[8 + k1], d = y[12 + k1];
-    dft4(a, b, c, d);  // over n2 -> k2
+    dft4<C, PK>(a, b, c, d);  // over n2 -> k2
     x[k1] = a;
     x[k1 + 4] = b;
     x[k1 + 8] = c;

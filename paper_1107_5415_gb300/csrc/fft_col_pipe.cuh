@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(256, 2) col_pipe_kernel(PassArgs a) {
     // stage 0 (Ns = 1), exchange in two rounds through X: round h moves
     // register half H = h xor bit 4 of p (positions 32 p + r written,
     // p + 32 r' read, split by bit 9 xor bit 4 of the position; bit 9 dropped)
-    dft_pow2<C, R>(v);
+    dft_pow2<C, R, false>(v);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (h) __syncthreads();  // round 0's reads of X are done
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256, 2) col_pipe_kernel(PassArgs a) {
     }
     // stage 1 (Ns = 32): v[r] = frequency p + 32 r
     if (p) main_twiddle<C, R>(v, stw + a.stw_off[1] + p * 5);
-    dft_pow2<C, R>(v);
+    dft_pow2<C, R, false>(v);
 
     if constexpr (FWD) {
       // sheared store in two rounds of 16 walk steps through X

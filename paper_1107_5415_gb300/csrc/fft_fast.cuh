@@ -26,7 +26,7 @@ namespace pfft {
 __device__ __forceinline__ int fphys(int x) { return x + (x >> 5); }
 
 // Length 32 as 16 x 2: n = 2 n1 + n2, k = k1 + 16 k2.
-template <typename C>
+template <typename C, bool PK = true>
 __device__ __forceinline__ void dft32(C* x) {
   C e[16], o[16];
 #pragma unroll
@@ -34,8 +34,8 @@ __device__ __forceinline__ void dft32(C* x) {
     e[i] = x[2 * i];
     o[i] = x[2 * i + 1];
   }
-  dft16(e);
-  dft16(o);
+  dft16<C, PK>(e);
+  dft16<C, PK>(o);
   using Rl = decltype(C::x);
   // cos and sin of 2 pi k / 32, k = 0..15
   const Rl cs[16] = {Rl(1.0), Rl(0.98078528040323044913), Rl(0.92387953251128675613),
@@ -54,23 +54,23 @@ __device__ __forceinline__ void dft32(C* x) {
   for (int k = 0; k < 16; ++k) {
     C t = o[k];
     if (k) t = cmul(t, cmake<C>(cs[k], -sn[k]));
-    x[k] = cadd(e[k], t);
-    x[k + 16] = csub(e[k], t);
+    x[k] = bsum<PK>(e[k], t);
+    x[k + 16] = bdiff<PK>(e[k], t);
   }
 }
 
-template <typename C, int R>
+template <typename C, int R, bool PK = true>
 __device__ __forceinline__ void dft_pow2(C* x) {
   if constexpr (R == 2) {
-    dft2(x[0], x[1]);
+    dft2<C, PK>(x[0], x[1]);
   } else if constexpr (R == 4) {
-    dft4(x[0], x[1], x[2], x[3]);
+    dft4<C, PK>(x[0], x[1], x[2], x[3]);
   } else if constexpr (R == 8) {
-    dft8(x);
+    dft8<C, PK>(x);
   } else if constexpr (R == 16) {
-    dft16(x);
+    dft16<C, PK>(x);
   } else {
-    dft32(x);
+    dft32<C, PK>(x);
   }
 }
 

@@ -1,8 +1,9 @@
-// Transform kernel templates for sm_103a: the row pass and the column pass of the
-// Kronecker factorisation in Smith coordinates (Theorem 1, eq. (KroneckerFFT)),
-// each a batched Stockham autosort DFT held in shared memory, with the
-// bit-exact gather / scatter between the Hermite boxes and the Smith
-// coordinates fused into the global loads and stores.
+// Row and column pass of split-precision plans (PFFT_FLAG_TC_SPLIT) whose lengths
+// the register-resident kernels do not take: batched Stockham autosort DFTs held
+// in shared memory, radix-32 and radix-16 stages on the tensor cores, the
+// gather / scatter between the Hermite boxes and the Smith coordinates fused
+// into the global loads and stores.  Every other pass of such lengths runs in
+// fft_mixed.cuh.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -498,7 +499,7 @@ __device__ __forceinline__ int shear_index(const PassArgs& a, int j, const int* 
 // Column pass: all LB rows of T adjacent workspace columns per CTA, smem
 // layout [i][t].  The DFT runs over the (D-1) cycles inside the pencil.
 // Loads and stores are batched per thread as in the row pass.
-template <typename C, int EPT, bool POW2, bool PAD, bool TCK = true, bool COH = false>
+template <typename C, int EPT, bool POW2, bool PAD, bool TCK = true>
 __device__ __forceinline__ void col_pass_body(const PassArgs& a, int tile, int sig, C* sm) {
   const C* __restrict__ tw = static_cast<const C*>(a.tw);
   const C* __restrict__ in = static_cast<const C*>(a.in) + (int64_t)sig * a.m;
@@ -532,7 +533,7 @@ __device__ __forceinline__ void col_pass_body(const PassArgs& a, int tile, int s
     if (w < n_ok) {
       const int j = a.divT.div(w);
       if (ws_in) {
-        v[k] = COH ? __ldcg(in + j * a.nD + p0 + tcol) : __ldg(in + j * a.nD + p0 + tcol);
+        v[k] = __ldg(in + j * a.nD + p0 + tcol);
         sidx[k] = j * a.T + tcol;
       } else {
         const int i = shear_index(a, j, off);

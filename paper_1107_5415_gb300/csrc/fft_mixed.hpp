@@ -1,0 +1,114 @@
+// Descriptors of the mixed-radix passes (fft_mixed.cuh): any cycle lengths, any
+// element type, one pattern per launch, grouped launches and the single-launch
+// queue alike.
+//
+// Three kinds of tile, all transformed in shared memory by the same stages:
+//
+//   row    T rows of the logical LB x nD array (the DFT over the last cycle);
+//          with a split last cycle the rows of a tile are adjacent lambda_a,
+//          which are adjacent input slots, so the tile is held [element][row]
+//          and the lanes of its box loads and stores run along the rows;
+//   column T adjacent workspace columns (the DFTs over the other cycles), held
+//          [row][column];
+//   whole  T complete signals of m points each (every cycle in one tile): the
+//          box side is read and written in slot order through a table of tile
+//          positions, so such a transform is one launch without a workspace.
+#pragma once
+#include <stdint.h>
+
+#include "fft_plan.hpp"
+
+namespace pfft {
+
+enum MixKind { MIX_ROW = 0, MIX_COL = 1, MIX_WHOLE = 2 };
+
+constexpr int kMixMaxStages = 16;
+constexpr int kMixPoints = 16;  // points a thread holds between the barriers of a stage, at most
+// Register butterflies reach radix 16; primes from 17 up are direct stages.
+constexpr int kMixMinDirect = 17;
+// Outputs pairs of one work item of a direct stage: kMixWide when every item
+// has a thread of its own, else kMixNarrow with at most kMixItems per thread.
+constexpr int kMixWide = 8, kMixNarrow = 4, kMixItems = 3;
+// Order in which the stages of the register radices run (mix_stages).
+constexpr int kMixOrder[15] = {15, 13, 11, 9, 16, 14, 12, 10, 8, 7, 6, 5, 4, 3, 2};
+template <typename C>
+constexpr int kMixThreads = sizeof(C) == 8 ? 1024 : 512;
+// Dynamic shared memory of a grouped tile: the 227 KB per CTA less room for the
+// static copy of its descriptor.
+constexpr int kMixGroupedSmem = 227 * 1024 - 4096;
+constexpr int kMixThreadsC64 = 1024, kMixThreadsC128 = 512;
+
+// One radix stage along one axis.  Tile positions of a butterfly (low, j, hi):
+// base + (j + r aR) sig -> base + ((j - k) R + k + r Ns) sig, k = j mod Ns,
+// base = hi blk + low, low < sig, j < aR, blk = aR R sig; sig is the axis's
+// stride in the tile (the columns of a tile are strides below every axis).
+// Tiles are padded from the first stage along the fastest axis on: when its
+// radix R1 is even, its outputs j R1 + r would meet in few banks, so `pad`
+// elements (one pencil position) follow every R1 of them from there.  R1 divides
+// every later step, so all accesses of a stage stay affine in r: istep and ostep
+// are the padded steps, ipad / opad the padding per pad unit (0: not padded).
+struct MixStage {
+  int R, aR, sig, Ns, blk;
+  int istep, ostep, ipad, opad;
+  int tw;       // twiddles of the stage in the stage table: [bit][k], w^(2^bit), w = exp(-2 pi i k / (Ns R))
+  int gen;      // direct stages: offset of g^t mod R (R - 1 ints) in the integer table
+  int twstep;   // direct stages: step of the root table per unit of exp(-2 pi i / (Ns R))
+  FastDiv div_sig, div_aR, div_Ns, div_nb;  // div_nb: direct stages, butterflies of the tile
+};
+
+struct alignas(16) MixDesc {
+  int kind, lay;  // lay 1: the tile is [element][row] (row tiles of a split last cycle)
+  int d, ts;
+  int L, T, logT, n;  // pencil length, pencils per tile, points of the tile
+  int nD, LB, m, batch;
+  int groups;         // tiles per signal (whole tiles: of the batch)
+  int nthreads, smem_bytes;
+  int pad;            // padding of the finished tile: position x at x + pad (x / pad unit)
+  FastDiv div_pad;    // by the pad unit (R1 positions of the fastest axis)
+  int pitch;          // row tiles in [row][element] order: distance of the finished rows
+  const int* psout;   // row tiles: padded element position of each column position (unpadded: PIinv)
+  int dir_off;        // tables of the direct stages after the tile (elements)
+  int nstages;
+  int tw_n;           // order of the root table
+  int load_mode, store_mode, conj_in, conj_out;
+  int in_sel, out_sel;  // grouped launches: in / out are byte offsets into base[in_sel] / base[out_sel]
+  double scale;
+  const void* in;
+  void* out;
+  const int *Atab, *Btab, *Ctab, *Etab, *PIinv;
+  const int *map_in, *map_out;  // whole tiles: tile position of box slot s (input box, output box)
+  const void* tw;               // roots exp(-2 pi i t / tw_n)
+  const void* stw;              // stage table
+  const int* gtab;              // integer table of the direct stages
+  const void *fs_lo, *fs_hi;    // phases of a split last cycle (fft_plan.hpp)
+  int fs_na;
+  FastDiv fs_div;
+  FastDiv divT, divnD, divL;
+  int nsub, sub_n[kMaxSub], alpha[kMaxSub];
+  FastDiv sub_div[kMaxSub];
+  BoxDesc boxH, boxG;
+  MixStage st[kMixMaxStages];
+};
+static_assert(sizeof(MixDesc) % 16 == 0, "descriptors are copied in 16-byte pieces");
+
+// What a launch sets on top of a plan's descriptor.
+struct MixCall {
+  int load_mode, store_mode, conj_in, conj_out;
+  double scale;
+  const void* in;
+  void* out;
+};
+
+// Stage twiddles: entry (s, b, k) = exp(-2 pi i (k 2^b mod Ns R) / (Ns R)).
+struct MixTableArgs {
+  int n, total;
+  int R[kMixMaxStages], Ns[kMixMaxStages], off[kMixMaxStages + 1];
+};
+
+// Host-side launchers (fft_mixed_c64.cu, fft_mixed_c128.cu, fft_support.cu).
+int launch_mixed_c64(const MixDesc& a, cudaStream_t s);
+int launch_mixed_c128(const MixDesc& a, cudaStream_t s);
+int launch_mixed_tables(void* tab, const MixTableArgs& t, int dtype, cudaStream_t s);
+int launch_whole_maps(const MixDesc& a, const int* PI, int* map_in, int* map_out, cudaStream_t s);
+
+}  // namespace pfft

@@ -7,10 +7,12 @@
 #include <cmath>
 #include <cstring>
 #include <new>
+#include <map>
 #include <string>
 #include <vector>
 
 #include "../../include/pfft.h"
+#include "fft_mixed.hpp"
 #include "fft_plan.hpp"
 #include "fft_tc.cuh"
 #include "lattice.hpp"
@@ -23,11 +25,9 @@ namespace {
 
 // Radices for a cycle length: primes from 11 up first (direct stages, up to
 // kMaxDirectRadix), then 16s, the rest of the power of two and 3, 5, 7 -- the
-// execution order of the stage regions.  Returns false if a prime factor is
-// not supported.
-// max2: the largest power-of-two radix (16, or 8 for the schedules the batch
-// autotuner may pick instead).
-bool factor_radices(int n, std::vector<int>& out, bool tc = false, int max2 = 16) {
+// execution order of the stage regions (split-precision plans).  Returns false
+// if a prime factor is not supported.
+bool factor_radices(int n, std::vector<int>& out, bool tc = false) {
   out.clear();
   for (int p = kMinDirectRadix; p <= kMaxDirectRadix && p <= n; p += 2) {
     bool prime = true;
@@ -51,7 +51,7 @@ bool factor_radices(int n, std::vector<int>& out, bool tc = false, int max2 = 16
     out.push_back(32);
     p2 -= 5;
   }
-  while (max2 >= 16 && p2 >= 4) {
+  while (p2 >= 4) {
     out.push_back(16);
     p2 -= 4;
   }
@@ -116,9 +116,9 @@ int primitive_root(int p) {
   return 0;
 }
 
-bool axis_stages(std::vector<StageDesc>& out, int a, int sigma, int nD, bool tc, int max2) {
+bool axis_stages(std::vector<StageDesc>& out, int a, int sigma, int nD, bool tc) {
   std::vector<int> rad;
-  if (!factor_radices(a, rad, tc, max2)) return false;
+  if (!factor_radices(a, rad, tc)) return false;
   int Ns = 1;
   for (int R : rad) {
     StageDesc s;
@@ -197,9 +197,9 @@ int threads_for(const PassArgs& p, int ept) {
 
 size_t elem_bytes(int dtype) { return dtype == PFFT_C64 ? 8 : 16; }
 
-// Whether one pencil of length L fits a CTA of the shared-memory kernels:
-// at most `row_max` elements and kMaxThreads threads for its stages.
-bool tile_fits(int L, int row_max, int ept) {
+// Whether one pencil of length L fits a CTA of the split-precision plans'
+// shared-memory kernels: at most `row_max` elements and kMaxThreads threads.
+bool tc_tile_fits(int L, int row_max) {
   if (L > row_max) return false;
   std::vector<int> rad;
   if (!factor_radices(L, rad)) return false;
@@ -210,7 +210,278 @@ bool tile_fits(int L, int row_max, int ept) {
   p.nstages = int(rad.size());
   if (p.nstages > kMaxStages) return false;
   for (int i = 0; i < p.nstages; ++i) p.st[i].R = rad[i];
-  return threads_for(p, ept) <= kMaxThreads;
+  return threads_for(p, 32) <= kMaxThreads;
+}
+
+// ------------------------------------------------ mixed-radix passes (fft_mixed.cuh)
+int mix_max_threads(int dtype) { return dtype == PFFT_C64 ? kMixThreadsC64 : kMixThreadsC128; }
+int mix_points(int R) { return R * std::max(1, kMixPoints / R); }  // points a thread takes in a radix-R stage
+
+// Instructions a point costs in one stage: 8 for the shared-memory round trip,
+// about 40 per butterfly for its indices, the butterfly and the twiddles
+// (operation counts of fft_mixed.cuh); a direct stage about 1.2 per unit of R
+// on top of its pre-pass.
+double radix_cost(int R) {
+  static const double flops[17] = {0, 0, 4, 6.7, 8, 11.2, 11, 14.4, 13, 15.6, 15.2, 19.6, 14.3, 21.7, 17.7, 17.6, 16.8};
+  return R >= kMixMinDirect ? 40 + 1.2 * R : 8 + 40.0 / R + flops[R];
+}
+
+// Cheapest radices covering n (factors 2, 3, 5, 7, 11, 13 through the register
+// butterflies, larger primes as direct stages, smallest first and before all
+// others), every one taking at least min_points points per thread.  cost: the
+// sum of radix_cost.  False when n has no such cover.
+struct RadixCover {
+  double cost;
+  int R;  // first radix (0: none)
+};
+RadixCover cover_smooth(int n, int min_points, int max2, std::map<int, RadixCover>& memo) {
+  if (n == 1) return {0, 1};
+  auto it = memo.find(n);
+  if (it != memo.end()) return it->second;
+  RadixCover best{1e30, 0};
+  for (int R = 16; R >= 2; --R) {
+    if (n % R || mix_points(R) < min_points || (R == 16 && max2 < 16)) continue;
+    const RadixCover rest = cover_smooth(n / R, min_points, max2, memo);
+    if (rest.R && rest.cost + radix_cost(R) < best.cost) best = {rest.cost + radix_cost(R), R};
+  }
+  memo[n] = best;
+  return best;
+}
+bool mixed_radices(int n, int min_points, int max2, std::vector<int>& out, double* cost = nullptr) {
+  out.clear();
+  double c = 0;
+  for (int p = kMixMinDirect; p <= kMaxDirectRadix && p <= n; p += 2) {
+    bool prime = p % 3 && p % 5 && p % 7 && p % 11 && p % 13;
+    for (int q = 17; prime && q * q <= p; q += 2) prime = p % q != 0;
+    if (!prime) continue;
+    for (; n % p == 0; n /= p) {
+      out.push_back(p);
+      c += radix_cost(p);
+    }
+  }
+  std::map<int, RadixCover> memo;
+  for (int x = n; x > 1;) {
+    const RadixCover r = cover_smooth(x, min_points, max2, memo);
+    if (!r.R) return false;
+    out.push_back(r.R);
+    c += radix_cost(r.R);
+    x /= r.R;
+  }
+  if (cost) *cost = c;
+  return true;
+}
+
+// Points per thread that every stage of a pencil of L points must reach.
+int mix_min_points(int L, int dtype) { return (L + mix_max_threads(dtype) - 1) / mix_max_threads(dtype); }
+
+// Threads of a mixed-radix tile of n points.
+int mix_threads(const std::vector<int>& radices, int n, int max_threads) {
+  int need = (n + kMixPoints - 1) / kMixPoints;
+  for (int R : radices) {
+    const int nbf = n / R;
+    if (R >= kMixMinDirect) {  // pre-pass pairs, then wide items or up to kMixItems narrow ones (mix_direct)
+      const int h = (R - 1) / 2;
+      const int wide = nbf * ((h + kMixWide - 1) / kMixWide), narrow = nbf * ((h + kMixNarrow - 1) / kMixNarrow);
+      need = std::max(need, (nbf * h + kMixPoints / 2 - 1) / (kMixPoints / 2));
+      need = std::max(need, wide <= max_threads ? wide : (narrow + kMixItems - 1) / kMixItems);
+    } else {
+      const int nb = std::max(1, kMixPoints / R);
+      need = std::max(need, (nbf + nb - 1) / nb);
+    }
+  }
+  return (need + 31) / 32 * 32;
+}
+
+// Whether a pencil of L points (one axis, or the axes of a column) fits a tile.
+bool mix_fits(const std::vector<int>& axes, int L, int dtype, double* cost = nullptr) {
+  if (L > (dtype == PFFT_C64 ? 16384 : 8192)) return false;
+  std::vector<int> all, rad;
+  double c = 0, ca = 0;
+  for (int a : axes) {
+    if (!mixed_radices(a, mix_min_points(L, dtype), 16, rad, &ca)) return false;
+    all.insert(all.end(), rad.begin(), rad.end());
+    c += ca;
+  }
+  if (cost) *cost = c;
+  return int(all.size()) <= kMixMaxStages && mix_threads(all, L, mix_max_threads(dtype)) <= mix_max_threads(dtype);
+}
+
+// The stages of a kind of tile (everything that does not depend on T) and
+// their tables.
+pfft_status mix_stages(pfft_plan_s& P, int kind) {
+  MixStages& S = P.stages[P.max2 == 16 ? 0 : 1][kind];
+  if (S.ready) return PFFT_OK;
+  const int L = kind == MIX_ROW ? P.nD : kind == MIX_COL ? P.LB : int(P.m);
+  const int tw_n = kind == MIX_COL && P.tw_col ? P.col_n : P.nD;
+  struct Axis {
+    int a, sigma, Ns;
+  };
+  std::vector<Axis> axes;
+  int sigma = 1;
+  if (kind != MIX_COL) {
+    axes.push_back({P.nD, 1, 1});
+    sigma = P.nD;
+  }
+  if (kind != MIX_ROW)
+    for (int s = int(P.pen.size()) - 1; s >= 0; --s) {
+      axes.push_back({P.pen[s], sigma, 1});
+      sigma *= P.pen[s];
+    }
+  std::vector<std::pair<int, int>> order;  // (radix, axis)
+  std::vector<int> rad;
+  for (size_t i = 0; i < axes.size(); ++i) {
+    if (!mixed_radices(axes[i].a, mix_min_points(L, P.dtype), P.max2, rad)) return PFFT_ERR_UNSUPPORTED;
+    for (int R : rad) order.push_back({R, int(i)});
+  }
+  if (order.size() > size_t(kMixMaxStages)) return PFFT_ERR_UNSUPPORTED;
+  std::stable_sort(order.begin(), order.end(), [](const std::pair<int, int>& x, const std::pair<int, int>& y) {
+    const bool dx = x.first >= kMixMinDirect, dy = y.first >= kMixMinDirect;
+    if (dx || dy) return dx != dy ? dx : x.first < y.first;
+    auto rank = [](int R) { return std::find(kMixOrder, kMixOrder + 15, R) - kMixOrder; };
+    return rank(x.first) < rank(y.first);
+  });
+  MixTableArgs t;
+  std::memset(&t, 0, sizeof(t));
+  std::vector<int> g;
+  for (auto& o : order) {
+    Axis& ax = axes[o.second];
+    MixStage s;
+    std::memset(&s, 0, sizeof(s));
+    s.R = o.first;
+    s.aR = ax.a / s.R;
+    s.sig = ax.sigma;
+    s.Ns = ax.Ns;
+    s.twstep = tw_n / (s.Ns * s.R);
+    s.div_aR.init(uint32_t(s.aR));
+    s.div_Ns.init(uint32_t(s.Ns));
+    if (s.R >= kMixMinDirect) {
+      s.gen = int(g.size());
+      const int r = primitive_root(s.R);
+      for (int e = 0, x = 1; e < s.R - 1; ++e, x = x * r % s.R) g.push_back(x);
+    } else if (s.Ns > 1) {
+      s.tw = t.total;
+      t.R[t.n] = s.R;
+      t.Ns[t.n] = s.Ns;
+      t.off[t.n++] = t.total;
+      t.total += s.Ns * (s.R > 8 ? 4 : s.R > 4 ? 3 : s.R > 2 ? 2 : 1);
+      t.off[t.n] = t.total;
+    }
+    ax.Ns *= s.R;
+    S.st.push_back(s);
+  }
+  if (t.total) {
+    if (int e = P.alloc(&S.stw, size_t(t.total) * elem_bytes(P.dtype))) return pfft_status(e);
+    if (launch_mixed_tables(S.stw, t, P.dtype, 0) != 0) return PFFT_ERR_CUDA;
+  }
+  if (!g.empty()) {
+    if (int e = P.alloc((void**)&S.gtab, g.size() * sizeof(int))) return pfft_status(e);
+    if (cudaMemcpy(S.gtab, g.data(), g.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
+      return PFFT_ERR_CUDA;
+  }
+  if (kind == MIX_ROW) {  // element positions x -> x + x / R1 when the first register stage pads
+    int R1 = 0;
+    for (auto& s : S.st)
+      if (s.Ns == 1 && s.R % 2 == 0) R1 = s.R;
+    if (R1) {
+      std::vector<int> ps(P.PIinv);
+      for (int& x : ps) x += x / R1;
+      if (int e = P.alloc((void**)&S.psout, ps.size() * sizeof(int))) return pfft_status(e);
+      if (cudaMemcpy(S.psout, ps.data(), ps.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
+        return PFFT_ERR_CUDA;
+    }
+  }
+  S.ready = true;
+  return PFFT_OK;
+}
+
+// The descriptor of a kind of tile with T pencils (T a power of two; any T for
+// row tiles in [row][element] order and whole tiles).
+pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
+  MixDesc& a = P.mix[kind];  // its plan-wide fields are set (plan_device)
+  const MixStages& S = P.stages[P.max2 == 16 ? 0 : 1][kind];
+  const int max_threads = mix_max_threads(P.dtype);
+  a.kind = kind;
+  a.lay = kind == MIX_ROW && P.fs_na > 1 ? 1 : 0;
+  a.L = kind == MIX_ROW ? P.nD : kind == MIX_COL ? P.LB : int(P.m);
+  a.T = T;
+  a.logT = 0;
+  while ((1 << a.logT) < T) ++a.logT;
+  a.n = T * a.L;
+  const int count = kind == MIX_ROW ? P.LB : kind == MIX_COL ? P.nD : int(P.batch);
+  a.groups = (count + T - 1) / T;
+  a.divT.init(uint32_t(T));
+  a.divnD.init(uint32_t(P.nD));
+  a.divL.init(uint32_t(a.L));
+  a.stw = S.stw;
+  a.gtab = S.gtab;
+  a.tw = kind == MIX_COL && P.tw_col ? P.tw_col : P.tw;
+  a.tw_n = kind == MIX_COL && P.tw_col ? P.col_n : P.nD;
+  const int tstride = kind == MIX_COL || a.lay ? T : 1;  // stride of the pencil index in the tile
+  a.nstages = int(S.st.size());
+  std::vector<int> rad;
+  int rmax = 0;
+  int unit = 0;  // pad unit, once padded
+  for (int i = 0; i < a.nstages; ++i) {
+    MixStage s = S.st[i];
+    const bool first = s.sig == 1 && s.Ns == 1 && s.R % 2 == 0 && tstride < 16;
+    s.sig *= tstride;
+    s.blk = s.aR * s.R * s.sig;
+    s.istep = s.aR * s.sig;
+    s.ostep = s.Ns * s.sig;
+    if (unit) {
+      s.ipad = tstride;
+      s.istep += s.istep / unit * tstride;
+    }
+    if (first) unit = s.R * tstride;
+    if (unit) {
+      s.opad = tstride;
+      if (!first) s.ostep += s.ostep / unit * tstride;
+    }
+    s.div_sig.init(uint32_t(s.sig));
+    s.div_nb.init(uint32_t(std::max(1, a.n / s.R)));
+    a.st[i] = s;
+    rad.push_back(s.R);
+    if (s.R >= kMixMinDirect) rmax = std::max(rmax, s.R);
+  }
+  a.nthreads = mix_threads(rad, a.n, max_threads);
+  if (tstride > 1 && a.nthreads % T) a.nthreads = (a.nthreads + T - 1) / T * T;  // each thread keeps one column
+  if (a.nthreads > max_threads) return PFFT_ERR_UNSUPPORTED;
+  a.pad = unit ? tstride : 0;
+  a.pitch = a.L;
+  a.psout = a.PIinv;
+  if (kind == MIX_ROW && unit) {
+    a.pitch = a.L + a.L / (unit / tstride);
+    a.psout = S.psout;
+  }
+  a.div_pad.init(uint32_t(unit ? unit : 1 << 30));
+  a.dir_off = a.n + (unit ? a.n / unit * tstride : 0);
+  // roots (R - 1 + kMixWide) and powers (R - 1 ints) of a direct stage
+  const int extra = rmax ? rmax + kMixWide + (rmax + 1) / 2 : 0;
+  a.smem_bytes = int(size_t(a.dir_off + extra) * elem_bytes(P.dtype));
+  return a.smem_bytes <= (P.generic_only ? kMixGroupedSmem : 227 * 1024) ? PFFT_OK : PFFT_ERR_UNSUPPORTED;
+}
+
+// Pencils per tile: as many as `budget` points hold (at most `cap`), up to
+// `lanes` of them (the adjacent pencils that fill a 32-byte sector) even when
+// that takes `most` points; but no more than leave `ctas` tiles for the launch
+// once those lanes are there.
+pfft_status mix_choose(pfft_plan_s& P, int kind, int cap, int budget, int most, int lanes, int ctas) {
+  pfft_status st = mix_stages(P, kind);
+  if (st != PFFT_OK) return st;
+  const int L = kind == MIX_ROW ? P.nD : kind == MIX_COL ? P.LB : int(P.m);
+  const i64 count = kind == MIX_ROW ? P.LB : kind == MIX_COL ? P.nD : P.batch;
+  const i64 signals = kind == MIX_WHOLE ? 1 : P.batch;
+  int T = 1;
+  while (2 * T <= cap && 2 * T <= count) {
+    const i64 n = 2 * i64(T) * L;
+    const bool few = (count + 2 * T - 1) / (2 * T) * signals < ctas;
+    if (n > (2 * T <= lanes ? std::max(most, budget) : budget) || (few && 2 * T > lanes && n > 256)) break;
+    T *= 2;
+  }
+  for (;; T /= 2) {
+    st = mix_configure(P, kind, T);
+    if (st == PFFT_OK || T == 1) return st;
+  }
 }
 
 // Register-resident column pass over two pencil axes (fft_fast2.cuh): the
@@ -234,25 +505,22 @@ bool fast2_axes(const pfft_plan_s& P, int top, int low) {
   return false;
 }
 
+// The register-resident pass of a power-of-two length with T pencils per CTA,
+// or, in split-precision plans, the shared-memory one.  PFFT_ERR_UNSUPPORTED
+// where neither applies.
 pfft_status configure_pass(PassArgs& p, const pfft_plan_s& P, bool cols, int T) {
-  const int ept = P.dtype == PFFT_C64 ? P.ept_c64 : 16;
   p.cols = cols;
-  p.nD = P.nD;
-  p.LB = P.LB;
-  p.m = int(P.m);
-  p.d = P.d;
-  p.batch = int(P.batch);
   p.T = T;
   std::vector<StageDesc> stg;
   if (!cols) {
     p.L = P.nD;
-    if (!axis_stages(stg, P.nD, 1, P.nD, P.tc, P.max2)) return PFFT_ERR_UNSUPPORTED;
+    if (!axis_stages(stg, P.nD, 1, P.nD, P.tc)) return PFFT_ERR_UNSUPPORTED;
     p.groups = (P.LB + T - 1) / T;
   } else {
     p.L = P.LB;
     int sigma = 1;
     for (int s = int(P.pen.size()) - 1; s >= 0; --s) {  // pencil axes, last fastest
-      if (!axis_stages(stg, P.pen[s], sigma, p.tw_n, P.tc, P.max2)) return PFFT_ERR_UNSUPPORTED;
+      if (!axis_stages(stg, P.pen[s], sigma, p.tw_n, P.tc)) return PFFT_ERR_UNSUPPORTED;
       sigma *= P.pen[s];
     }
     p.groups = (P.nD + T - 1) / T;
@@ -301,10 +569,9 @@ pfft_status configure_pass(PassArgs& p, const pfft_plan_s& P, bool cols, int T) 
       p.tc = 0;
     }
   }
-  // generic kernels: 16 points per thread (64 registers, two CTAs per SM)
-  // when the tile fits 512 threads, else 32; the tensor-core stages need 32
-  p.ept = ept;
-  if (P.dtype == PFFT_C64 && !P.tc && ept == 32 && threads_for(p, 16) <= kMaxThreads) p.ept = 16;
+  if (!P.tc) return PFFT_ERR_UNSUPPORTED;  // the mixed-radix passes take it
+  // shared-memory kernels of split-precision plans: 32 points per thread
+  p.ept = 32;
   p.nthreads = threads_for(p, p.ept);
   if (cols && T > 32) p.nthreads = (p.nthreads + T - 1) / T * T;  // each thread keeps one column
   if (p.nthreads > kMaxThreads) return PFFT_ERR_UNSUPPORTED;
@@ -316,10 +583,9 @@ pfft_status configure_pass(PassArgs& p, const pfft_plan_s& P, bool cols, int T) 
   p.dir_off = p.pad ? (nel - 1) + ((nel - 1) >> 4) + 1 : nel;
   // direct-stage tables: omega_R^{g^t} (R - 1 complex) and g^t (R - 1 int), with slack
   p.smem_bytes = int(size_t(p.dir_off + 2 * rmax) * elem_bytes(P.dtype));
-  p.tc = P.tc ? 1 : 0;
+  p.tc = 1;
   p.tc_off = (p.smem_bytes + 15) & ~15;
-  if (p.tc) {  // tensor-core stages (fft_tc.cuh), in the 32-points-per-thread kernels only
-    if (p.ept != 32) return PFFT_ERR_UNSUPPORTED;
+  {  // tensor-core stages (fft_tc.cuh)
     // the hi / lo rows of a stage's 128-butterfly chunks overwrite the tile
     for (int i = 0; i < p.nstages; ++i) {
       const int R = p.st[i].R;
@@ -339,7 +605,8 @@ pfft_status configure_pass(PassArgs& p, const pfft_plan_s& P, bool cols, int T) 
 }
 
 // Choose the pencils-per-CTA count: the largest power of two (<= cap) whose
-// tile fits `budget` elements and the thread limit.
+// tile fits `budget` elements and the thread limit.  PFFT_ERR_UNSUPPORTED when
+// the pass is one for the mixed-radix kernels.
 pfft_status choose_and_configure(PassArgs& p, const pfft_plan_s& P, bool cols, int cap, int budget) {
   const int L = cols ? P.LB : P.nD;
   const int limit = cols ? P.nD : P.LB;
@@ -347,7 +614,7 @@ pfft_status choose_and_configure(PassArgs& p, const pfft_plan_s& P, bool cols, i
   while (T * 2 <= cap && T * 2 <= limit && T * 2 * L <= budget) T *= 2;
   for (;;) {
     pfft_status st = configure_pass(p, P, cols, T);
-    if (st == PFFT_OK) return st;
+    if (st == PFFT_OK || !P.tc) return st;
     if (T == 1) return st;
     T /= 2;
   }
@@ -436,21 +703,42 @@ pfft_status pfft::plan_host(pfft_plan_s& P, int d, const int64_t* Mv) {
   // length-n_b DFTs (twiddle exp(-2 pi i lambda_a mu_b / n) between the passes)
   // and lambda_a becomes one more pencil axis of the column pass.
   const int row_max = P.dtype == PFFT_C64 ? 16384 : 8192;
-  const int ept = P.dtype == PFFT_C64 ? P.ept_c64 : 16;
-  if (P.fs_N > 1 && !tile_fits(int(std::min<i64>(P.fs_N, row_max + 1)), row_max, ept)) {
-    const i64 other = P.m / P.fs_N;
+  const i64 n = P.fs_N;
+  const bool split = n > 1 && (n > row_max || !(P.tc ? tc_tile_fits(int(n), row_max) : mix_fits({int(n)}, int(n), P.dtype)));
+  if (split) {
+    const i64 other = P.m / n;
     int best = 0;
-    for (i64 nb = std::min<i64>(row_max, P.fs_N - 1); nb >= 2; --nb) {
-      if (P.fs_N % nb) continue;
-      const i64 na = P.fs_N / nb;
-      if (other * na > row_max || !tile_fits(int(nb), row_max, ept) || !tile_fits(int(other * na), row_max, ept))
-        continue;
-      best = int(nb);
-      break;
+    double best_cost = 1e30;
+    for (i64 nb = std::min<i64>(row_max, n - 1); nb >= 2; --nb) {
+      if (n % nb) continue;
+      const i64 na = n / nb, lb = other * na;
+      if (lb > row_max) break;  // only grows as nb falls
+      if (P.tc) {  // the longest row
+        if (!tc_tile_fits(int(nb), row_max) || !tc_tile_fits(int(lb), row_max)) continue;
+        best = int(nb);
+        break;
+      }
+      // Stages of both passes, and what a tile loses when it cannot hold eight
+      // pencils: above 2048 points eight adjacent pencils (64-byte accesses) no
+      // longer leave room for a second tile on the SM, above 4096 the accesses
+      // fall to 16 bytes, and fewer than eight rows lambda_a are not eight
+      // adjacent slots.  Weights measured with the passes' own times: 10800 =
+      // 16 15 15 3 runs at 28 instructions a point and stage.
+      double cr = 0, cc = 0;
+      std::vector<int> pen(P.pen.begin(), P.pen.end());
+      pen.push_back(int(na));
+      if (!mix_fits({int(nb)}, int(nb), P.dtype, &cr) || !mix_fits(pen, int(lb), P.dtype, &cc)) continue;
+      const int unit = P.dtype == PFFT_C64 ? 1024 : 512;
+      auto long_tile = [&](i64 L) { return L > 8 * unit ? 60.0 : L > 4 * unit ? 30.0 : L > 2 * unit ? 12.0 : L > unit ? 3.0 : 0.0; };
+      const double c = cr + cc + long_tile(nb) + long_tile(lb) + 3.0 * std::max<i64>(0, 8 - na);
+      if (c < best_cost) {
+        best_cost = c;
+        best = int(nb);
+      }
     }
     if (!best) return PFFT_ERR_UNSUPPORTED;
     P.nD = best;
-    P.fs_na = int(P.fs_N / best);
+    P.fs_na = int(n / best);
     P.pen.push_back(P.fs_na);
   }
   if (P.pen.size() > size_t(kMaxSub)) return PFFT_ERR_UNSUPPORTED;
@@ -483,6 +771,19 @@ std::vector<i64> combo(const std::vector<std::vector<i64>>& gens, const std::vec
   return y;
 }
 }  // namespace
+
+// The tile of one kind for a points budget: whole and plain row tiles need no
+// adjacent pencils, the others four.  Small tiles are the faster ones, several
+// of them filling an SM's 1024 threads in different phases (M = [[1200, 240],
+// [0, 1080]] x 8 there and back: 0.446 ms with 2048 points, 0.468 with 4096),
+// except that four adjacent pencils of a long cycle are worth 8192 points
+// ([[2048, 8], [0, 2048]] x 8: 1.03 ms, against 1.17 with two pencils of 2048).
+static pfft_status mix_tile(pfft_plan_s& P, int kind, int budget, int ctas) {
+  const bool adjacent = kind == MIX_COL || (kind == MIX_ROW && P.fs_na > 1);
+  const bool c64 = P.dtype == PFFT_C64;
+  return mix_choose(P, kind, 64, kind == MIX_WHOLE ? (c64 ? 2048 : 1024) : budget, c64 ? 8192 : 4096, adjacent ? 4 : 1,
+                    ctas);
+}
 
 pfft_status pfft::plan_device(pfft_plan_s& P) {
   const int d = P.d, D = P.D;
@@ -555,6 +856,7 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
       PIinv[pos] = int(mu);
     }
   }
+  P.PIinv = PIinv;
   // index tables
   const int ts = d <= 2 ? 2 : 4;  // int32 per entry, so that one vector load fetches a point
   std::vector<int> tab(size_t(2 * LB + 2 * nD) * ts + 2 * nD, 0);
@@ -606,11 +908,22 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
     for (int a : P.pen) l = l / gcd64(l, a) * a;
     if (npen >= 1 && nD % l != 0) {
       col_n = int(l);
+      P.col_n = col_n;
       if (int e_ = P.alloc(&P.tw_col, size_t(col_n) * eb)) return pfft_status(e_);
       if (launch_twiddles(P.tw_col, col_n, P.dtype, 0) != 0) return PFFT_ERR_CUDA;
     }
   }
-  if (npen >= 1 && P.own_workspace)
+  // Whole signals in one tile: one launch, no workspace.  Up to 8192 complex64
+  // points two such tiles share an SM; up to 16384 one tile takes the SM, worth
+  // it once the batch alone nearly fills the chip (otherwise two passes use
+  // more SMs).
+  {
+    const i64 half = P.dtype == PFFT_C64 ? 8192 : 4096;
+    std::vector<int> axes(P.pen.begin(), P.pen.end());
+    axes.push_back(nD);
+    P.mixed[MIX_WHOLE] = !P.tc && na == 1 && P.m <= (P.batch >= 64 ? 2 * half : half) && mix_fits(axes, int(P.m), P.dtype);
+  }
+  if (npen >= 1 && P.own_workspace && !P.mixed[MIX_WHOLE])
     if (int e_ = P.alloc(&P.ws, size_t(P.m) * P.batch * eb)) return pfft_status(e_);
   if (na > 1) {  // exp(-2 pi i t / n) for t < n, as lo[t & 2047] * hi[t >> 11]
     const int nhi = int((P.fs_N + 2047) >> 11);
@@ -685,6 +998,12 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
     p->tw = colt ? P.tw_col : P.tw;
     p->tw_n = colt ? col_n : nD;
     p->ts = ts;
+    p->cols = p == &P.colp;
+    p->nD = nD;
+    p->LB = LB;
+    p->m = int(P.m);
+    p->d = d;
+    p->batch = int(P.batch);
     p->status = P.status;
     p->spin_limit = kSpinLimit;
     set_box(p->boxH, P.H);
@@ -707,11 +1026,66 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
     p->fs_lo = P.fs_tab;
     p->fs_hi = P.fs_tab ? static_cast<const char*>(P.fs_tab) + size_t(2048) * eb : nullptr;
   }
-  pfft_status st = choose_and_configure(P.rowp, P, false, 64, std::max(budget, nD));
-  if (st != PFFT_OK) return st;
-  if (npen >= 1) {
-    // generic column tiles may hold many short columns (split last cycles)
-    st = choose_and_configure(P.colp, P, true, P.generic_only ? 512 : 16, std::max(budget, LB));
+  // The register-resident kernels take power-of-two passes (rows of a cycle that
+  // is not split, whose box loads need no lanes across rows); the mixed-radix
+  // ones everything else.
+  auto no_pass = [](PassArgs& p) { p.fast = p.tc = 0; };
+  if (P.mixed[MIX_WHOLE]) {
+    no_pass(P.rowp);
+    no_pass(P.colp);
+  } else {
+    pfft_status st = PFFT_ERR_UNSUPPORTED;
+    if (P.tc || na == 1) st = choose_and_configure(P.rowp, P, false, 64, std::max(budget, nD));
+    if (st != PFFT_OK) {
+      if (P.tc) return st;
+      no_pass(P.rowp);
+      P.mixed[MIX_ROW] = true;
+    }
+    if (npen >= 1) {
+      st = choose_and_configure(P.colp, P, true, P.generic_only ? 512 : 16, std::max(budget, LB));
+      if (st != PFFT_OK) {
+        if (P.tc) return st;
+        no_pass(P.colp);
+        P.mixed[MIX_COL] = true;
+      }
+    }
+  }
+  for (int kind = 0; kind < 3; ++kind) {
+    if (!P.mixed[kind]) continue;
+    MixDesc& a = P.mix[kind];
+    std::memset(&a, 0, sizeof(a));
+    const PassArgs& p = kind == MIX_COL ? P.colp : P.rowp;
+    a.d = d;
+    a.ts = ts;
+    a.nD = nD;
+    a.LB = LB;
+    a.m = int(P.m);
+    a.batch = int(P.batch);
+    a.Atab = p.Atab;
+    a.Btab = p.Btab;
+    a.Ctab = p.Ctab;
+    a.Etab = p.Etab;
+    a.PIinv = p.PIinv;
+    a.fs_lo = p.fs_lo;
+    a.fs_hi = p.fs_hi;
+    a.fs_na = na;
+    a.fs_div = p.fs_div;
+    a.nsub = p.nsub;
+    for (int s = 0; s < npen; ++s) {
+      a.sub_n[s] = p.sub_n[s];
+      a.sub_div[s] = p.sub_div[s];
+      a.alpha[s] = p.alpha[s];
+    }
+    a.boxH = p.boxH;
+    a.boxG = p.boxG;
+    if (kind == MIX_WHOLE) {
+      if (int e_ = P.alloc((void**)&P.maps, 2 * size_t(P.m) * sizeof(int))) return pfft_status(e_);
+      a.map_in = P.maps;
+      a.map_out = P.maps + P.m;
+      if (launch_whole_maps(a, P.rowp.PI, P.maps, P.maps + P.m, 0) != 0) return PFFT_ERR_CUDA;
+    }
+    // a launch of its own leaves at least two tiles per SM where the lanes of its accesses allow
+    const pfft_status st = mix_tile(P, kind, 2048, P.generic_only ? 0 : 304);
     if (st != PFFT_OK) return st;
   }
   // stage twiddle tables of the register-resident passes, gathered on the
@@ -873,11 +1247,14 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
 }
 
 pfft_status pfft::plan_retile(pfft_plan_s& P, int row_budget, int col_budget, int max2) {
-  if (!P.generic_only || P.D == 0 || (max2 != 16 && max2 != 8)) return PFFT_ERR_ARG;
+  if (!P.generic_only || P.tc || P.D == 0 || (max2 != 16 && max2 != 8)) return PFFT_ERR_ARG;
   P.max2 = max2;
-  pfft_status st = choose_and_configure(P.rowp, P, false, 64, std::max(row_budget, P.nD));
-  if (st != PFFT_OK || P.pen.empty()) return st;
-  return choose_and_configure(P.colp, P, true, 512, std::max(col_budget, P.LB));
+  for (int kind = 0; kind < 3; ++kind) {
+    if (!P.mixed[kind]) continue;
+    const pfft_status st = mix_tile(P, kind, kind == MIX_COL ? col_budget : row_budget, 0);
+    if (st != PFFT_OK) return st;
+  }
+  return PFFT_OK;
 }
 
 void pfft::plan_release(pfft_plan_s* P) {
@@ -887,8 +1264,13 @@ void pfft::plan_release(pfft_plan_s* P) {
     plan_release(P->tr);
   }
   if (!P->arena) {
-    for (void* p : {(void*)P->dtab, P->tw, P->tw_col, P->ws, P->stw, P->fs_tab, (void*)P->runs, (void*)P->status})
+    for (void* p : {(void*)P->dtab, P->tw, P->tw_col, P->ws, P->stw, P->fs_tab, (void*)P->runs, (void*)P->status,
+                    (void*)P->maps})
       if (p) cudaFree(p);
+    for (auto& by_max2 : P->stages)
+      for (auto& S : by_max2)
+        for (void* p : {S.stw, (void*)S.gtab, (void*)S.psout})
+          if (p) cudaFree(p);
   }
   delete P;
 }
@@ -1017,8 +1399,25 @@ extern "C" pfft_status pfft_device_index_map(pfft_plan p, int which, int64_t* sl
              : PFFT_ERR_CUDA;
 }
 
-static pfft_status run_pass(pfft_plan_s* P, PassArgs a, int load, int store, int cin, int cout,
-                            double scale, const void* in, void* out, cudaStream_t s, int which) {
+// One pass of plan t (kind: row, column or whole tiles), its time recorded under P.
+static pfft_status run_pass(pfft_plan_s* P, const pfft_plan_s* t, int kind, int load, int store, int cin, int cout,
+                            double scale, const void* in, void* out, cudaStream_t s) {
+  const int which = kind == MIX_COL ? 1 : 0;
+  if (t->mixed[kind]) {
+    MixDesc a = t->mix[kind];
+    a.load_mode = load;
+    a.store_mode = store;
+    a.conj_in = cin;
+    a.conj_out = cout;
+    a.scale = scale;
+    a.in = in;
+    a.out = out;
+    P->prof.begin(which, s);
+    if ((P->dtype == PFFT_C64 ? launch_mixed_c64(a, s) : launch_mixed_c128(a, s)) != 0) return PFFT_ERR_CUDA;
+    P->prof.end(which, s);
+    return PFFT_OK;
+  }
+  PassArgs a = kind == MIX_COL ? t->colp : t->rowp;
   a.load_mode = load;
   a.store_mode = store;
   a.conj_in = cin;
@@ -1039,18 +1438,18 @@ static pfft_status transform_transposed(pfft_plan p, const void* in, void* out, 
   pfft_plan_s* t = p->tr;
   const double scale = 1.0 / std::sqrt(double(p->m));
   const int c = inverse ? 1 : 0;
-  if (t->pen.empty()) {
-    return run_pass(p, t->rowp, inverse ? MAP_BOX_H : MAP_BOX_G, inverse ? MAP_BOX_G : MAP_BOX_H, c, c, scale, in,
-                    out, s, 0);
+  if (t->pen.empty() || t->mixed[MIX_WHOLE]) {
+    return run_pass(p, t, t->mixed[MIX_WHOLE] ? MIX_WHOLE : MIX_ROW, inverse ? MAP_BOX_H : MAP_BOX_G,
+                    inverse ? MAP_BOX_G : MAP_BOX_H, c, c, scale, in, out, s);
   }
   if (inverse) {
-    pfft_status st = run_pass(p, t->rowp, MAP_BOX_H, MAP_WS, 1, 0, 1.0, in, t->ws, s, 0);
+    pfft_status st = run_pass(p, t, MIX_ROW, MAP_BOX_H, MAP_WS, 1, 0, 1.0, in, t->ws, s);
     if (st != PFFT_OK) return st;
-    return run_pass(p, t->colp, MAP_WS, MAP_BOX_G, 0, 1, scale, t->ws, out, s, 1);
+    return run_pass(p, t, MIX_COL, MAP_WS, MAP_BOX_G, 0, 1, scale, t->ws, out, s);
   }
-  pfft_status st = run_pass(p, t->colp, MAP_BOX_G, MAP_WS, 0, 0, 1.0, in, t->ws, s, 1);
+  pfft_status st = run_pass(p, t, MIX_COL, MAP_BOX_G, MAP_WS, 0, 0, 1.0, in, t->ws, s);
   if (st != PFFT_OK) return st;
-  return run_pass(p, t->rowp, MAP_WS, MAP_BOX_H, 0, 0, scale, t->ws, out, s, 0);
+  return run_pass(p, t, MIX_ROW, MAP_WS, MAP_BOX_H, 0, 0, scale, t->ws, out, s);
 }
 
 static pfft_status transform_route(pfft_plan p, const void* in, void* out, cudaStream_t s, bool inverse,
@@ -1063,18 +1462,18 @@ static pfft_status transform_route(pfft_plan p, const void* in, void* out, cudaS
   }
   if (via_tr) return transform_transposed(p, in, out, s, inverse);
   const int ci = inverse ? 1 : 0;
-  if (p->pen.empty()) {
-    return run_pass(p, p->rowp, inverse ? MAP_BOX_G : MAP_BOX_H, inverse ? MAP_BOX_H : MAP_BOX_G, ci, ci,
-                    scale, in, out, s, 0);
+  if (p->pen.empty() || p->mixed[MIX_WHOLE]) {
+    return run_pass(p, p, p->mixed[MIX_WHOLE] ? MIX_WHOLE : MIX_ROW, inverse ? MAP_BOX_G : MAP_BOX_H,
+                    inverse ? MAP_BOX_H : MAP_BOX_G, ci, ci, scale, in, out, s);
   }
   if (!inverse) {
-    pfft_status st = run_pass(p, p->rowp, MAP_BOX_H, MAP_WS, 0, 0, 1.0, in, p->ws, s, 0);
+    pfft_status st = run_pass(p, p, MIX_ROW, MAP_BOX_H, MAP_WS, 0, 0, 1.0, in, p->ws, s);
     if (st != PFFT_OK) return st;
-    return run_pass(p, p->colp, MAP_WS, MAP_BOX_G, 0, 0, scale, p->ws, out, s, 1);
+    return run_pass(p, p, MIX_COL, MAP_WS, MAP_BOX_G, 0, 0, scale, p->ws, out, s);
   }
-  pfft_status st = run_pass(p, p->colp, MAP_BOX_G, MAP_WS, 1, 0, 1.0, in, p->ws, s, 1);
+  pfft_status st = run_pass(p, p, MIX_COL, MAP_BOX_G, MAP_WS, 1, 0, 1.0, in, p->ws, s);
   if (st != PFFT_OK) return st;
-  return run_pass(p, p->rowp, MAP_WS, MAP_BOX_H, 0, 1, scale, p->ws, out, s, 0);
+  return run_pass(p, p, MIX_ROW, MAP_WS, MAP_BOX_H, 0, 1, scale, p->ws, out, s);
 }
 
 static pfft_status transform(pfft_plan p, const void* in, void* out, void* stream, bool inverse) {
@@ -1136,7 +1535,7 @@ static pfft_status plan_route(pfft_plan_s& P, int d, const int64_t* M, unsigned 
   } catch (const LatticeError& e) {
     st = pfft_status(e.code);
   }
-  if (st == PFFT_OK && (T->rowp.pipe || T->pen.size() != P.pen.size())) st = PFFT_ERR_UNSUPPORTED;
+  if (st == PFFT_OK && (T->rowp.pipe || T->pen.size() != P.pen.size() || T->mixed[MIX_WHOLE] != P.mixed[MIX_WHOLE])) st = PFFT_ERR_UNSUPPORTED;
   if (st != PFFT_OK) {
     plan_release(T);
     return force ? st : PFFT_OK;

@@ -166,8 +166,8 @@ __global__ void __launch_bounds__(512, 1) row_pipe_kernel(PassArgs a) {
     __syncthreads();  // S is read
     if constexpr (X1S) {
       // ---- tail stage (radix 16) and exchange 1 in one round through S and X
-      dft16(v);
-      dft16(v + 16);
+      dft16<C, false>(v);
+      dft16<C, false>(v + 16);
 #pragma unroll
       for (int q = 0; q < 2; ++q)
 #pragma unroll
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(512, 1) row_pipe_kernel(PassArgs a) {
       // ---- tail stage (radix 16) and exchange 1, one round per butterfly
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        dft16(v + 16 * q);
+        dft16<C, false>(v + 16 * q);
 #pragma unroll
         for (int r = 0; r < 16; ++r) X[xphys((p << 4) | r)] = v[16 * q + r];
         __syncthreads();
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(512, 1) row_pipe_kernel(PassArgs a) {
     {
       const int k = p & 15;
       if (k) main_twiddle<C, R>(v, stw + a.stw_off[0] + k * 5);
-      dft_pow2<C, R>(v);
+      dft_pow2<C, R, false>(v);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         if ((h ^ (p >> 8)) & 1)
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(512, 1) row_pipe_kernel(PassArgs a) {
     }
     // ---- stage 1 (Ns = 512): v[r] = frequency p + P r
     if (p) main_twiddle<C, R>(v, stw + a.stw_off[1] + p * 5);
-    dft_pow2<C, R>(v);
+    dft_pow2<C, R, false>(v);
 
     // ---- output
     if constexpr (FWD && DIRECT) {

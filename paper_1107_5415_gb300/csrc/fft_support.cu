@@ -1,6 +1,7 @@
 // Transform support kernels: pass dispatch, twiddle table, index probe.
 #include <cuda_runtime.h>
 
+#include "fft_mixed.hpp"
 #include "fft_plan.hpp"
 
 namespace pfft {
@@ -116,6 +117,46 @@ int launch_index_probe(const PassArgs& rowp, const PassArgs& colp, int which, in
   const int blk = 256;
   const int grd = int((int64_t(rowp.m) + blk - 1) / blk);
   index_probe_kernel<<<grd, blk, 0, s>>>(rowp, rowp.PIinv + rowp.nD, which, out);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+// Stage tables of the mixed-radix passes (exact integer argument, FP64 sincospi).
+template <typename C>
+__global__ void mixed_table_kernel(C* tab, MixTableArgs t) {
+  using Rl = decltype(C::x);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < t.total; i += gridDim.x * blockDim.x) {
+    int s = 0;
+    while (i >= t.off[s + 1]) ++s;
+    const int Ns = t.Ns[s], q = Ns * t.R[s];
+    const int b = (i - t.off[s]) / Ns, k = i - t.off[s] - b * Ns;
+    double sn, c;
+    sincospi(2.0 * double((long long)(k) << b) / double(q), &sn, &c);
+    tab[i] = cmake<C>(Rl(c), Rl(-sn));
+  }
+}
+
+int launch_mixed_tables(void* tab, const MixTableArgs& t, int dtype, cudaStream_t s) {
+  if (t.total == 0) return 0;
+  const int blk = 256, grd = (t.total + blk - 1) / blk;
+  if (dtype == 0)
+    mixed_table_kernel<float2><<<grd, blk, 0, s>>>(static_cast<float2*>(tab), t);
+  else
+    mixed_table_kernel<double2><<<grd, blk, 0, s>>>(static_cast<double2*>(tab), t);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+// Tile position of every slot of the two boxes (tiles that hold whole signals:
+// row r, element e at r nD + e).
+__global__ void whole_map_kernel(MixDesc a, const int* __restrict__ PI, int* map_in, int* map_out) {
+  for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < a.m; w += gridDim.x * blockDim.x) {
+    const int row = w / a.nD, e = w - row * a.nD;
+    map_in[box_sum_slot(a.boxH, a.Atab + row * a.ts, a.Btab + e * a.ts)] = w;
+    map_out[box_sum_slot(a.boxG, a.Ctab + row * a.ts, a.Etab + PI[e] * a.ts)] = w;
+  }
+}
+
+int launch_whole_maps(const MixDesc& a, const int* PI, int* map_in, int* map_out, cudaStream_t s) {
+  whole_map_kernel<<<(a.m + 255) / 256, 256, 0, s>>>(a, PI, map_in, map_out);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

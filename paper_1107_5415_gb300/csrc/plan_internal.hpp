@@ -7,9 +7,19 @@
 #include <vector>
 
 #include "../../include/pfft.h"
+#include "fft_mixed.hpp"
 #include "fft_plan.hpp"
 #include "lattice.hpp"
 #include "plan_common.hpp"
+
+// The stages of one kind of mixed-radix tile and their device tables.
+struct MixStages {
+  bool ready = false;
+  std::vector<pfft::MixStage> st;  // sig, blk and the divisors of a tile are set with its T
+  void* stw = nullptr;
+  int* gtab = nullptr;
+  int* psout = nullptr;
+};
 
 struct pfft_plan_s {
   int d = 0;
@@ -32,18 +42,26 @@ struct pfft_plan_s {
   bool generic_only = false;     // shared-memory Stockham kernels only (grouped launches)
   bool own_workspace = true;     // allocate the LB x nD workspace
   bool tc = false;               // split-precision tensor-core radix-16 / 32 stages
-  int ept_c64 = 32;              // complex64 points per thread of the generic kernels
-  int max2 = 16;                 // largest power-of-two radix of the generic kernels (16 or 8)
+  int max2 = 16;                 // largest power-of-two radix of the mixed-radix passes (16 or 8)
   // device state
   int device = 0;
   int* dtab = nullptr;
   void* tw = nullptr;
+  int col_n = 0;           // order of tw_col
   void* tw_col = nullptr;  // column-pass table when its axes do not divide nD (split last cycle)
   void* ws = nullptr;
   void* stw = nullptr;  // stage twiddle tables of the register-resident passes
   int* runs = nullptr;  // bulk-copy runs of the row pass
   int* status = nullptr;  // device status word
   pfft::PassArgs rowp{}, colp{};
+  // mixed-radix passes (fft_mixed.cuh), by MixKind: which ones the plan runs
+  // (a whole tile replaces both passes), their descriptors, and the stages for
+  // max2 = 16 [0] and 8 [1]
+  bool mixed[3] = {false, false, false};
+  pfft::MixDesc mix[3]{};
+  MixStages stages[2][3];
+  std::vector<int> PIinv;  // element of each column position
+  int* maps = nullptr;  // whole tiles: tile positions of the input box's slots, then of the output box's
   pfft::Profiler prof;
   // Transposed route.  Entry (k, y) of F(M) is entry (y, k) of F(M^T) in box
   // order (eq. (Fouriermatrix) read for M^T), so the forward transform of M
