@@ -96,8 +96,8 @@ __global__ void __launch_bounds__(kSplitThreads) grouped_prime_kernel(const Prim
   const long long mN = it.P.mN;
   if (w >= mN * it.P.nch) return;
   const int ch = int(w / mN), gs = int(w - ch * mN);
-  prime_split_item<C, 0>(it.P, gs, ch * kPrimeChunk, chat + it.in_off, nullptr, nullptr, nullptr,
-                         sc + it.sc_off + gs, wv + it.wv_off + gs, mN);
+  prime_item<C, 0>(it.P, gs, ch * kPrimeChunk, chat + it.in_off, nullptr, nullptr, nullptr,
+                   sc + it.sc_off + gs, wv + it.wv_off + gs, mN);
 }
 
 // Bounded wait (thread 0) until *done reaches need: spin_limit tries and about
@@ -141,9 +141,9 @@ __device__ __noinline__ void queue_prime(const PrimeItem& pi, int local, const Q
   const long long mN = pi.P.mN;
   if (threadIdx.x >= kMaxThreads || w >= mN * pi.P.nch) return;
   const int ch = int(w / mN), gs = int(w - ch * mN);
-  prime_split_item<C, 0, true>(pi.P, gs, ch * kPrimeChunk, static_cast<const C*>(g.base[2]) + pi.in_off, nullptr,
-                               nullptr, nullptr, static_cast<C*>(g.sc) + pi.sc_off + gs,
-                               static_cast<C*>(g.wv) + pi.wv_off + gs, mN);
+  prime_item<C, 0, true>(pi.P, gs, ch * kPrimeChunk, static_cast<const C*>(g.base[2]) + pi.in_off, nullptr,
+                         nullptr, nullptr, static_cast<C*>(g.sc) + pi.sc_off + gs,
+                         static_cast<C*>(g.wv) + pi.wv_off + gs, mN);
 }
 
 // One unit of the launch: find its item, wait (bounded) for its dependency,

@@ -177,6 +177,71 @@ __device__ __forceinline__ int box_sum_slot_t(const BoxDesc& B, const int* a, co
   }
 }
 
+// Slot of a box point that advances by a fixed box point.  A carry out of the
+// last coordinate takes H's last column off the others, so each coordinate has
+// one step without and one with the carries below it; the first coordinate is
+// carried in the slot itself (it wraps exactly when the slot passes m).
+template <int DIM>
+struct BoxWalk {
+  int slot, m;
+  int y1, c1, h1;          // DIM 2: last coordinate; DIM 3: middle one
+  int y2, c2, h2, c1c;     // DIM 3: last coordinate; middle step with its carry
+  int d0, d1, d2, d3;      // slot steps by carries (last | middle << 1)
+  __device__ __forceinline__ static int wrap(int x, int n) { return x < 0 ? x + n : x >= n ? x - n : x; }
+  __device__ __forceinline__ BoxWalk(const BoxDesc& B, const int* y, const int* c, int m_) : m(m_) {
+    if constexpr (DIM == 1) {
+      slot = y[0];
+      d0 = c[0];
+    } else if constexpr (DIM == 2) {
+      slot = y[0] * B.stride[0] + y[1];
+      y1 = y[1];
+      c1 = c[1];
+      h1 = B.H[1][1];
+      d0 = c[0] * B.stride[0] + c1;
+      d1 = wrap(c[0] - B.H[0][1], B.H[0][0]) * B.stride[0] + c1 - h1;
+    } else {
+      slot = y[0] * B.stride[0] + y[1] * B.stride[1] + y[2];
+      y2 = y[2];
+      c2 = c[2];
+      h2 = B.H[2][2];
+      y1 = y[1];
+      c1 = c[1];
+      h1 = B.H[1][1];
+      const int H0 = B.H[0][0], s0 = B.stride[0], s1 = B.stride[1];
+      // middle step with the carry of the last coordinate, kept in [0, h1): a
+      // negative one borrows a column of its own
+      const int r1 = c1 - B.H[1][2];
+      c1c = r1 < 0 ? r1 + h1 : r1;
+      const int x0 = wrap(c[0] - B.H[0][2], H0);                 // after the last coordinate's carry
+      const int x0c = r1 < 0 ? wrap(x0 + B.H[0][1], H0) : x0;    // and the borrow
+      d0 = c[0] * s0 + c1 * s1 + c2;
+      d1 = x0c * s0 + c1c * s1 + c2 - h2;
+      d2 = wrap(c[0] - B.H[0][1], H0) * s0 + (c1 - h1) * s1 + c2;
+      d3 = wrap(x0c - B.H[0][1], H0) * s0 + (c1c - h1) * s1 + c2 - h2;
+    }
+  }
+  __device__ __forceinline__ void step() {
+    if constexpr (DIM == 1) {
+      slot += d0;
+    } else if constexpr (DIM == 2) {
+      y1 += c1;
+      const bool p = y1 >= h1;
+      if (p) y1 -= h1;
+      slot += p ? d1 : d0;
+    } else {
+      y2 += c2;
+      const bool p = y2 >= h2;
+      if (p) y2 -= h2;
+      y1 += p ? c1c : c1;
+      const bool q = y1 >= h1;
+      if (q) y1 -= h1;
+      const int lo = q ? d2 : d0, hi = q ? d3 : d1;
+      slot += p ? hi : lo;
+    }
+    if (slot >= m) slot -= m;
+  }
+};
+
 // A table entry of a box point: TS = 2 (d <= 2) or 4 (d = 3, 4) int32,
 // fetched with one vector load.
 template <int TS>

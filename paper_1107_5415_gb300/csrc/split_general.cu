@@ -21,6 +21,7 @@
 #include "device_common.cuh"
 #include "lattice.hpp"
 #include "split_prime.cuh"
+#include "wavelet_kernels.cuh"
 
 namespace pfft {
 
@@ -108,11 +109,64 @@ __global__ void __launch_bounds__(256) split_prime_kernel(PrimeDesc P, int batch
        w += (long long)gridDim.x * blockDim.x) {
     const int ch = int(w / P.mN), gs = int(w - (long long)ch * P.mN);
     const long long off = (long long)b * P.mN + gs;
-    prime_split_item<C, MODE>(P, gs, ch * kPrimeChunk, MODE == 0 ? cin + (long long)b * P.mM : nullptr,
-                              MODE == 0 ? nullptr : cout + (long long)b * P.mM, MODE == 0 ? nullptr : din + off,
-                              MODE == 0 ? nullptr : din + off + dstride, MODE == 0 ? dout + off : nullptr,
-                              MODE == 0 ? dout + off + dstride : nullptr, dstride);
+    prime_item<C, MODE>(P, gs, ch * kPrimeChunk, MODE == 0 ? cin + (long long)b * P.mM : nullptr,
+                        MODE == 0 ? nullptr : cout + (long long)b * P.mM, MODE == 0 ? nullptr : din + off,
+                        MODE == 0 ? nullptr : din + off + dstride, MODE == 0 ? dout + off : nullptr,
+                        MODE == 0 ? dout + off + dstride : nullptr, dstride);
   }
+}
+
+// Small primes on the int32 index path: one thread per fibre, which keeps its
+// slots, weights and band phases for the signals [y chunk, (y + 1) chunk).
+// Evaluating them again for every signal, with 64-bit remainders, was most of
+// the time ([[768, 96], [0, 729]] x 8 by diag(3, 1), split and merged: 0.252 ms,
+// now 0.092).
+template <typename C, int MODE, int PR, int DIM>
+__global__ void __launch_bounds__(256) split_prime_small_kernel(const __grid_constant__ PrimeDesc P, int batch,
+                                                                int chunk, const C* __restrict__ cin,
+                                                                C* __restrict__ cout, const C* __restrict__ din,
+                                                                C* __restrict__ dout) {
+  const int b0 = blockIdx.y * chunk, nb = min(chunk, batch - b0);
+  const long long dstride = (long long)batch * P.mN;
+  for (int gs = blockIdx.x * blockDim.x + threadIdx.x; gs < P.mN; gs += gridDim.x * blockDim.x) {
+    const long long om = (long long)b0 * P.mM, on = (long long)b0 * P.mN + gs;
+    prime_fibre_small<C, MODE, PR, DIM>(P, gs, nb, MODE == 0 ? cin + om : nullptr, MODE == 0 ? nullptr : cout + om,
+                                        MODE == 0 ? nullptr : din + on, MODE == 0 ? nullptr : din + on + dstride,
+                                        MODE == 0 ? dout + on : nullptr, MODE == 0 ? dout + on + dstride : nullptr,
+                                        dstride);
+  }
+}
+
+template <typename C, int PR, int DIM>
+static void launch_prime_small_t(const PrimeDesc& P, int batch, int mode, const void* src, void* dst, cudaStream_t s) {
+  unsigned gx, gy;
+  int chunk;
+  split_grid(P.mN, batch, gx, gy, chunk);
+  if (mode == 0)
+    split_prime_small_kernel<C, 0, PR, DIM><<<dim3(gx, gy), 256, 0, s>>>(P, batch, chunk, static_cast<const C*>(src),
+                                                                         nullptr, nullptr, static_cast<C*>(dst));
+  else
+    split_prime_small_kernel<C, 1, PR, DIM><<<dim3(gx, gy), 256, 0, s>>>(P, batch, chunk, nullptr, static_cast<C*>(dst),
+                                                                         static_cast<const C*>(src), nullptr);
+}
+
+// Launches the small-prime kernel when one matches; false otherwise.
+template <typename C>
+static bool launch_prime_small(const PrimeDesc& P, int batch, int mode, const void* src, void* dst, cudaStream_t s) {
+  if (!P.small || (P.d != 2 && P.d != 3)) return false;
+#define PFFT_SMALL_PRIME(PR)                                   \
+  case PR:                                                     \
+    P.d == 2 ? launch_prime_small_t<C, PR, 2>(P, batch, mode, src, dst, s) \
+             : launch_prime_small_t<C, PR, 3>(P, batch, mode, src, dst, s); \
+    return true;
+  switch (P.p) {
+    PFFT_SMALL_PRIME(2)
+    PFFT_SMALL_PRIME(3)
+    PFFT_SMALL_PRIME(5)
+    PFFT_SMALL_PRIME(7)
+    default: return false;
+  }
+#undef PFFT_SMALL_PRIME
 }
 
 }  // namespace pfft
@@ -263,6 +317,28 @@ pfft_status pfft::describe_prime_level(int d, const int64_t* Mv, const int64_t* 
     P.phw[i] = sM > 0 ? r : (m - r) % m;
   }
   P.nch = int((p + kPrimeChunk - 1) / kPrimeChunk);
+  // int32 index path
+  {
+    i128 pbound = 0;
+    for (int r = 0; r < d; ++r) {
+      i64 c = P.phw[r];
+      if (2 * c > m) c -= m;
+      P.ph32[r] = int(c);
+      pbound += (i128)(c < 0 ? -c : c) * HN(r, r);
+    }
+    const i128 lim = (i128)1 << 29;
+    P.small = d <= 3 && p <= kPrimeSmallP && bound < lim && pbound < lim && m < (i64(1) << 29);
+    if (P.small) {
+      for (int k = 0; k < d * d; ++k) P.K32[k] = int(P.K[k]);
+      P.divq.init(uint32_t(m));
+      P.divp.init(uint32_t(p));
+      P.cq = int(bound / m) + 1;
+      P.offq = int(P.cq * m);
+      P.kp = int((P.cq + 2 + p - 1) / p * p);
+      for (int r = 0; r < d; ++r) P.v32[r] = int(P.v[r]);
+      P.offph = int((i64(pbound) / m + 1) * m);
+    }
+  }
   *out = P;
   return PFFT_OK;
 }
@@ -278,12 +354,15 @@ static pfft_status prime_run(int mode, int d, const int64_t* M, const int64_t* J
   }
   if (st != PFFT_OK) return st;
   if (int64_t(P.mM) * batch >= (int64_t(1) << 40)) return PFFT_ERR_OVERFLOW;
+  cudaStream_t s = (cudaStream_t)stream;
+  if (dtype == PFFT_C64 ? launch_prime_small<float2>(P, int(batch), mode, src, dst, s)
+                        : launch_prime_small<double2>(P, int(batch), mode, src, dst, s))
+    return cudaGetLastError() == cudaSuccess ? PFFT_OK : PFFT_ERR_CUDA;
   const int blk = 256;
   long long gx = ((long long)P.mN * P.nch + blk - 1) / blk;
   const long long cap = (152LL * 16 + batch - 1) / batch;
   if (gx > cap) gx = cap;
   dim3 grid(unsigned(gx < 1 ? 1 : gx), unsigned(batch));
-  cudaStream_t s = (cudaStream_t)stream;
   if (dtype == PFFT_C64) {
     using C = float2;
     if (mode == 0)

@@ -49,7 +49,17 @@ struct alignas(16) PrimeDesc {
   long long v[4];          // n in J^T Z^d <=> v . n = 0 mod p; v . l = 1
   long long phw[4];        // sign(det M) adj(M) (J z) mod q: phase numerator of g is g . phw
   int nch;                 // chunks of kPrimeChunk band outputs per fibre
+  // int32 index path (d <= 3, p <= kPrimeSmallP and every numerator below 2^29)
+  int small;
+  int K32[16];
+  FastDiv divq, divp;
+  int offq, cq;            // offq = cq q >= |K h|
+  int kp;                  // multiple of p that makes every shift k non-negative
+  int v32[4];              // v mod p
+  int ph32[4], offph;      // phw centred; multiple of q >= |ph32 . g|
 };
+
+constexpr int kPrimeSmallP = 1024;
 
 // Box point g + t s reduced into the box of H (coordinates of g, s in the
 // box, 0 <= t < 2^20): last coordinate first, exact in 64 bits.
@@ -239,6 +249,222 @@ __device__ __forceinline__ void prime_split_item(const PrimeDesc& P, int gs, int
         if (r < P.d) y[r] += P.shift[r];
       box_fix(P.HM, y);
     }
+  }
+}
+
+// ---- int32 index path: the same quantities from FastDiv divisions
+template <int DIM>
+__device__ __forceinline__ void prime_fibre(const PrimeDesc& P, int gs, int* g) {
+  int s = gs;
+#pragma unroll
+  for (int r = DIM - 1; r > 0; --r) {
+    const int qd = P.divHN[r].div(s);
+    g[r] = s - qd * P.HNext[r];
+    s = qd;
+  }
+  g[0] = s;
+}
+
+// Calls add(t, w) for every member t of the fibre of g that a shift gives weight
+// w (the same member may come up again).
+template <typename Rl, int DIM, typename Add>
+__device__ __forceinline__ void prime_weights_small(const PrimeDesc& P, const int* g, Add add) {
+  int k0[DIM], two[DIM];
+  Rl w = Rl(1);
+  int n = 0;
+#pragma unroll
+  for (int j = 0; j < DIM; ++j) {
+    int acc = P.offq;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) acc += P.K32[j * DIM + i] * g[i];
+    const int f = P.divq.div(acc);
+    const int r = acc - f * P.divq.d;  // a + k q = r in [0, q) for k = cq - f
+    const int twice = 2 * r, q = int(P.divq.d);
+    two[j] = twice == q;               // half way: k - 1 and k with weight 1/2 each
+    k0[j] = P.kp + P.cq - f - (twice >= q);
+    if (two[j]) {
+      w *= Rl(0.5);
+      ++n;
+    }
+  }
+  for (int c = 0; c < (1 << n); ++c) {
+    int t = 0, bit = 0;
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) {
+      int k = k0[j];
+      if (two[j]) k += (c >> bit++) & 1;
+      t += P.v32[j] * P.divp.mod(k);
+    }
+    add(P.divp.mod(t), w);
+  }
+}
+
+template <int DIM>
+__device__ __forceinline__ int prime_phase_numerator(const PrimeDesc& P, const int* g) {
+  int acc = P.offph;
+#pragma unroll
+  for (int r = 0; r < DIM; ++r) acc += P.ph32[r] * g[r];
+  return P.divq.mod(acc);
+}
+
+// One fibre of a small prime PR in registers, for nb signals: slots, weights and
+// band phases once, then 2 PR accesses and about 12 PR operations a signal.
+// dstr: distance of consecutive bands; band 0 may lie elsewhere (d0).
+template <typename C, int MODE, int PR, int DIM, bool COH = false>
+__device__ __forceinline__ void prime_fibre_small(const PrimeDesc& P, int gs, int nb, const C* __restrict__ cin,
+                                                  C* __restrict__ cout, const C* __restrict__ din0,
+                                                  const C* __restrict__ dinw, C* __restrict__ dout0,
+                                                  C* __restrict__ doutw, long long dstr) {
+  using Rl = decltype(C::x);
+  int g[4] = {0, 0, 0, 0};
+  prime_fibre<DIM>(P, gs, g);
+  Rl u[PR];
+#pragma unroll
+  for (int t = 0; t < PR; ++t) u[t] = Rl(0);
+  prime_weights_small<Rl, DIM>(P, g, [&](int tt, Rl w) {
+#pragma unroll
+    for (int t = 0; t < PR; ++t) u[t] += t == tt ? w : Rl(0);
+  });
+#pragma unroll
+  for (int t = 0; t < PR; ++t) u[t] = u[t] == Rl(0) || u[t] == Rl(1) ? u[t] : sqrt(u[t]);
+  const Rl coef = Rl(2) / (Rl(2) + Rl(2) * u[0]);  // 2 / (V^T V), V = u + e_0
+  const int num = prime_phase_numerator<DIM>(P, g);
+  C e[PR];
+  int slot[PR];
+  BoxWalk<DIM> walk(P.HM, g, P.shift, P.mM);
+  int tn = 0;
+#pragma unroll
+  for (int t = 0; t < PR; ++t) {
+    slot[t] = walk.slot;
+    walk.step();
+    e[t] = t == 0 ? cmake<C>(1, 0) : prime_phase<C>(tn, P.q);
+    tn += num;
+    if (tn >= int(P.divq.d)) tn -= int(P.divq.d);
+  }
+#pragma unroll 1
+  for (int b = 0; b < nb; ++b) {
+    const long long om = (long long)b * P.mM, on = (long long)b * P.mN;
+    C x[PR];
+#pragma unroll
+    for (int t = 0; t < PR; ++t) {
+      if (MODE == 0)
+        x[t] = load_c<COH>(cin + om + slot[t]);
+      else
+        x[t] = (t == 0 ? din0 : dinw + (long long)(t - 1) * dstr)[on];
+    }
+    if (MODE == 1) {
+#pragma unroll
+      for (int t = 1; t < PR; ++t) x[t] = cmul(x[t], e[t]);
+    }
+    C sig = x[0];  // V . x: the e_0 part, then the weighted members
+#pragma unroll
+    for (int t = 0; t < PR; ++t)
+      if (u[t] != Rl(0)) sig = cadd(sig, cscale(x[t], u[t]));
+    sig = cscale(sig, coef);
+#pragma unroll
+    for (int t = 0; t < PR; ++t) {
+      const C y = csub(cscale(sig, u[t] + Rl(t == 0)), x[t]);
+      if (MODE == 0)
+        (t == 0 ? dout0 : doutw + (long long)(t - 1) * dstr)[on] = t == 0 ? y : cmul(cconj(e[t]), y);
+      else
+        cout[om + slot[t]] = y;
+    }
+  }
+}
+
+// One chunk of bands of one fibre and signal for larger primes.
+template <typename C, int MODE, int DIM, bool COH = false>
+__device__ __forceinline__ void prime_chunk_small(const PrimeDesc& P, int gs, int j0, const C* __restrict__ cin,
+                                                  C* __restrict__ cout, const C* __restrict__ din0,
+                                                  const C* __restrict__ dinw, C* __restrict__ dout0,
+                                                  C* __restrict__ doutw, long long dstr) {
+  using Rl = decltype(C::x);
+  int g[4] = {0, 0, 0, 0};
+  prime_fibre<DIM>(P, gs, g);
+  constexpr int NW = 1 << DIM;
+  int tm[NW];
+  Rl um[NW];
+  int nw = 0;
+  prime_weights_small<Rl, DIM>(P, g, [&](int t, Rl w) {
+    int i = 0;
+    while (i < nw && tm[i] != t) ++i;
+    if (i == nw) {
+      tm[nw] = t;
+      um[nw++] = Rl(0);
+    }
+    um[i] += w;
+  });
+  Rl u0 = Rl(0);
+  for (int i = 0; i < nw; ++i) {
+    um[i] = sqrt(um[i]);
+    if (tm[i] == 0) u0 = um[i];
+  }
+  const Rl coef = Rl(2) / (Rl(2) + Rl(2) * u0);
+  const int num = prime_phase_numerator<DIM>(P, g), q = int(P.divq.d);
+  C sig = MODE == 0 ? load_c<COH>(cin + prime_slot(P.HM, g)) : din0[0];
+  for (int i = 0; i < nw; ++i) {
+    C xt;
+    if (MODE == 0) {
+      int y[4];
+      prime_member(P.HM, g, P.shift, tm[i], y);
+      xt = load_c<COH>(cin + prime_slot(P.HM, y));
+    } else {
+      xt = cmul(tm[i] == 0 ? din0[0] : dinw[(long long)(tm[i] - 1) * dstr],
+                prime_phase<C>((long long)tm[i] * num % q, P.q));
+    }
+    sig = cadd(sig, cscale(xt, um[i]));
+  }
+  sig = cscale(sig, coef);
+  const int j1 = min(j0 + kPrimeChunk, P.p);
+  int y[4] = {g[0], g[1], g[2], g[3]};
+  int tn = 0;
+  if (j0) {
+    prime_member(P.HM, g, P.shift, j0, y);
+    tn = int((long long)j0 * num % q);
+  }
+  BoxWalk<DIM> walk(P.HM, y, P.shift, P.mM);
+  for (int j = j0; j < j1; ++j) {
+    Rl vj = Rl(j == 0);
+    for (int i = 0; i < nw; ++i)
+      if (tm[i] == j) vj += um[i];
+    const C e = prime_phase<C>(tn, P.q);
+    if (MODE == 0) {
+      const C xj = csub(cscale(sig, vj), load_c<COH>(cin + walk.slot));
+      (j == 0 ? dout0 : doutw + (long long)(j - 1) * dstr)[0] = cmul(cconj(e), xj);
+    } else {
+      cout[walk.slot] = csub(cscale(sig, vj), cmul((j == 0 ? din0 : dinw + (long long)(j - 1) * dstr)[0], e));
+    }
+    walk.step();
+    tn += num;
+    if (tn >= q) tn -= q;
+  }
+}
+
+// One work item of one signal (the batch launches): the fibre when p is small,
+// else a chunk of its bands.
+template <typename C, int MODE, bool COH = false>
+__device__ __forceinline__ void prime_item(const PrimeDesc& P, int gs, int j0, const C* __restrict__ cin,
+                                           C* __restrict__ cout, const C* __restrict__ din0,
+                                           const C* __restrict__ dinw, C* __restrict__ dout0,
+                                           C* __restrict__ doutw, long long dstr) {
+  if (!P.small) {
+    prime_split_item<C, MODE, COH>(P, gs, j0, cin, cout, din0, dinw, dout0, doutw, dstr);
+  } else if (P.d == 3) {
+    if (P.p == 3)
+      prime_fibre_small<C, MODE, 3, 3, COH>(P, gs, 1, cin, cout, din0, dinw, dout0, doutw, dstr);
+    else if (P.p == 5)
+      prime_fibre_small<C, MODE, 5, 3, COH>(P, gs, 1, cin, cout, din0, dinw, dout0, doutw, dstr);
+    else
+      prime_chunk_small<C, MODE, 3, COH>(P, gs, j0, cin, cout, din0, dinw, dout0, doutw, dstr);
+  } else if (P.d == 2) {
+    if (P.p == 3)
+      prime_fibre_small<C, MODE, 3, 2, COH>(P, gs, 1, cin, cout, din0, dinw, dout0, doutw, dstr);
+    else if (P.p == 5)
+      prime_fibre_small<C, MODE, 5, 2, COH>(P, gs, 1, cin, cout, din0, dinw, dout0, doutw, dstr);
+    else
+      prime_chunk_small<C, MODE, 2, COH>(P, gs, j0, cin, cout, din0, dinw, dout0, doutw, dstr);
+  } else {
+    prime_chunk_small<C, MODE, 1, COH>(P, gs, j0, cin, cout, din0, dinw, dout0, doutw, dstr);
   }
 }
 

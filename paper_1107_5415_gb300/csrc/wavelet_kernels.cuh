@@ -58,7 +58,10 @@ struct LevelDesc {
 };
 
 // Periodised weight w(N^{-T} h) of the point h (see the header comment);
-// the fibre partner has weight 1 - w.
+// the fibre partner has weight 1 - w.  U_j(t) = sum_n B(t + n) (-1)^(v_j n): B is
+// a partition of unity, so U_j = 1 where v_j is even and only the odd
+// coordinates are evaluated; for the Dirichlet symbol U_j is 1 near the integers
+// of even n, -1 near those of odd n and 0 half way between.
 template <typename Rl, bool SMALL>
 __device__ __forceinline__ Rl fibre_weight(const LevelDesc& L, const int* h) {
   using I = typename std::conditional<SMALL, int, long long>::type;
@@ -68,6 +71,7 @@ __device__ __forceinline__ Rl fibre_weight(const LevelDesc& L, const int* h) {
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     if (j >= d) break;
+    if (!(L.vpar[j] & 1)) continue;
     I t;  // numerator of (N^{-T} h)_j mod 2, in [0, 2q)
     if constexpr (SMALL) {
       int acc = L.off2q;
@@ -83,24 +87,33 @@ __device__ __forceinline__ Rl fibre_weight(const LevelDesc& L, const int* h) {
       t = acc % (2 * q);
       if (t < 0) t += 2 * q;
     }
-    Rl U = Rl(0);
+    if (L.symbol == PWT_DIRICHLET) {
+      const I x = t < q ? t : 2 * q - t;  // distance from the nearest even integer, times q
+      prod *= 2 * x == q ? Rl(0) : 2 * x < q ? Rl(1) : Rl(-1);
+    } else {
+      const Rl eta = Rl(L.eta);
+      Rl U = Rl(0);
 #pragma unroll
-    for (int n = 0; n >= -2; --n) {  // shifts with |t/q + n| possibly < 1
-      const I sn = t + I(n) * q;
-      const I an = sn < 0 ? -sn : sn;
-      Rl b;
-      if (L.symbol == PWT_DIRICHLET) {
-        b = (2 * an < q) ? Rl(1) : (2 * an == q) ? Rl(0.5) : Rl(0);
-      } else {
-        const Rl eta = Rl(L.eta);
-        b = (Rl(0.5) * (Rl(1) + eta) - Rl(an) / Rl(q)) / eta;
+      for (int n = 0; n >= -2; --n) {  // shifts with |t/q + n| possibly < 1
+        const I sn = t + I(n) * q;
+        const I an = sn < 0 ? -sn : sn;
+        Rl b = (Rl(0.5) * (Rl(1) + eta) - Rl(an) / Rl(q)) / eta;
         b = b < Rl(0) ? Rl(0) : (b > Rl(1) ? Rl(1) : b);
+        U += (n & 1) ? -b : b;
       }
-      U += ((L.vpar[j] & n) & 1) ? -b : b;
+      prod *= U;
     }
-    prod *= U;
   }
   return Rl(0.5) * (Rl(1) + prod);
+}
+
+// Scaling symbol of a fibre member of weight w: sqrt(2 w) (Dirichlet, w one of
+// 0, 1/2 and 1) or sqrt(2) w.
+template <typename Rl>
+__device__ __forceinline__ Rl fibre_scaling(const LevelDesc& L, Rl w) {
+  const Rl r = Rl(1.41421356237309504880);
+  if (L.symbol == PWT_DIRICHLET) return w == Rl(0) ? Rl(0) : w == Rl(1) ? r : Rl(1);
+  return r * w;
 }
 
 template <typename C, bool TAB = true, bool SMALL = false>
@@ -138,6 +151,24 @@ __device__ __forceinline__ C wavelet_phase(const LevelDesc& L, const int* h) {
   return cmul(hi[t >> kLoBits], lo[t & ((1 << kLoBits) - 1)]);
 }
 
+// Box point g of slot gs of the box of H(N^T) and the slots of its fibre
+// {g, g + N^T l1} in the box of H(M^T).
+template <int DIM>
+__device__ __forceinline__ void fibre_slots(const LevelDesc& L, int gs, int* g, int& slot0, int& slot1) {
+  int s = gs;
+#pragma unroll
+  for (int r = DIM - 1; r > 0; --r) {
+    const int qd = L.divHN[r].div(s);
+    g[r] = s - qd * L.HNext[r];
+    s = qd;
+  }
+  g[0] = s;
+  slot0 = 0;
+#pragma unroll
+  for (int r = 0; r < DIM; ++r) slot0 += g[r] * L.HM.stride[r];
+  slot1 = box_sum_slot_t<DIM>(L.HM, g, L.shift1);
+}
+
 // mode 0: decompose c -> (d1, d2); 1: reconstruct; 2: adjoint, for the
 // fibre of slot gs of the box of H(N^T) in each of `batch` signals (signal b
 // at c + b mM, d + b mN).  The symbols depend on the fibre only: they are
@@ -148,26 +179,14 @@ __device__ __forceinline__ void split_fibre(const LevelDesc& L, int gs, int batc
                                             const C* __restrict__ d2in, C* __restrict__ d1out,
                                             C* __restrict__ d2out) {
   using Rl = decltype(C::x);
-  int g[4] = {0, 0, 0, 0}, h1[4] = {0, 0, 0, 0};
-  int s = gs;
-  for (int r = L.d - 1; r >= 0; --r) {
-    const int qd = L.divHN[r].div(s);
-    g[r] = s - qd * L.HNext[r];
-    s = qd;
+  int g[4] = {0, 0, 0, 0};
+  int slot0, slot1;
+  switch (L.d) {
+    case 1: fibre_slots<1>(L, gs, g, slot0, slot1); break;
+    case 2: fibre_slots<2>(L, gs, g, slot0, slot1); break;
+    case 3: fibre_slots<3>(L, gs, g, slot0, slot1); break;
+    default: fibre_slots<4>(L, gs, g, slot0, slot1);
   }
-  int slot0 = 0;
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    if (r < L.d) {
-      h1[r] = g[r] + L.shift1[r];
-      slot0 += g[r] * L.HM.stride[r];
-    }
-  }
-  box_fix(L.HM, h1);
-  int slot1 = 0;
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-    if (r < L.d) slot1 += h1[r] * L.HM.stride[r];
   if (L.snf_D) {  // coefficients on G(M^T) in Smith-coordinate order
     slot0 = slot1 = 0;
 #pragma unroll
@@ -199,13 +218,8 @@ __device__ __forceinline__ void split_fibre(const LevelDesc& L, int gs, int batc
   if (!tabulated) {
     const Rl w0 = fibre_weight<Rl, SMALL>(L, g);
     const Rl w1 = Rl(1) - w0;
-    if (L.symbol == PWT_DIRICHLET) {
-      A0 = sqrt(Rl(2) * w0);
-      A1 = sqrt(Rl(2) * w1);
-    } else {
-      A0 = Rl(1.41421356237309504880) * w0;
-      A1 = Rl(1.41421356237309504880) * w1;
-    }
+    A0 = fibre_scaling(L, w0);
+    A1 = fibre_scaling(L, w1);
     e0 = wavelet_phase<C, TAB, SMALL>(L, g);
   }
   // B(h0) = A(h1) e(h0), B(h1) = A(h0) e(h1), e(h1) = -e(h0)
@@ -258,13 +272,8 @@ __device__ __forceinline__ void fibre_symbols(const LevelDesc& L, const int* g, 
                                               decltype(C::x)& a1, C& ph) {
   using Rl = decltype(C::x);
   const Rl w = fibre_weight<Rl, true>(L, g);
-  if (L.symbol == PWT_DIRICHLET) {
-    a0 = sqrt(Rl(2) * w);
-    a1 = sqrt(Rl(2) * (Rl(1) - w));
-  } else {
-    a0 = Rl(1.41421356237309504880) * w;
-    a1 = Rl(1.41421356237309504880) * (Rl(1) - w);
-  }
+  a0 = fibre_scaling(L, w);
+  a1 = fibre_scaling(L, Rl(1) - w);
   ph = cconj(wavelet_phase<C, true, true>(L, g));
 }
 
