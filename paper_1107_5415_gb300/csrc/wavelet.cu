@@ -477,11 +477,11 @@ static int fuse_count(const pwt_plan_s* P, int l) {
   return F < 2 ? 1 : F;
 }
 
-template <int F>
-static int launch_fused_t(pwt_plan_s* P, int l, const void* cin, void* sout, void* const* wavelets,
+template <int F, int MODE>
+static int launch_fused_t(pwt_plan_s* P, int l, const void* coef, const void* scal, const void* const* wavelets,
                           cudaStream_t s) {
-  constexpr int smem = fused_smem_bytes<float2, F>();
-  static const bool ok = cudaFuncSetAttribute(reinterpret_cast<const void*>(fused_split_kernel<float2, F>),
+  constexpr int smem = fused_smem_bytes<float2, F, MODE>();
+  static const bool ok = cudaFuncSetAttribute(reinterpret_cast<const void*>(fused_split_kernel<float2, F, MODE>),
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
   if (!ok) return -1;
   // fibres of the last level over CTAs of kFuseThreads threads, about
@@ -494,19 +494,26 @@ static int launch_fused_t(pwt_plan_s* P, int l, const void* cin, void* sout, voi
   if (y > P->batch) y = P->batch;
   const int chunk = int((P->batch + y - 1) / y);
   const unsigned gy = unsigned((P->batch + chunk - 1) / chunk);
+  auto p = [](const void* q) { return static_cast<float2*>(const_cast<void*>(q)); };
   float2* w[3] = {nullptr, nullptr, nullptr};
-  for (int k = 0; k < F; ++k) w[k] = static_cast<float2*>(wavelets[l + k]);
-  fused_split_kernel<float2, F><<<dim3(unsigned(x), gy), kFuseThreads, smem, s>>>(
-      P->dlv + l, int(P->batch), chunk, static_cast<const float2*>(cin), static_cast<float2*>(sout), w[0], w[1],
-      w[2]);
+  for (int k = 0; k < F; ++k) w[k] = p(wavelets[l + k]);
+  fused_split_kernel<float2, F, MODE><<<dim3(unsigned(x), gy), kFuseThreads, smem, s>>>(
+      P->dlv + l, int(P->batch), chunk, p(coef), p(scal), w[0], w[1], w[2]);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-static int launch_fused(pwt_plan_s* P, int l, int F, const void* cin, void* sout, void* const* wavelets,
-                        cudaStream_t s) {
+// Levels l .. l + F - 1: analysis (mode 0: coef -> scal, wavelets), reconstruct (1)
+// or adjoint (2): scal, wavelets -> coef.
+static int launch_fused(pwt_plan_s* P, int l, int F, int mode, const void* coef, const void* scal,
+                        const void* const* wavelets, cudaStream_t s) {
   P->prof.begin(0, s);
-  const int rc = F == 3 ? launch_fused_t<3>(P, l, cin, sout, wavelets, s)
-                        : launch_fused_t<2>(P, l, cin, sout, wavelets, s);
+  int rc;
+  if (mode == 0)
+    rc = F == 3 ? launch_fused_t<3, 0>(P, l, coef, scal, wavelets, s) : launch_fused_t<2, 0>(P, l, coef, scal, wavelets, s);
+  else if (mode == 1)
+    rc = F == 3 ? launch_fused_t<3, 1>(P, l, coef, scal, wavelets, s) : launch_fused_t<2, 1>(P, l, coef, scal, wavelets, s);
+  else
+    rc = F == 3 ? launch_fused_t<3, 2>(P, l, coef, scal, wavelets, s) : launch_fused_t<2, 2>(P, l, coef, scal, wavelets, s);
   P->prof.end(0, s);
   return rc;
 }
@@ -522,7 +529,7 @@ extern "C" pfft_status pwt_decompose(pwt_plan p, const void* c_hat, void* scalin
   for (int l = 0; l < p->levels; ++g) {
     const int F = fuse_count(p, l);
     void* d1 = (l + F == p->levels) ? scaling : p->ws[g & 1];
-    const int rc = F > 1 ? launch_fused(p, l, F, cur, d1, wavelets, s)
+    const int rc = F > 1 ? launch_fused(p, l, F, 0, cur, d1, wavelets, s)
                          : run_level(p, l, 0, cur, nullptr, nullptr, nullptr, d1, wavelets[l], s);
     if (rc != 0) return PFFT_ERR_CUDA;
     cur = d1;
@@ -537,10 +544,19 @@ static pfft_status synthesise(pwt_plan p, const void* scaling, const void* const
   for (int l = 0; l < p->levels; ++l)
     if (!wavelets[l]) return PFFT_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
+  // the launches of the analysis in reverse
+  int first[64], count[64], n = 0;
+  for (int l = 0; l < p->levels; l += count[n++]) {
+    first[n] = l;
+    count[n] = fuse_count(p, l);
+  }
   const void* cur = scaling;
-  for (int l = p->levels - 1; l >= 0; --l) {
-    void* dst = (l == 0) ? c_hat : p->ws[l & 1];
-    if (run_level(p, l, mode, nullptr, dst, cur, wavelets[l], nullptr, nullptr, s) != 0) return PFFT_ERR_CUDA;
+  for (int g = n - 1; g >= 0; --g) {
+    void* dst = g == 0 ? c_hat : p->ws[g & 1];
+    const int l = first[g], F = count[g];
+    const int rc = F > 1 ? launch_fused(p, l, F, mode, dst, cur, wavelets, s)
+                         : run_level(p, l, mode, nullptr, dst, cur, wavelets[l], nullptr, nullptr, s);
+    if (rc != 0) return PFFT_ERR_CUDA;
     cur = dst;
   }
   return PFFT_OK;

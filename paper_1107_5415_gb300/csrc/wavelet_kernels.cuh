@@ -297,49 +297,59 @@ __global__ void __launch_bounds__(256) symbol_table_kernel(LevelDesc L, float4* 
 }
 
 // ---- Several levels in one launch (the repetition of steps 2-4 at the end
-// of Section 5.3).  After F levels, a fibre g of G(N_F^T) (the last level's
-// output) draws on 2^F coefficients of the first level's input: its two
-// members are fibres of level F - 1, theirs of level F - 2, and so on.  One
-// thread takes g, reads those 2^F inputs once per signal, runs the 2^F - 1
-// butterflies of the tree level by level and writes every wavelet part once
-// and the last scaling part; the scaling parts of the inner levels never
-// leave registers.  The symbols depend on the fibres only: each thread
-// takes them once per g (top-down, so that only the box points of the
-// current level are live) from the plan's per-fibre symbol table (or
-// evaluates them) into its column of shared-memory tables and applies them
-// to every signal of its chunk, two signals at a time so that the loads of
-// both are in flight together.
+// of Section 5.3), analysis and synthesis.  After F levels, a fibre g of
+// G(N_F^T) (the last level's output) draws on 2^F coefficients of the first
+// level's input: its two members are fibres of level F - 1, theirs of level F - 2,
+// and so on.  One thread takes g and, per signal, reads its 2^F values once
+// (analysis: the coefficients; synthesis: the scaling part and the wavelet parts
+// of the tree), runs the 2^F - 1 butterflies of the tree level by level and writes
+// 2^F values once; the scaling parts of the inner levels never leave registers.
+// The symbols depend on the fibres only: each thread takes them once per g
+// (top-down, so that only the box points of the current level are live) from the
+// plan's per-fibre symbol table (or evaluates them) into its column of
+// shared-memory tables and applies them to every signal of its chunk, two
+// signals at a time so that the loads of both are in flight together.
+// Twelve levels of 2^21 x 16 coefficients: analysis 0.146 ms in four launches;
+// synthesis 0.216 ms in twelve one-level launches (28 bytes of traffic a
+// coefficient against 18), 0.163 ms in four.
 constexpr int kFuseThreads = 128;
 constexpr int kFuseMax = 3;   // levels per launch (4 needs more registers than pays off)
 constexpr int kFuseWaves = 8; // resident waves of CTAs for the fibres
 
-// Dynamic shared memory of fused_split_kernel<C, F>: per thread and fibre of
-// the tree (2^F - 1) the symbols (A(h0), A(h1), conjugate phase) and the
-// output slot, per member of the first level (2^F) the input slot.
-template <typename C, int F>
+// Values kept per fibre of the tree: the symbols A(h0), A(h1) and the conjugate
+// phase; the synthesis adds its scale (1 / sqrt 2, or sqrt 2 / (A(h0)^2 + A(h1)^2)).
+template <int MODE>
+constexpr int kFuseSym = MODE == 0 ? 4 : 5;
+
+// Dynamic shared memory of fused_split_kernel<C, F, MODE>: per thread and fibre of
+// the tree (2^F - 1) the symbols and the slot of its wavelet part, per member of
+// the first level (2^F) the coefficient's slot.
+template <typename C, int F, int MODE>
 __host__ __device__ constexpr int fused_smem_bytes() {
-  return kFuseThreads * (((1 << F) - 1) * (4 * int(sizeof(decltype(C::x))) + 4) + (1 << F) * 4);
+  return kFuseThreads * (((1 << F) - 1) * (kFuseSym<MODE> * int(sizeof(decltype(C::x))) + 4) + (1 << F) * 4);
 }
 
-// F levels of the analysis (mode 0) starting at the level whose descriptor is
-// lvg[0]: inputs cin (the first level's coefficients), wavelet parts of level
-// k at w_k, the last scaling part at sout; signals [y chunk, (y + 1) chunk).
-// Every level of the group has the int32 index path (`small`).
-template <typename C, int F>
+// F levels starting at the level whose descriptor is lvg[0]: the first level's
+// coefficients at coef, the wavelet parts of level k at w_k, the last scaling part
+// at scal; signals [y chunk, (y + 1) chunk).  MODE 0 reads coef and writes the
+// parts; 1 (reconstruct) and 2 (adjoint) read the parts and write coef.  Every
+// level of the group has the int32 index path (`small`).
+template <typename C, int F, int MODE>
 __global__ void __launch_bounds__(kFuseThreads, 4)
-    fused_split_kernel(const LevelDesc* __restrict__ lvg, int batch, int chunk, const C* __restrict__ cin,
-                       C* __restrict__ sout, C* __restrict__ w0, C* __restrict__ w1, C* __restrict__ w2) {
+    fused_split_kernel(const LevelDesc* __restrict__ lvg, int batch, int chunk, C* __restrict__ coef,
+                       C* __restrict__ scal, C* __restrict__ w0, C* __restrict__ w1, C* __restrict__ w2) {
   using Rl = decltype(C::x);
   constexpr int NT = kFuseThreads;
   constexpr int NL = 1 << (F - 1);   // fibres of the first level per thread
   constexpr int FIB = (1 << F) - 1;  // fibres of the tree
   constexpr int SG = 2;              // signals per iteration
+  constexpr int NS = kFuseSym<MODE>;
   __shared__ LevelDesc lv[F];
   extern __shared__ __align__(16) unsigned char fsm[];
-  // per-thread tables, thread index fastest: symbols [FIB][4][NT] (A0, A1,
-  // phase), output slots [FIB][NT], input slots [2^F][NT]
+  // per-thread tables, thread index fastest: symbols [FIB][NS][NT] (A0, A1, phase,
+  // scale), slots of the wavelet parts [FIB][NT], coefficient slots [2^F][NT]
   Rl* sym = reinterpret_cast<Rl*>(fsm);
-  int* osl = reinterpret_cast<int*>(fsm + size_t(FIB) * NT * 4 * sizeof(Rl));
+  int* osl = reinterpret_cast<int*>(fsm + size_t(FIB) * NT * NS * sizeof(Rl));
   int* isl = osl + FIB * NT;
   static_assert(sizeof(LevelDesc) % 4 == 0, "level descriptors are copied as 32-bit words");
   for (int i = threadIdx.x; i < int(F * sizeof(LevelDesc) / 4); i += blockDim.x)
@@ -349,8 +359,9 @@ __global__ void __launch_bounds__(kFuseThreads, 4)
   const int nb = min(chunk, batch - b0);
   if (nb <= 0) return;
   const LevelDesc& Lt = lv[F - 1];
-  C* const wout[3] = {w0, w1, w2};
+  C* const wpart[3] = {w0, w1, w2};
   const int tid = threadIdx.x;
+  const Rl r2 = Rl(0.70710678118654752440);
   // fibre i of level k has the flat index 2^(F-1-k) - 1 + i in the tables
   for (int gs = blockIdx.x * NT + tid; gs < Lt.mN; gs += gridDim.x * NT) {
     int cur[NL][4];
@@ -394,13 +405,14 @@ __global__ void __launch_bounds__(kFuseThreads, 4)
         } else {
           fibre_symbols<C>(L, cur[i], a0, a1, ph);
         }
-        sym[(4 * f + 0) * NT + tid] = a0;
-        sym[(4 * f + 1) * NT + tid] = a1;
-        sym[(4 * f + 2) * NT + tid] = ph.x;
-        sym[(4 * f + 3) * NT + tid] = ph.y;
+        sym[(NS * f + 0) * NT + tid] = a0;
+        sym[(NS * f + 1) * NT + tid] = a1;
+        sym[(NS * f + 2) * NT + tid] = ph.x;
+        sym[(NS * f + 3) * NT + tid] = ph.y;
+        if constexpr (MODE == 1) sym[(NS * f + 4) * NT + tid] = Rl(1.41421356237309504880) / (a0 * a0 + a1 * a1);
       }
       // the members of this level's fibres: the fibres of level k - 1 (for
-      // k = 0, the input slots); highest first, so that cur[i] is read
+      // k = 0, the coefficient slots); highest first, so that cur[i] is read
       // before cur[2 i], cur[2 i + 1] overwrite it
 #pragma unroll
       for (int i = (1 << (F - 1 - k)) - 1; i >= 0; --i) {
@@ -427,38 +439,79 @@ __global__ void __launch_bounds__(kFuseThreads, 4)
         }
       }
     }
-    const Rl r2 = Rl(0.70710678118654752440);
     for (int bb = 0; bb < nb; bb += SG) {
       C v[SG][2 * NL];
+      if constexpr (MODE == 0) {
 #pragma unroll
-      for (int j = 0; j < SG; ++j)
-        if (j == 0 || bb + j < nb) {
+        for (int j = 0; j < SG; ++j)
+          if (j == 0 || bb + j < nb) {
 #pragma unroll
-          for (int i = 0; i < 2 * NL; ++i)
-            v[j][i] = cin[(long long)(b0 + bb + j) * lv[0].mM + isl[i * NT + tid]];
+            for (int i = 0; i < 2 * NL; ++i)
+              v[j][i] = coef[(long long)(b0 + bb + j) * lv[0].mM + isl[i * NT + tid]];
+          }
+#pragma unroll
+        for (int k = 0; k < F; ++k) {
+#pragma unroll
+          for (int i = 0; i < (1 << (F - 1 - k)); ++i) {
+            const int f = (1 << (F - 1 - k)) - 1 + i;
+            const Rl a0 = sym[(NS * f + 0) * NT + tid], a1 = sym[(NS * f + 1) * NT + tid];
+            const C ph = cmake<C>(sym[(NS * f + 2) * NT + tid], sym[(NS * f + 3) * NT + tid]);
+            const int os = osl[f * NT + tid];
+#pragma unroll
+            for (int j = 0; j < SG; ++j)
+              if (j == 0 || bb + j < nb) {
+                const C c0 = v[j][2 * i], c1 = v[j][2 * i + 1];
+                const C d1 = cscale(cadd(cscale(c0, a0), cscale(c1, a1)), r2);
+                const C d2 = cscale(cmul(ph, csub(cscale(c0, a1), cscale(c1, a0))), r2);
+                wpart[k][(long long)(b0 + bb + j) * lv[k].mN + os] = d2;
+                v[j][i] = d1;
+              }
+          }
         }
 #pragma unroll
-      for (int k = 0; k < F; ++k) {
+        for (int j = 0; j < SG; ++j)
+          if (j == 0 || bb + j < nb) scal[(long long)(b0 + bb + j) * Lt.mN + gs] = v[j][0];
+      } else {
+        // the wavelet parts of the tree at v[1 ..] by flat fibre index, the scaling part at v[0]
+        C d[SG][FIB];
 #pragma unroll
-        for (int i = 0; i < (1 << (F - 1 - k)); ++i) {
-          const int f = (1 << (F - 1 - k)) - 1 + i;
-          const Rl a0 = sym[(4 * f + 0) * NT + tid], a1 = sym[(4 * f + 1) * NT + tid];
-          const C ph = cmake<C>(sym[(4 * f + 2) * NT + tid], sym[(4 * f + 3) * NT + tid]);
-          const int os = osl[f * NT + tid];
+        for (int j = 0; j < SG; ++j)
+          if (j == 0 || bb + j < nb) {
+            v[j][0] = scal[(long long)(b0 + bb + j) * Lt.mN + gs];
 #pragma unroll
-          for (int j = 0; j < SG; ++j)
-            if (j == 0 || bb + j < nb) {
-              const C c0 = v[j][2 * i], c1 = v[j][2 * i + 1];
-              const C d1 = cscale(cadd(cscale(c0, a0), cscale(c1, a1)), r2);
-              const C d2 = cscale(cmul(ph, csub(cscale(c0, a1), cscale(c1, a0))), r2);
-              wout[k][(long long)(b0 + bb + j) * lv[k].mN + os] = d2;
-              v[j][i] = d1;
-            }
+            for (int k = F - 1; k >= 0; --k)
+#pragma unroll
+              for (int i = 0; i < (1 << (F - 1 - k)); ++i) {
+                const int f = (1 << (F - 1 - k)) - 1 + i;
+                d[j][f] = wpart[k][(long long)(b0 + bb + j) * lv[k].mN + osl[f * NT + tid]];
+              }
+          }
+#pragma unroll
+        for (int k = F - 1; k >= 0; --k) {
+          // highest first: v[i] is read before v[2 i], v[2 i + 1] overwrite it
+#pragma unroll
+          for (int i = (1 << (F - 1 - k)) - 1; i >= 0; --i) {
+            const int f = (1 << (F - 1 - k)) - 1 + i;
+            const Rl a0 = sym[(NS * f + 0) * NT + tid], a1 = sym[(NS * f + 1) * NT + tid];
+            const C e = cmake<C>(sym[(NS * f + 2) * NT + tid], -sym[(NS * f + 3) * NT + tid]);
+            const Rl fac = MODE == 1 ? sym[(NS * f + 4) * NT + tid] : r2;
+#pragma unroll
+            for (int j = 0; j < SG; ++j)
+              if (j == 0 || bb + j < nb) {
+                const C x = v[j][i], eb = cmul(e, d[j][f]);
+                v[j][2 * i] = cscale(cadd(cscale(x, a0), cscale(eb, a1)), fac);
+                v[j][2 * i + 1] = cscale(csub(cscale(x, a1), cscale(eb, a0)), fac);
+              }
+          }
         }
+#pragma unroll
+        for (int j = 0; j < SG; ++j)
+          if (j == 0 || bb + j < nb) {
+#pragma unroll
+            for (int i = 0; i < 2 * NL; ++i)
+              coef[(long long)(b0 + bb + j) * lv[0].mM + isl[i * NT + tid]] = v[j][i];
+          }
       }
-#pragma unroll
-      for (int j = 0; j < SG; ++j)
-        if (j == 0 || bb + j < nb) sout[(long long)(b0 + bb + j) * Lt.mN + gs] = v[j][0];
     }
   }
 }
