@@ -7,12 +7,13 @@
 
 namespace pfft {
 
-template <int DIM, int LOGL, int LOGT>
+template <int DIM, int LOGL, int LOGT, bool AX2 = false>
 static int launch_ct(const PassArgs& a, cudaStream_t s) {
-  static const int ok = configure_kernel(reinterpret_cast<const void*>(col_fast_ct_kernel<float2, DIM, LOGL, LOGT>));
+  static const int ok =
+      configure_kernel(reinterpret_cast<const void*>(col_fast_ct_kernel<float2, DIM, LOGL, LOGT, AX2>));
   if (ok != 0) return -1;
   dim3 grid(a.groups, a.batch), block(ct_threads<LOGL, LOGT>());
-  col_fast_ct_kernel<float2, DIM, LOGL, LOGT><<<grid, block, a.smem_bytes, s>>>(a);
+  col_fast_ct_kernel<float2, DIM, LOGL, LOGT, AX2><<<grid, block, a.smem_bytes, s>>>(a);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -49,6 +50,20 @@ static int launch_cpipe(const PassArgs& a, cudaStream_t s) {
   if (a.d == 2) return fwd ? launch_cpipe_t<2, true>(a, s) : inv ? launch_cpipe_t<2, false>(a, s) : -2;
   if (a.d == 3) return fwd ? launch_cpipe_t<3, true>(a, s) : inv ? launch_cpipe_t<3, false>(a, s) : -2;
   return -2;
+}
+
+// Pencils over two cycles (three cycles in all: d = 3), the first at least 32
+// rows long; returns -2 when no kernel matches.
+int launch_col_ct2_f32(const PassArgs& a, cudaStream_t s) {
+  if (!a.cols || a.d != 3 || a.nsub != 2 || a.sub_n[0] < 32 || a.LB != a.L || a.nthreads != a.T * a.L / 32) return -2;
+  switch (a.L) {
+    case 1 << 9: return a.T == 16 ? launch_ct<3, 9, 4, true>(a, s) : -2;
+    case 1 << 10: return a.T == 8 ? launch_ct<3, 10, 3, true>(a, s) : -2;
+    case 1 << 11: return a.T == 4 ? launch_ct<3, 11, 2, true>(a, s) : -2;
+    case 1 << 12: return a.T == 2 ? launch_ct<3, 12, 1, true>(a, s) : -2;
+    case 1 << 13: return a.T == 1 ? launch_ct<3, 13, 0, true>(a, s) : -2;
+    default: return -2;
+  }
 }
 
 // Launches the specialised column pass when one matches (L, T, d); returns

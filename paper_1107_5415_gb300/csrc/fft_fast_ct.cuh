@@ -126,11 +126,20 @@ __host__ __device__ constexpr int ct_threads() {
   return (1 << (LOGL + LOGT)) / 32;
 }
 
-template <typename C, int DIM, int LOGL, int LOGT>
+// AX2: the pencil holds the rows r = i0 n1 + i1 of two cycles of lengths n0 x n1
+// (powers of two, n0 >= 32, so that the P rows between two walk steps are whole
+// multiples of n1).  The stages are those of one axis of length n0 n1 with the
+// cross-axis twiddles taken out of the plan's stage tables (fft_fast2.cuh), which
+// leaves frequency (f0, f1) at position f0 + n0 f1; the walk advances i0 alone,
+// by P / n1 rows of the first cycle, and its box point still by the point of row
+// P.  (cycles 64 x 32 beside 8192, batch 4: the column pass took 0.775 / 0.795 ms
+// in col_fast2_kernel, two thirds of its instructions index arithmetic; forward and
+// adjoint of M = [[256, 64, 0], [0, 256, 32], [0, 0, 256]] x 4: 2.176 -> 1.614 ms.)
+template <typename C, int DIM, int LOGL, int LOGT, bool AX2 = false>
 __global__ void __launch_bounds__(ct_threads<LOGL, LOGT>(), 512 / ct_threads<LOGL, LOGT>())
     col_fast_ct_kernel(PassArgs a) {
   constexpr int R = 32;
-  constexpr int L = 1 << LOGL, T = 1 << LOGT, P = L / R;
+  constexpr int L = 1 << LOGL, T = 1 << LOGT, P = L / R, LP = LOGL - 5;
   constexpr int TS = DIM <= 2 ? 2 : 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* sm = reinterpret_cast<C*>(smem_raw);
@@ -142,24 +151,38 @@ __global__ void __launch_bounds__(ct_threads<LOGL, LOGT>(), 512 / ct_threads<LOG
   const int p0 = blockIdx.x * T;
   C* smc = sm + tcol;
   const bool walk_in = a.load_mode != MAP_WS, walk_out = a.store_mode != MAP_WS;
-  // the sheared walk of this thread: rows i0 + j P (mod L), box points z_j of i_j g + e
-  int i0 = 0, z[4] = {0, 0, 0, 0}, cP[4] = {0, 0, 0, 0};
+  // two axes: log2 of their lengths; row of the transform's output at position pos
+  const int l0 = AX2 ? 31 - __clz(a.sub_n[0]) : 0, l1 = AX2 ? LOGL - l0 : 0;
+  auto row_of = [&](int pos) { return AX2 ? ((pos & ((1 << l0) - 1)) << l1) | (pos >> l0) : pos; };
+  // the sheared walk of this thread: rows i0 + j P (mod L), or (i0 + j P / n1 mod
+  // n0, i1), with box points z_j
+  int i0 = 0, i1 = 0, z[4] = {0, 0, 0, 0}, cP[4] = {0, 0, 0, 0};
   if (walk_in || walk_out) {
     int et[4], ct[4];
     load_point<TS>(a.Etab, p0 + tcol, et);
-    const int off = int((int64_t(tcol) * a.alpha[0]) % L);
-    i0 = p + off;
-    if (i0 >= L) i0 -= L;
-    load_point<TS>(a.Ctab, i0, ct);
+    const int off = int((int64_t(tcol) * a.alpha[0]) % (AX2 ? a.sub_n[0] : L));
+    if constexpr (AX2) {
+      const int n1 = 1 << l1;
+      i1 = ((p & (n1 - 1)) + tcol * a.alpha[1]) & (n1 - 1);
+      i0 = ((p >> l1) + off) & ((1 << l0) - 1);
+      load_point<TS>(a.Ctab, (i0 << l1) | i1, ct);
+    } else {
+      i0 = p + off;
+      if (i0 >= L) i0 -= L;
+      load_point<TS>(a.Ctab, i0, ct);
+    }
     load_point<TS>(a.Ctab, P, cP);
 #pragma unroll
     for (int r = 0; r < 4; ++r) z[r] = ct[r];
     box_add_t<DIM>(a.boxG, z, et);
   }
-  // shared-memory position of walk row i0 + j P (mod L), column tcol
+  BoxWalk<DIM> walk(a.boxG, z, cP, a.m);
+  // shared-memory position of walk step j, column tcol
   constexpr int WRAP = ct_phys<LOGT>(L);
   auto walk_addr = [&](int j) {
-    if constexpr (P >= 32) {
+    if constexpr (AX2) {
+      return ct_phys<LOGT>((((i0 + (j << LP >> l1)) & ((1 << l0) - 1)) << l1) | i1);
+    } else if constexpr (P >= 32) {
       return ct_phys<LOGT>(i0) + ct_phys<LOGT>(j * P) - (i0 + j * P >= L ? WRAP : 0);
     } else {
       const int i = i0 + j * P;
@@ -181,10 +204,10 @@ __global__ void __launch_bounds__(ct_threads<LOGL, LOGT>(), 512 / ct_threads<LOG
   } else {
 #pragma unroll
     for (int j = 0; j < R; ++j) {
-      C x = __ldg(in + box_slot_t<DIM>(a.boxG, z));
+      C x = __ldg(in + walk.slot);
       if (a.conj_in) x = cconj(x);
       smc[walk_addr(j)] = x;
-      if (j + 1 < R) box_add_t<DIM>(a.boxG, z, cP);
+      walk.step();
     }
     cp_async_wait_all();
     __syncthreads();
@@ -195,23 +218,34 @@ __global__ void __launch_bounds__(ct_threads<LOGL, LOGT>(), 512 / ct_threads<LOG
   }
   fast_pencil_ct<C, LOGL, LOGT>(v, smc, stw, a, p);
   if (!walk_out) {
-    C* dst = out + p0 + tcol + p * a.nD;
-    const int stride = P * a.nD;
+    C* dst = out + p0 + tcol;
+    if constexpr (AX2) {
 #pragma unroll
-    for (int k = 0; k < R; ++k) dst[k * stride] = v[k];
+      for (int k = 0; k < R; ++k) dst[(size_t)row_of(p + k * P) * a.nD] = v[k];
+    } else {
+      const int stride = P * a.nD;
+      dst += p * a.nD;
+#pragma unroll
+      for (int k = 0; k < R; ++k) dst[k * stride] = v[k];
+    }
   } else {
     using Rl = decltype(C::x);
     const Rl sx = Rl(a.scale), sy = a.conj_out ? -sx : sx;
     __syncthreads();  // the last stage's shared-memory reads are done
-    C* wb = smc + ct_phys<LOGT>(p);
+    if constexpr (AX2) {
 #pragma unroll
-    for (int k = 0; k < R; ++k) wb[ct_phys<LOGT>(k * P)] = v[k];
+      for (int k = 0; k < R; ++k) smc[ct_phys<LOGT>(row_of(p + k * P))] = v[k];
+    } else {
+      C* wb = smc + ct_phys<LOGT>(p);
+#pragma unroll
+      for (int k = 0; k < R; ++k) wb[ct_phys<LOGT>(k * P)] = v[k];
+    }
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < R; ++j) {
       const C x = smc[walk_addr(j)];
-      out[box_slot_t<DIM>(a.boxG, z)] = cmake<C>(x.x * sx, x.y * sy);
-      if (j + 1 < R) box_add_t<DIM>(a.boxG, z, cP);
+      out[walk.slot] = cmake<C>(x.x * sx, x.y * sy);
+      walk.step();
     }
   }
 }

@@ -5,7 +5,8 @@
 
 namespace pfft {
 
-int launch_col_ct_f32(const PassArgs& a, cudaStream_t s);  // fft_fast_ct.cu
+int launch_col_ct_f32(const PassArgs& a, cudaStream_t s);   // fft_fast_ct.cu
+int launch_col_ct2_f32(const PassArgs& a, cudaStream_t s);  // two pencil axes
 
 template <int DIM, bool TC>
 static int launch_dim(const PassArgs& a, cudaStream_t s) {
@@ -36,8 +37,11 @@ static int launch_fast2(const PassArgs& a, cudaStream_t s) {
 }
 
 int launch_fast_f32(const PassArgs& a, cudaStream_t s) {
-  if (a.cols && a.nsub == 2)  // two axes without a four-step split: three cycles, d = 3
+  if (a.cols && a.nsub == 2) {  // two axes without a four-step split: three cycles, d = 3
+    const int rc = launch_col_ct2_f32(a, s);
+    if (rc != -2) return rc;
     return a.d == 3 ? launch_fast2<3>(a, s) : -1;
+  }
   if (a.cols && !a.tc) {
     const int rc = launch_col_ct_f32(a, s);
     if (rc != -2) return rc;
