@@ -114,6 +114,11 @@ __device__ __forceinline__ void main_twiddle(C* v, const C* stw) {
   for (int r = 1; r < R; ++r) v[r] = cmul(v[r], f[r]);
 }
 
+// Table entries per span position k of a main stage: w^(2^b), b < 5 (complex64,
+// radix 32), or the 8 factors of fused_dft (complex128, radix 16).
+template <typename C>
+constexpr int kStageFactors = sizeof(C) == 8 ? 5 : 8;
+
 // All stages of one pencil on the thread's registers v[R].  On entry v holds
 // elements p + P k; on exit v holds output frequencies p + P k.
 // TC (complex64, radix 32): the main stages' butterflies on the tensor cores
@@ -143,9 +148,21 @@ __device__ __forceinline__ void fast_pencil_dft(C* v, C* sm, const C* stw, const
       __syncthreads();
     }
     const int k = p & (Ns - 1);
-    constexpr int NB = (R == 32) ? 5 : 4;
-    if (k) main_twiddle<C, R>(v, stw + a.stw_off[s] + k * NB);
-    if constexpr (TC) {
+    constexpr int NB = kStageFactors<C>;
+    if constexpr (sizeof(C) == 16) {
+      if (Ns > 1) {
+        C t[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) t[b] = stw[a.stw_off[s] + k * NB + b];
+        fused_dft<C, R>(v, t);
+      } else {
+        dft_pow2<C, R>(v);
+      }
+    } else {
+      if (k) main_twiddle<C, R>(v, stw + a.stw_off[s] + k * NB);
+    }
+    if constexpr (sizeof(C) == 16) {
+    } else if constexpr (TC) {
       if (in_regs) __syncthreads();  // the tile may hold the input gather's staging
       tc_dft32_regs(v, *tcx, a);
     } else {

@@ -206,8 +206,11 @@ __device__ __forceinline__ void mdft(C* x) {
 // consecutive entries; w^r = w^(r - r mod 4) w^(r mod 4) keeps three low powers
 // and one high one live, and no factor carries more than log2(R) - 1 rounded
 // products.
-template <int R>
-constexpr int kMixPowers = R > 8 ? 4 : R > 4 ? 3 : R > 2 ? 2 : 1;
+// Power-of-two radices of complex128 run as fused_dft on its R / 2 factors.
+template <typename C, int R>
+constexpr bool kMixFused = sizeof(C) == 16 && (R & (R - 1)) == 0;
+template <typename C, int R>
+constexpr int kMixPowers = kMixFused<C, R> ? R / 2 : R > 8 ? 4 : R > 4 ? 3 : R > 2 ? 2 : 1;
 
 template <typename C, int R>
 __device__ __forceinline__ void mix_twiddle(C* v, const C* w) {
@@ -238,7 +241,7 @@ __device__ __forceinline__ void mix_twiddle(C* v, const C* w) {
 template <typename C, int R>
 __device__ __forceinline__ void mix_stage(C* sm, const MixDesc& a, const MixStage& s) {
   constexpr int NB = kMixPoints / R;  // butterflies a thread holds (at least one)
-  constexpr int NP = kMixPowers<R>;
+  constexpr int NP = kMixPowers<C, R>;
   const int total = a.n / R;
   const int istep = s.istep, ostep = s.ostep;
   const C* __restrict__ tab = static_cast<const C*>(a.stw) + s.tw;
@@ -263,8 +266,15 @@ __device__ __forceinline__ void mix_stage(C* sm, const MixDesc& a, const MixStag
       const C* src = sm + x + s.ipad * a.div_pad.div(x);
 #pragma unroll
       for (int r = 0; r < R; ++r) v[q][r] = src[r * istep];
-      if (s.Ns > 1) mix_twiddle<C, R>(v[q], w);
-      mdft<C, R>(v[q]);
+      if constexpr (kMixFused<C, R>) {
+        if (s.Ns > 1)
+          fused_dft<C, R>(v[q], w);
+        else
+          mdft<C, R>(v[q]);
+      } else {
+        if (s.Ns > 1) mix_twiddle<C, R>(v[q], w);
+        mdft<C, R>(v[q]);
+      }
       const int y = base + ((j - k) * R + k) * s.sig;
       ob[q] = y + s.opad * a.div_pad.div(y);
     }

@@ -50,7 +50,7 @@ constexpr int kMixThreadsC64 = 1024, kMixThreadsC128 = 512;
 struct MixStage {
   int R, aR, sig, Ns, blk;
   int istep, ostep, ipad, opad;
-  int tw;       // twiddles of the stage in the stage table: [bit][k], w^(2^bit), w = exp(-2 pi i k / (Ns R))
+  int tw;       // twiddles of the stage in the stage table: [b][k] (MixTableArgs)
   int gen;      // direct stages: offset of g^t mod R (R - 1 ints) in the integer table
   int twstep;   // direct stages: step of the root table per unit of exp(-2 pi i / (Ns R))
   FastDiv div_sig, div_aR, div_Ns, div_nb;  // div_nb: direct stages, butterflies of the tile
@@ -99,9 +99,12 @@ struct MixCall {
   void* out;
 };
 
-// Stage twiddles: entry (s, b, k) = exp(-2 pi i (k 2^b mod Ns R) / (Ns R)).
+// Stage twiddles: entry (s, b, k) = exp(-2 pi i k 2^b / (Ns R)), or, for the
+// stages of fused_dft (fused), factor b of its levels: exp(-2 pi i (k + c Ns) /
+// (Ns 2^l)), b = fused_first(l) + c.
 struct MixTableArgs {
   int n, total;
+  int fused[kMixMaxStages];
   int R[kMixMaxStages], Ns[kMixMaxStages], off[kMixMaxStages + 1];
 };
 

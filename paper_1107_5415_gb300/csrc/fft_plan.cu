@@ -360,10 +360,12 @@ pfft_status mix_stages(pfft_plan_s& P, int kind) {
       for (int e = 0, x = 1; e < s.R - 1; ++e, x = x * r % s.R) g.push_back(x);
     } else if (s.Ns > 1) {
       s.tw = t.total;
+      const bool fused = P.dtype == PFFT_C128 && (s.R & (s.R - 1)) == 0;
       t.R[t.n] = s.R;
       t.Ns[t.n] = s.Ns;
+      t.fused[t.n] = fused;
       t.off[t.n++] = t.total;
-      t.total += s.Ns * (s.R > 8 ? 4 : s.R > 4 ? 3 : s.R > 2 ? 2 : 1);
+      t.total += s.Ns * (fused ? s.R / 2 : s.R > 8 ? 4 : s.R > 4 ? 3 : s.R > 2 ? 2 : 1);
       t.off[t.n] = t.total;
     }
     ax.Ns *= s.R;
@@ -546,11 +548,13 @@ pfft_status configure_pass(PassArgs& p, const pfft_plan_s& P, bool cols, int T) 
       p.fast_nmain = lg / lr;
       p.fast_tail = 1 << (lg - p.fast_nmain * lr);
       p.nthreads = T * L / Rm;
-      // stage twiddle table: for main stage s (span Ns), w^(2^b) for k < Ns, b < log2 R
+      // stage twiddle table: for main stage s (span Ns) and k < Ns, w^(2^b), b < log2 R
+      // (complex64), or the R / 2 factors of fused_dft (complex128)
+      const int per = P.dtype == PFFT_C64 ? lr : Rm / 2;
       int off = 0, Ns = p.fast_tail;
       for (int s = 0; s < p.fast_nmain; ++s) {
         p.stw_off[s] = off;
-        off += Ns * lr;
+        off += Ns * per;
         Ns *= Rm;
       }
       p.stw_n = (off + 1) & ~1;
@@ -1112,7 +1116,12 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
       const int NsR = (two ? Ns / top : Ns) * Rm;
       for (int k = 0; k < Ns; ++k) {
         const int kk = two ? k / top : k;
-        for (int b = 0; b < lr; ++b) idx.push_back(int(((int64_t(kk) << b) % NsR) * (nD / NsR)));
+        if (P.dtype == PFFT_C64)
+          for (int b = 0; b < lr; ++b) idx.push_back(int(((int64_t(kk) << b) % NsR) * (nD / NsR)));
+        else
+          for (int l = 1; l <= lr; ++l)
+            for (int c = 0; c < std::max(1, (1 << l) / 4); ++c)
+              idx.push_back(int((Rm >> l) * (int64_t(kk) + int64_t(c) * Ns) % NsR * (nD / NsR)));
       }
       Ns *= Rm;
     }

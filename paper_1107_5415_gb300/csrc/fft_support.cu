@@ -130,7 +130,13 @@ __global__ void mixed_table_kernel(C* tab, MixTableArgs t) {
     const int Ns = t.Ns[s], q = Ns * t.R[s];
     const int b = (i - t.off[s]) / Ns, k = i - t.off[s] - b * Ns;
     double sn, c;
-    sincospi(2.0 * double((long long)(k) << b) / double(q), &sn, &c);
+    if (t.fused[s]) {
+      int l = 1;
+      while (fused_first(l + 1) <= b) ++l;
+      sincospi(2.0 * double(k + (b - fused_first(l)) * Ns) / double((long long)Ns << l), &sn, &c);
+    } else {
+      sincospi(2.0 * double((long long)(k) << b) / double(q), &sn, &c);
+    }
     tab[i] = cmake<C>(Rl(c), Rl(-sn));
   }
 }
