@@ -117,16 +117,14 @@ void make_buckets(std::vector<Item>& items, int order, std::vector<Bucket>& out,
       std::stable_sort(v.begin(), v.end(), [](const Item& x, const Item& y) { return x.cost > y.cost; });
     Bucket b;
     b.n = int(v.size());
-    int tmax = 1;
     for (auto& it : v) {
       b.nctas += it.a.groups;
       b.threads = std::max(b.threads, it.a.nthreads);
       b.smem = std::max(b.smem, it.a.smem_bytes);
-      tmax = std::max(tmax, it.a.T);
     }
-    // a thread keeps one pencil of a tile that holds them side by side: the
-    // block size must be a multiple of every item's T (powers of two up to 64)
-    if (b.threads % tmax) b.threads = (b.threads + tmax - 1) / tmax * tmax;
+    // a thread keeps one pencil of a tile that holds them side by side: the block
+    // size must be a multiple of T for columns (up to 64) and 4 T for rows (T up to 16)
+    b.threads = (b.threads + 63) / 64 * 64;
     out.push_back(b);
     groups.push_back(std::move(v));
   }

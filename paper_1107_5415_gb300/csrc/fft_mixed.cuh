@@ -18,7 +18,12 @@
 // thread) and now: [[1200, 240], [0, 1080]] x 8: 1.538 -> 0.448 ms (171 thread
 // instructions a point in the row pass, 450 before); [[2048, 8], [0, 2048]] x 8:
 // 1.993 -> 1.027 ms; [[64, 16], [-16, 64]] x 1: 0.089 -> 0.033 ms; a mix of 512
-// patterns: 3.65 -> 2.84 ms.
+// patterns: 3.65 -> 2.84 ms.  With the setups of a thread's loops trimmed (stage
+// tests by group, shears by multiply-high, one row per thread of a split tile):
+// 0.402, 0.964, 0.033 and, with the 32-bit splits, 2.33 ms.  Reading the workspace
+// straight into the first butterflies of a column tile and writing it from the last
+// ones saves instructions in such tiles but costs every other stage (0.415 for
+// the first).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -300,7 +305,8 @@ __device__ __forceinline__ void mix_stage(C* sm, const MixDesc& a, const MixStag
 // A work item takes Q consecutive n of one butterfly: a_m and b_m are read once
 // for its Q outputs and the Q roots slide by one entry per step, so a step is
 // three shared-memory reads for 4 Q multiply-adds (in 2 Q packed instructions);
-// the reads bound it, hence the wide items wherever every item has a thread.
+// the reads bound it, hence the wide items wherever every item has a thread (six
+// pairs: eight spill, 2.36 against 2.33 ms for the mix below).
 template <typename C>
 __device__ __forceinline__ void mix_locate(const MixStage& s, int b, int& base, int& j, int& k) {
   const int t = s.div_sig.div(b), low = b - t * s.sig;
@@ -436,36 +442,45 @@ __device__ __noinline__ void mix_direct(C* sm, const MixDesc& a, const MixStage&
     mix_direct_pairs<C, kMixItems, kMixNarrow>(sm, s, nbf, P, gp);
 }
 
-// The stages come sorted (direct ones first, then in the order below: a first
-// stage of an odd radix of nine or more needs no padding; stages of one axis may
-// run in any order and different axes commute), one loop per radix: a switch
-// inside one loop made the compiler spill every butterfly at its barrier.
+// The stages come sorted (direct ones first, then in the order of kMixOrder: a
+// first stage of an odd radix of nine or more needs no padding; stages of one axis
+// may run in any order and different axes commute), one loop per radix: a switch
+// inside one loop made the compiler spill every butterfly at its barrier.  The
+// radices are tested in groups of their rank, so that a pass of three stages does
+// not make fifteen tests.
 template <typename C, int R>
-__device__ __forceinline__ void mix_stages_of(C* sm, const MixDesc& a, int& i) {
+__device__ __forceinline__ void mix_stages_of(C* sm, const MixDesc& a, int& i, int& R_next) {
 #pragma unroll 1
-  for (; i < a.nstages && a.st[i].R == R; ++i) mix_stage<C, R>(sm, a, a.st[i]);
+  while (R_next == R) {
+    mix_stage<C, R>(sm, a, a.st[i]);
+    ++i;
+    R_next = i < a.nstages ? a.st[i].R : 0;
+  }
+}
+template <typename C, int R0, int R1, int R2, int R3>
+__device__ __forceinline__ void mix_stages_of4(C* sm, const MixDesc& a, int& i, int& R) {
+  if (!((1 << R) & ((1 << R0) | (1 << R1) | (1 << R2) | (1 << R3)))) return;
+  mix_stages_of<C, R0>(sm, a, i, R);
+  mix_stages_of<C, R1>(sm, a, i, R);
+  mix_stages_of<C, R2>(sm, a, i, R);
+  mix_stages_of<C, R3>(sm, a, i, R);
 }
 
 template <typename C>
 __device__ __forceinline__ void mix_stages(C* sm, const MixDesc& a) {
-  int i = 0;
+  int i = 0, R = a.nstages ? a.st[0].R : 0;
 #pragma unroll 1
-  for (; i < a.nstages && a.st[i].R >= kMixMinDirect; ++i) mix_direct<C>(sm, a, a.st[i]);
-  mix_stages_of<C, 15>(sm, a, i);
-  mix_stages_of<C, 13>(sm, a, i);
-  mix_stages_of<C, 11>(sm, a, i);
-  mix_stages_of<C, 9>(sm, a, i);
-  mix_stages_of<C, 16>(sm, a, i);
-  mix_stages_of<C, 14>(sm, a, i);
-  mix_stages_of<C, 12>(sm, a, i);
-  mix_stages_of<C, 10>(sm, a, i);
-  mix_stages_of<C, 8>(sm, a, i);
-  mix_stages_of<C, 7>(sm, a, i);
-  mix_stages_of<C, 6>(sm, a, i);
-  mix_stages_of<C, 5>(sm, a, i);
-  mix_stages_of<C, 4>(sm, a, i);
-  mix_stages_of<C, 3>(sm, a, i);
-  mix_stages_of<C, 2>(sm, a, i);
+  while (R >= kMixMinDirect) {
+    mix_direct<C>(sm, a, a.st[i]);
+    ++i;
+    R = i < a.nstages ? a.st[i].R : 0;
+  }
+  mix_stages_of4<C, 15, 13, 11, 9>(sm, a, i, R);
+  mix_stages_of4<C, 16, 14, 12, 10>(sm, a, i, R);
+  mix_stages_of4<C, 8, 7, 6, 5>(sm, a, i, R);
+  mix_stages_of<C, 4>(sm, a, i, R);
+  mix_stages_of<C, 3>(sm, a, i, R);
+  mix_stages_of<C, 2>(sm, a, i, R);
 }
 
 // ---------------------------------------------------------- loads and stores
@@ -497,12 +512,36 @@ __device__ __forceinline__ C mix_ld(const C* p) {
 __device__ __forceinline__ float2 mix_scale(float2 v, float sx, float sy) { return __fmul2_rn(v, make_float2(sx, sy)); }
 __device__ __forceinline__ double2 mix_scale(double2 v, double sx, double sy) { return make_double2(v.x * sx, v.y * sy); }
 
-// reduce(a + b) of two box points, the point itself.
+// reduce(a + b) of two box points, the point itself (the corrections of
+// box_sum_slot_t).
 template <int DIM>
 __device__ __forceinline__ void box_sum_point(const BoxDesc& B, int* y, const int* a, const int* b) {
 #pragma unroll
-  for (int r = 0; r < 4; ++r) y[r] = r < B.d ? a[r] + b[r] : 0;
-  box_fix(B, y);
+  for (int r = 0; r < 4; ++r) y[r] = r < DIM ? a[r] + b[r] : 0;
+  if constexpr (DIM == 1) {
+    y[0] -= y[0] >= B.H[0][0] ? B.H[0][0] : 0;
+  } else if constexpr (DIM == 2) {
+    const int c1 = y[1] >= B.H[1][1];
+    y[1] -= c1 * B.H[1][1];
+    y[0] -= c1 * B.H[0][1];
+    y[0] += (y[0] < 0) * B.H[0][0];
+    y[0] -= (y[0] >= B.H[0][0]) * B.H[0][0];
+  } else if constexpr (DIM == 3) {
+    const int c2 = y[2] >= B.H[2][2];
+    y[2] -= c2 * B.H[2][2];
+    y[1] -= c2 * B.H[1][2];
+    y[0] -= c2 * B.H[0][2];
+    const int c1 = (y[1] >= B.H[1][1]) - (y[1] < 0);
+    y[1] -= c1 * B.H[1][1];
+    y[0] -= c1 * B.H[0][1];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      y[0] += (y[0] < 0) * B.H[0][0];
+      y[0] -= (y[0] >= B.H[0][0]) * B.H[0][0];
+    }
+  } else {
+    box_fix(B, y);
+  }
 }
 
 // Phase exp(-2 pi i lambda_a mu_b / n) of a split last cycle (fs_twiddle of fft_plan.hpp).
@@ -626,38 +665,22 @@ __device__ __forceinline__ void mix_row_ws(const MixDesc& a, int tile, const C* 
   const int* __restrict__ ps = LOAD ? a.PIinv : a.psout;
   const Rl sy = (LOAD ? a.conj_in : 0) ? Rl(-1) : Rl(1);
   if constexpr (FS) {
-    const int logT = pinned(a.logT), quad = a.T >= 4 ? 2 : 0, mT = a.T - 1;
-    const int la0 = r0 - a.fs_div.div(r0) * a.fs_na, na = a.fs_na;
-    const FastDiv df = a.fs_div;
-    const int n = ((nD + (1 << quad) - 1) >> quad) << (quad + logT);
-    auto split = [&](int w, int& t, int& e) {
-      t = (w >> quad) & mT;
-      e = ((w >> (quad + logT)) << quad) | (w & ((1 << quad) - 1));
-    };
+    // blockDim.x is a multiple of 4 T (mix_configure): a thread keeps its row
+    const int logT = pinned(a.logT), quad = a.T >= 4 ? 2 : 0, sh = quad + logT, mq = (1 << quad) - 1;
+    const int t = (threadIdx.x >> quad) & (a.T - 1);
+    const bool live = t < rows;
+    const int row = r0 + (live ? t : 0);
+    const int la = row - a.fs_div.div(row) * a.fs_na, base = row * nD;
+    const int n = ((nD + mq) >> quad) << sh;
+    const int* __restrict__ mu = a.PIinv;
+    auto elem = [&](int w) { return min(((w >> sh) << quad) | (w & mq), nD - 1); };
     mix_move<C, LOAD, false>(
-        n, in, out, sm,
-        [&](int w) {
-          int t, e;
-          split(w, t, e);
-          return (r0 + min(t, rows - 1)) * nD + min(e, nD - 1);
-        },
-        [&](int w) {
-          int t, e;
-          split(w, t, e);
-          return (__ldg(ps + min(e, nD - 1)) << logT) + t;
-        },
-        [&](int w) {
-          int t, e;
-          split(w, t, e);
-          return t < rows && e < nD;
-        },
+        n, in, out, sm, [&](int w) { return base + elem(w); },
+        [&](int w) { return (__ldg(ps + elem(w)) << logT) + t; },
+        [&](int w) { return live && (((w >> sh) << quad) | (w & mq)) < nD; },
         [&](C v, int w) {
-          int t, e;
-          split(w, t, e);
-          int la = la0 + t;
-          la -= df.div(la) * na;
           if constexpr (LOAD) v = mix_scale(v, Rl(1), sy);
-          return cmul(v, mix_phase<C>(a, la, __ldg(a.PIinv + min(e, nD - 1))));
+          return cmul(v, mix_phase<C>(a, la, __ldg(mu + elem(w))));
         });
   } else {
     const int pitch = LOAD ? nD : a.pitch, base = r0 * nD;
@@ -713,7 +736,7 @@ __device__ __forceinline__ void mix_col_box(const MixDesc& a, int tile, const C*
 #pragma unroll
   for (int s = 0; s < kMaxSub; ++s)
     if (s < nsub) {
-      off[s] = (tcol * a.alpha[s]) % a.sub_n[s];
+      off[s] = a.sub_div[s].mod(tcol * a.alpha[s]);
       row = row * a.sub_n[s] + off[s];
     }
   int f[4], p[4], q[4];

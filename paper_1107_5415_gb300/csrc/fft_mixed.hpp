@@ -28,7 +28,7 @@ constexpr int kMixPoints = 16;  // points a thread holds between the barriers of
 constexpr int kMixMinDirect = 17;
 // Outputs pairs of one work item of a direct stage: kMixWide when every item
 // has a thread of its own, else kMixNarrow with at most kMixItems per thread.
-constexpr int kMixWide = 8, kMixNarrow = 4, kMixItems = 3;
+constexpr int kMixWide = 6, kMixNarrow = 4, kMixItems = 3;
 // Order in which the stages of the register radices run (mix_stages).
 constexpr int kMixOrder[15] = {15, 13, 11, 9, 16, 14, 12, 10, 8, 7, 6, 5, 4, 3, 2};
 template <typename C>

@@ -446,7 +446,9 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
     if (s.R >= kMixMinDirect) rmax = std::max(rmax, s.R);
   }
   a.nthreads = mix_threads(rad, a.n, max_threads);
-  if (tstride > 1 && a.nthreads % T) a.nthreads = (a.nthreads + T - 1) / T * T;  // each thread keeps one column
+  // each thread keeps one column (or, of a [element][row] tile, one row in turns of four elements)
+  const int keep = a.lay ? 4 * T : tstride;
+  if (a.nthreads % keep) a.nthreads = (a.nthreads + keep - 1) / keep * keep;
   if (a.nthreads > max_threads) return PFFT_ERR_UNSUPPORTED;
   a.pad = unit ? tstride : 0;
   a.pitch = a.L;
@@ -785,7 +787,7 @@ std::vector<i64> combo(const std::vector<std::vector<i64>>& gens, const std::vec
 static pfft_status mix_tile(pfft_plan_s& P, int kind, int budget, int ctas) {
   const bool adjacent = kind == MIX_COL || (kind == MIX_ROW && P.fs_na > 1);
   const bool c64 = P.dtype == PFFT_C64;
-  return mix_choose(P, kind, 64, kind == MIX_WHOLE ? (c64 ? 2048 : 1024) : budget, c64 ? 8192 : 4096, adjacent ? 4 : 1,
+  return mix_choose(P, kind, kind == MIX_ROW ? 16 : 64, kind == MIX_WHOLE ? (c64 ? 2048 : 1024) : budget, c64 ? 8192 : 4096, adjacent ? 4 : 1,
                     ctas);
 }
 
