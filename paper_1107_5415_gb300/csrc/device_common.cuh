@@ -93,6 +93,31 @@ struct FastDiv {
   __device__ __forceinline__ int mod(int n) const { return n - div(n) * int(d); }
 };
 
+// Quotient and remainder of 0 <= n < 2^62 by a fixed 1 <= d < 2^31, by one 64-bit
+// multiply-high: mul = floor((2^64 - 1) / d) makes the estimate at most one short.
+struct FastDiv64 {
+  unsigned long long mul;
+  uint32_t d;
+  __host__ void init(uint32_t dv) {
+    d = dv;
+    mul = ~0ull / dv;
+  }
+  __device__ __forceinline__ int divmod(long long n, long long& quot) const {
+    unsigned long long f = __umul64hi((unsigned long long)n, mul);
+    unsigned long long r = (unsigned long long)n - f * d;
+    if (r >= d) {
+      r -= d;
+      ++f;
+    }
+    quot = (long long)f;
+    return int(r);
+  }
+  __device__ __forceinline__ int mod(long long n) const {
+    long long f;
+    return divmod(n, f);
+  }
+};
+
 // ------------------------------------------------------------ Hermite box
 // Upper-triangular H (d <= 4) with row-major slot strides.  A point y of the
 // box x_r [0, H_rr) is stored as int32 coordinates.

@@ -317,7 +317,7 @@ pfft_status pfft::describe_prime_level(int d, const int64_t* Mv, const int64_t* 
     P.phw[i] = sM > 0 ? r : (m - r) % m;
   }
   P.nch = int((p + kPrimeChunk - 1) / kPrimeChunk);
-  // int32 index path
+  // index path by multiply-high divisions
   {
     i128 pbound = 0;
     for (int r = 0; r < d; ++r) {
@@ -326,17 +326,23 @@ pfft_status pfft::describe_prime_level(int d, const int64_t* Mv, const int64_t* 
       P.ph32[r] = int(c);
       pbound += (i128)(c < 0 ? -c : c) * HN(r, r);
     }
-    const i128 lim = (i128)1 << 29;
-    P.small = d <= 3 && p <= kPrimeSmallP && bound < lim && pbound < lim && m < (i64(1) << 29);
+    const i128 lim = (i128)1 << 29, lim64 = (i128)1 << 60;
+    if (d <= 3 && p <= kPrimeSmallP && m < (i64(1) << 29) && bound < lim64 && pbound < lim64 && bound / m < (i64(1) << 28))
+      P.small = bound < lim && pbound < lim ? 1 : 2;
     if (P.small) {
-      for (int k = 0; k < d * d; ++k) P.K32[k] = int(P.K[k]);
       P.divq.init(uint32_t(m));
       P.divp.init(uint32_t(p));
+      P.divq64.init(uint32_t(m));
       P.cq = int(bound / m) + 1;
-      P.offq = int(P.cq * m);
+      P.offq64 = (long long)P.cq * m;
+      P.offph64 = (long long)((pbound / m + 1) * m);
+      if (P.small == 1) {
+        for (int k = 0; k < d * d; ++k) P.K32[k] = int(P.K[k]);
+        P.offq = int(P.offq64);
+        P.offph = int(P.offph64);
+      }
       P.kp = int((P.cq + 2 + p - 1) / p * p);
       for (int r = 0; r < d; ++r) P.v32[r] = int(P.v[r]);
-      P.offph = int((i64(pbound) / m + 1) * m);
     }
   }
   *out = P;

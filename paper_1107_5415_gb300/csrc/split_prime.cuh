@@ -49,8 +49,11 @@ struct alignas(16) PrimeDesc {
   long long v[4];          // n in J^T Z^d <=> v . n = 0 mod p; v . l = 1
   long long phw[4];        // sign(det M) adj(M) (J z) mod q: phase numerator of g is g . phw
   int nch;                 // chunks of kPrimeChunk band outputs per fibre
-  // int32 index path (d <= 3, p <= kPrimeSmallP and every numerator below 2^29)
+  // index path by multiply-high divisions (d <= 3, p <= kPrimeSmallP): small = 1
+  // with every numerator below 2^29 (int32), 2 with numerators below 2^60
   int small;
+  FastDiv64 divq64;
+  long long offq64, offph64;
   int K32[16];
   FastDiv divq, divp;
   int offq, cq;            // offq = cq q >= |K h|
@@ -252,7 +255,7 @@ __device__ __forceinline__ void prime_split_item(const PrimeDesc& P, int gs, int
   }
 }
 
-// ---- int32 index path: the same quantities from FastDiv divisions
+// ---- the same quantities by multiply-high divisions
 template <int DIM>
 __device__ __forceinline__ void prime_fibre(const PrimeDesc& P, int gs, int* g) {
   int s = gs;
@@ -274,11 +277,20 @@ __device__ __forceinline__ void prime_weights_small(const PrimeDesc& P, const in
   int n = 0;
 #pragma unroll
   for (int j = 0; j < DIM; ++j) {
-    int acc = P.offq;
+    int f, r;  // a + k q = r in [0, q) for k = cq - f
+    if (P.small == 1) {
+      int acc = P.offq;
 #pragma unroll
-    for (int i = 0; i < DIM; ++i) acc += P.K32[j * DIM + i] * g[i];
-    const int f = P.divq.div(acc);
-    const int r = acc - f * P.divq.d;  // a + k q = r in [0, q) for k = cq - f
+      for (int i = 0; i < DIM; ++i) acc += P.K32[j * DIM + i] * g[i];
+      f = P.divq.div(acc);
+      r = acc - f * P.divq.d;
+    } else {
+      long long acc = P.offq64, f64;
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) acc += P.K[j * DIM + i] * (long long)g[i];
+      r = P.divq64.divmod(acc, f64);
+      f = int(f64);
+    }
     const int twice = 2 * r, q = int(P.divq.d);
     two[j] = twice == q;               // half way: k - 1 and k with weight 1/2 each
     k0[j] = P.kp + P.cq - f - (twice >= q);
@@ -301,10 +313,16 @@ __device__ __forceinline__ void prime_weights_small(const PrimeDesc& P, const in
 
 template <int DIM>
 __device__ __forceinline__ int prime_phase_numerator(const PrimeDesc& P, const int* g) {
-  int acc = P.offph;
+  if (P.small == 1) {
+    int acc = P.offph;
 #pragma unroll
-  for (int r = 0; r < DIM; ++r) acc += P.ph32[r] * g[r];
-  return P.divq.mod(acc);
+    for (int r = 0; r < DIM; ++r) acc += P.ph32[r] * g[r];
+    return P.divq.mod(acc);
+  }
+  long long acc = P.offph64;
+#pragma unroll
+  for (int r = 0; r < DIM; ++r) acc += (long long)P.ph32[r] * g[r];
+  return P.divq64.mod(acc);
 }
 
 // One fibre of a small prime PR in registers, for nb signals: slots, weights and

@@ -290,6 +290,14 @@ static pfft_status plan_levels(pwt_plan_s& P, const int64_t* Mv, const int64_t* 
         L.divq.init(uint32_t(q));
         L.offq = int(((pbound / q) + 1) * q);
       }
+      const i128 mlim = (i128)1 << 60;
+      L.mid = bound + twoq < mlim && pbound + q < mlim && twoq < ((i128)1 << 31);
+      if (L.mid) {
+        L.mod2q.init(uint32_t(2 * q));
+        L.modq.init(uint32_t(q));
+        L.off2q64 = (long long)((bound / twoq + 1) * twoq);
+        L.offq64 = (long long)((pbound / q + 1) * q);
+      }
       // parity vector: v . n = 0 mod 2 exactly on J^T Z^d (its columns span it)
       bool found = false;
       for (int v = 1; v < (1 << d) && !found; ++v) {

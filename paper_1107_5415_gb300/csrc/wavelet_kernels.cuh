@@ -41,6 +41,11 @@ struct LevelDesc {
   int ph32[4];           // sign(det M) adj(M) (J z) mod q (int32 path)
   FastDiv divq;          // division by q (int32 path)
   int offq;              // multiple of q that makes ph32 . h non-negative
+  // 64-bit path by multiply-high, where the numerators stay below 2^60 (mid): off2q64
+  // and offq64 are multiples of 2q and q that make K h and phw . h non-negative
+  int mid;
+  FastDiv64 mod2q, modq;
+  long long off2q64, offq64;
   const void* tab_lo;    // exp(-2 pi i t / q), t < 2^kLoBits
   const void* tab_hi;    // exp(-2 pi i (t << kLoBits) / q)
   // per-fibre symbols of the fused launches, by slot of G(N^T): float4
@@ -84,8 +89,12 @@ __device__ __forceinline__ Rl fibre_weight(const LevelDesc& L, const int* h) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (i < d) acc += L.K[j * d + i] * (long long)h[i];
-      t = acc % (2 * q);
-      if (t < 0) t += 2 * q;
+      if (L.mid) {
+        t = L.mod2q.mod(acc + L.off2q64);
+      } else {
+        t = acc % (2 * q);
+        if (t < 0) t += 2 * q;
+      }
     }
     if (L.symbol == PWT_DIRICHLET) {
       const I x = t < q ? t : 2 * q - t;  // distance from the nearest even integer, times q
@@ -125,6 +134,12 @@ __device__ __forceinline__ C wavelet_phase(const LevelDesc& L, const int* h) {
     for (int i = 0; i < 4; ++i)
       if (i < L.d) acc += L.ph32[i] * h[i];
     t = L.divq.mod(acc);
+  } else if (L.mid) {
+    long long acc = L.offq64;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i < L.d) acc += (long long)L.ph32[i] * h[i];
+    t = L.modq.mod(acc);
   } else {
 #pragma unroll
     for (int i = 0; i < 4; ++i)  // each product < 2^62; reduce term by term

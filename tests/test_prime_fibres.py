@@ -1,7 +1,7 @@
 """GPU parity of the built-in band system on its int32 index path: the primes
 that a thread holds whole (2, 3, 5, 7) and those split into chunks of bands, d =
 1 .. 3, fibres on the symbol's boundary (even sides), several signals per
-thread, and a matrix whose numerators need the 64-bit path.  Tolerances are those
+thread, and matrices whose numerators need 64 bits.  Tolerances are those
 of the parity bar."""
 import numpy as np
 import pytest
@@ -44,6 +44,23 @@ def test_prime_bands(case, dtype):
     assert rel_l2(parts.transpose(1, 0, 2).reshape(batch, -1), ref.transpose(1, 0, 2).reshape(batch, -1)) <= tol
     back = pf.merge_general(M, J, None, torch.from_numpy(np.ascontiguousarray(ref)).to(dtype).cuda()).cpu().numpy()
     assert rel_l2(back, c) <= tol
+
+
+@pytest.mark.parametrize("dtype", [torch.complex64, torch.complex128], ids=["c64", "c128"])
+@pytest.mark.parametrize("M", [[[32, 16000002], [0, 27]], [[-32, 16000002], [0, 27]]], ids=["pos", "neg"])
+def test_two_band_split_with_large_numerators(M, dtype):
+    """Numerators between 2^29 and 2^60: the 64-bit multiply-high path of the
+    weights and phases, both symbols, split and inverse."""
+    J, batch = [[2, 0], [0, 1]], 3
+    m, tol = abs(L.det(M)), TOL["c64" if dtype == torch.complex64 else "c128"]
+    c = SI.complex_normal(batch, m, 77, dtype=np.complex128)
+    x = torch.from_numpy(c).to(dtype).cuda()
+    plan = pf.WaveletSplit(M, [J], pf.PWT_DIRICHLET, 0.125, batch, dtype)
+    s, w = plan.decompose(x)
+    s_ref, w_ref = oracle.wavelet_cascade(M, [J], c)
+    assert rel_l2(s.cpu().numpy(), s_ref) <= tol and rel_l2(w[0].cpu().numpy(), w_ref[0]) <= tol
+    plan = pf.WaveletSplit(M, [J], pf.PWT_DLVP, 0.125, batch, dtype)
+    assert rel_l2(plan.reconstruct(*plan.decompose(x)).cpu().numpy(), c) <= tol
 
 
 def test_zero_weight_members_stay_apart():
