@@ -63,9 +63,18 @@ def _dtype_code(dtype) -> int:
     raise ValueError("dtype must be torch.complex64 or torch.complex128")
 
 
+# The current stream's handle without building a Stream object (3.0 -> 0.2 us of
+# the 16 us that a call on a small signal takes on the host).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is not None:
+        return int(stream.cuda_stream)
+    if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+        return _raw_stream(_raw_device())
+    return int(torch.cuda.current_stream().cuda_stream)
 
 
 def _check_tensor(x: torch.Tensor, dtype, shape, name: str):
@@ -317,8 +326,19 @@ class PatternBatch:
 
 
 def _det_int(A) -> int:
+    """|det A| of an integer matrix, exact (Laplace expansion along the first row)."""
     A = np.asarray(A, dtype=np.int64)
-    return int(round(abs(np.linalg.det(A.astype(np.float64)))))
+    if A.ndim != 2 or A.shape[0] != A.shape[1]:
+        raise np.linalg.LinAlgError("A must be a square matrix")
+
+    def det(a):
+        if len(a) == 0:
+            return 1
+        if len(a) == 2:
+            return a[0][0] * a[1][1] - a[0][1] * a[1][0]
+        return sum((-1) ** j * a[0][j] * det([r[:j] + r[j + 1:] for r in a[1:]]) for j in range(len(a)) if a[0][j])
+
+    return abs(det(A.tolist()))
 
 
 def split_general(M, J, symbols, c_hat: torch.Tensor, stream=None) -> torch.Tensor:

@@ -103,6 +103,8 @@ def declared_symbols():
 def lib(build: bool = True):
     """Load (building first if needed) the in-tree library."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = build_lib.build() if build else build_lib.LIB
@@ -352,21 +354,30 @@ def pfft_batch_destroy(batch):
 
 
 # ------------------------------------------------------------ general split step
+def _mat_array(M):
+    """(d, int64 array) of a square integer matrix, for the entry points that plan
+    on every call: a plain ctypes array costs a third of a numpy pointer cast."""
+    A = np.asarray(M, dtype=np.int64)
+    if A.ndim != 2 or A.shape[0] != A.shape[1]:
+        raise ValueError("M must be a square integer matrix")
+    return A.shape[0], (ctypes.c_int64 * A.size)(*A.ravel().tolist())
+
+
 def _mj(M, J):
-    d, (a, p) = _mat(M)
-    dj, (b, q) = _mat(J)
+    d, a = _mat_array(M)
+    dj, b = _mat_array(J)
     if dj != d:
         raise ValueError("M and J must have the same size")
-    return d, a, p, b, q
+    return d, a, b
 
 
 def pwt_split_general(M, J, batch: int, dtype: int, symbols_ptr: int, c_hat_ptr: int, parts_ptr: int, stream: int):
-    d, a, p, b, q = _mj(M, J)
-    _check(lib().pwt_split_general(d, p, q, int(batch), int(dtype), symbols_ptr, c_hat_ptr, parts_ptr, stream),
+    d, a, b = _mj(M, J)
+    _check(lib().pwt_split_general(d, a, b, int(batch), int(dtype), symbols_ptr, c_hat_ptr, parts_ptr, stream),
            "pwt_split_general")
 
 
 def pwt_merge_general(M, J, batch: int, dtype: int, symbols_ptr: int, parts_ptr: int, c_hat_ptr: int, stream: int):
-    d, a, p, b, q = _mj(M, J)
-    _check(lib().pwt_merge_general(d, p, q, int(batch), int(dtype), symbols_ptr, parts_ptr, c_hat_ptr, stream),
+    d, a, b = _mj(M, J)
+    _check(lib().pwt_merge_general(d, a, b, int(batch), int(dtype), symbols_ptr, parts_ptr, c_hat_ptr, stream),
            "pwt_merge_general")
