@@ -275,4 +275,172 @@ __global__ void __launch_bounds__(256, 2) col_pipe_kernel(PassArgs a) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// The forward pass for pencils of 2^11 points, four columns per tile: one cycle of 2048
+// rows, or two cycles of 64 x 32 (AX2, rows r = 32 i0 + i1, the stage tables of
+// fft_fast2.cuh).  Thread (c, p), c < 4, p < 64.
+//
+// Stages 2 x 32 x 32.  The radix-2 stage is folded into the reads of the tile:
+// stage 0 of thread p takes the outputs p mod 2 of the butterflies j = floor(p /
+// 2) + 32 r, so it reads rows j and j + 1024 and keeps their sum or difference (64
+// reads where a stage of its own would take 32 reads, 32 writes and 32 reads, and
+// a barrier).  Stage 0 (Ns = 2) writes position (floor(p / 2) << 6) | (r << 1) |
+// (p mod 2), stage 1 (Ns = 64) reads (r' << 6) | p: two rounds, split by bit 5 xor
+// bit 10, so that thread p moves register half h xor bit 5 of p in round h
+// (warp-uniform); dropping bit 10 maps a round one-to-one onto 1024 rows of X.
+//
+// Stage 1 leaves frequency p + 64 r in register r: with two cycles that is row
+// 32 p + r.  The walk of thread (c, p) visits, with two cycles, the rows (u_0 + 2 j
+// mod 64, u_1), u_0 = floor(p / 32) + off_0, u_1 = p + off_1 mod 32 (off_s the
+// column's shears), with one the rows p + off + 64 j mod 2048; either way step j
+// adds the box point of row 64.  Its store goes through X in two rounds of 16
+// steps, slot 64 t + (place of the walker): with two cycles all registers of a
+// holder belong to one step, and the padding of ct_phys keeps the holders of a
+// half warp in different banks.
+//
+// M = [[256, 64, 0], [0, 256, 32], [0, 0, 256]] x 4, forward column pass: 0.541 ms in
+// col_fast_ct_kernel (load, stages and store in turn), 0.423 ms here.  The inverse
+// stays there: gathering the next tile with 8-byte asynchronous copies as
+// col_pipe_kernel does took 0.559 ms against 0.482.
+template <int H>
+__device__ __forceinline__ void cpipe2_x_write(const float2* v, float2* X, int p, int tcol) {
+  float2* wb = X + tcol;
+  const int s0 = (((p >> 1) & 15) << 6) | (p & 1);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) wb[ct_phys<2>(s0 + ((16 * H + i) << 1))] = v[16 * H + i];
+}
+template <int H>
+__device__ __forceinline__ void cpipe2_x_read(float2* v, const float2* X, int p, int tcol) {
+  const float2* rb = X + ct_phys<2>(p) + tcol;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[16 * H + i] = rb[ct_phys<2>(64 * i)];
+}
+
+template <int DIM, bool AX2>
+__global__ void __launch_bounds__(256, 2) col_pipe2_kernel(PassArgs a) {
+  using C = float2;
+  constexpr int R = 32, L = 2048, LOGT = 2, T = 4, P = 64, NT = 256;
+  constexpr int TS = DIM <= 2 ? 2 : 4;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* S = reinterpret_cast<C*>(smem_raw);
+  C* X = S + a.cpipe_x_off;
+  const int tid = threadIdx.x;
+  const int tcol = tid & (T - 1), p = tid >> LOGT;
+  const int ntile = a.nD >> LOGT;
+  const int total = ntile * a.batch;
+  const C* __restrict__ in_all = static_cast<const C*>(a.in);
+  C* __restrict__ out_all = static_cast<C*>(a.out);
+  C* stw = stage_table(S, a);
+
+  const int off0 = AX2 ? (tcol * a.alpha[0]) & 63 : int((int64_t(tcol) * a.alpha[0]) & (L - 1));
+  const int off1 = AX2 ? (tcol * a.alpha[1]) & 31 : 0;
+  // first row of this thread's walk
+  const int start = AX2 ? ((((p >> 5) + off0) & 63) << 5) | ((p + off1) & 31) : (p + off0) & (L - 1);
+
+  // column points of the tiles, copied ahead (double-buffered by the tile count's parity)
+  int* Es = reinterpret_cast<int*>(S + a.cpipe_e_off);  // [2][T][TS]
+  auto copy_points = [&](int g, int slot) {
+    if (tid < T) {
+      const int b = g / ntile, p0 = (g - b * ntile) << LOGT;
+      if constexpr (TS == 2)
+        cp_async8(Es + (slot * T + tid) * TS, a.Etab + (size_t)(p0 + tid) * TS);
+      else
+        cp_async16(Es + (slot * T + tid) * TS, a.Etab + (size_t)(p0 + tid) * TS);
+    }
+  };
+  // the walk of the tile whose column points are in `slot`
+  auto tile_walk = [&](int slot) {
+    int z[4], e[4], c[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) e[r] = r < TS ? Es[(slot * T + tcol) * TS + r] : 0;
+    load_point<TS>(a.Ctab, start, z);
+    load_point<TS>(a.Ctab, P, c);
+    box_add_t<DIM>(a.boxG, z, e);
+    return BoxWalk<DIM>(a.boxG, z, c, a.m);
+  };
+  // the workspace tile in 16-byte pieces, dense [row][column]
+  auto issue = [&](int g, int n) {
+    const int b = g / ntile, p0 = (g - b * ntile) << LOGT;
+    const C* in = in_all + (int64_t)b * a.m + p0;
+#pragma unroll
+    for (int i = 0; i < L * T / 2 / NT; ++i) {
+      const int c = tid + NT * i;
+      cp_async16(S + (c >> 1) * T + (c & 1) * 2, in + (size_t)(c >> 1) * a.nD + (c & 1) * 2);
+    }
+    copy_points(g, n & 1);
+  };
+
+  if (blockIdx.x < total) issue(blockIdx.x, 0);
+  int n = 0;  // this CTA's tile count
+  for (int g = blockIdx.x; g < total; g += gridDim.x, ++n) {
+    const int gn = g + gridDim.x;
+    cp_async_wait_all();
+    __syncthreads();  // the tile (and, once, the stage table) has landed
+    C v[R];
+    {  // rows j and j + 1024, j = floor(p / 2) + 32 r: their sum or difference
+      const float sg = (p & 1) ? -1.0f : 1.0f;
+      const C* src = S + (p >> 1) * T + tcol;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const C x = src[32 * r * T], y = src[(32 * r + 1024) * T];
+        v[r] = __ffma2_rn(y, make_float2(sg, sg), x);
+      }
+    }
+    __syncthreads();  // S is read: the next tile may land in it
+    if (gn < total) issue(gn, n + 1);
+    // stage 0 (Ns = 2), exchange in two rounds through X
+    if (p & 1) main_twiddle<C, R>(v, stw + a.stw_off[0] + 5);
+    dft_pow2<C, R>(v);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (h) __syncthreads();  // round 0's reads of X are done
+      if ((h ^ (p >> 5)) & 1)
+        cpipe2_x_write<1>(v, X, p, tcol);
+      else
+        cpipe2_x_write<0>(v, X, p, tcol);
+      __syncthreads();
+      if ((h ^ (p >> 5)) & 1)
+        cpipe2_x_read<1>(v, X, p, tcol);
+      else
+        cpipe2_x_read<0>(v, X, p, tcol);
+    }
+    // stage 1 (Ns = 64): v[r] = frequency p + 64 r
+    if (p) main_twiddle<C, R>(v, stw + a.stw_off[1] + p * 5);
+    dft_pow2<C, R>(v);
+
+    // sheared store in two rounds of 16 walk steps through X
+    BoxWalk<DIM> walk = tile_walk(n & 1);
+    C* out = out_all + (int64_t)(g / ntile) * a.m;
+    const float sc = float(a.scale);
+    const int u = (p - off0) & 63;                // AX2: step and walker half of row p of the first cycle
+    const int m0 = ((u + off0) & (L - 1)) >> 6;   // one cycle: floor(i_0 / 64) of the walker of residue p
+    const int sw = AX2 ? p : (p + off0) & 63;     // residue this thread reads as a walker
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      __syncthreads();  // the previous reads of X are done
+      if constexpr (AX2) {
+        if ((u >> 5) == h) {
+          C* wb = X + tcol;
+          const int s0 = (u & 31) << 5;
+#pragma unroll
+          for (int r = 0; r < R; ++r) wb[ct_phys<2>(s0 + ((r - off1) & 31))] = v[r];
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int t = (r - m0 - 16 * h) & 31;
+          if (t < 16) X[(t * P + p) * T + tcol] = v[r];
+        }
+      }
+      __syncthreads();
+#pragma unroll 2
+      for (int t = 0; t < 16; ++t) {
+        const C x = AX2 ? X[ct_phys<2>(t * P + sw) + tcol] : X[(t * P + sw) * T + tcol];
+        out[walk.slot] = __fmul2_rn(x, make_float2(sc, sc));
+        walk.step();
+      }
+    }
+  }
+}
+
 }  // namespace pfft

@@ -42,11 +42,26 @@ static int launch_cpipe_t(const PassArgs& a, cudaStream_t s) {
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+template <int DIM, bool AX2>
+static int launch_cpipe2_t(const PassArgs& a, cudaStream_t s) {
+  static const int ok = configure_kernel(reinterpret_cast<const void*>(col_pipe2_kernel<DIM, AX2>));
+  if (ok != 0) return -1;
+  const int total = (a.nD / 4) * a.batch;
+  dim3 grid(total < a.cpipe_grid ? total : a.cpipe_grid), block(256);
+  col_pipe2_kernel<DIM, AX2><<<grid, block, a.smem_bytes, s>>>(a);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
 // The pipelined column pass serves the two-pass directions: forward
 // (workspace -> box, scaled) and inverse (box -> workspace, conjugated input).
 static int launch_cpipe(const PassArgs& a, cudaStream_t s) {
   const bool fwd = a.load_mode == MAP_WS && a.store_mode == MAP_BOX_G && !a.conj_in && !a.conj_out;
   const bool inv = a.load_mode == MAP_BOX_G && a.store_mode == MAP_WS && a.conj_in && !a.conj_out && a.scale == 1.0;
+  if (a.L == 2048) {  // the forward pass only
+    if (!fwd) return -2;
+    if (a.nsub == 2) return a.d == 3 ? launch_cpipe2_t<3, true>(a, s) : -2;
+    return a.d == 2 ? launch_cpipe2_t<2, false>(a, s) : a.d == 3 ? launch_cpipe2_t<3, false>(a, s) : -2;
+  }
   if (a.d == 2) return fwd ? launch_cpipe_t<2, true>(a, s) : inv ? launch_cpipe_t<2, false>(a, s) : -2;
   if (a.d == 3) return fwd ? launch_cpipe_t<3, true>(a, s) : inv ? launch_cpipe_t<3, false>(a, s) : -2;
   return -2;
@@ -56,6 +71,10 @@ static int launch_cpipe(const PassArgs& a, cudaStream_t s) {
 // rows long; returns -2 when no kernel matches.
 int launch_col_ct2_f32(const PassArgs& a, cudaStream_t s) {
   if (!a.cols || a.d != 3 || a.nsub != 2 || a.sub_n[0] < 32 || a.LB != a.L || a.nthreads != a.T * a.L / 32) return -2;
+  if (a.cpipe) {
+    const int rc = launch_cpipe(a, s);
+    if (rc != -2) return rc;
+  }
   switch (a.L) {
     case 1 << 9: return a.T == 16 ? launch_ct<3, 9, 4, true>(a, s) : -2;
     case 1 << 10: return a.T == 8 ? launch_ct<3, 10, 3, true>(a, s) : -2;

@@ -1248,10 +1248,13 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
       }
     }
   }
-  // pencils of 2^10 complex64 points, 8 per tile: the persistent pipelined column pass
-  if (npen == 1 && P.dtype == PFFT_C64 && !P.tc && P.colp.fast && P.colp.L == (1 << kCPipeLogL) && P.colp.T == 8 &&
-      P.colp.LB == P.colp.L && P.colp.nthreads == 256 && P.colp.fast_tail == 1 && P.colp.fast_nmain == 2 &&
-      (d == 2 || d == 3) && P.nD % 8 == 0) {
+  // pencils of 2^10 complex64 points, 8 per tile, or 2^11, 4 per tile (one cycle, or
+  // two of 64 x 32; forward only): the persistent pipelined column passes
+  const bool cpipe10 = npen == 1 && P.colp.L == (1 << kCPipeLogL) && P.colp.T == 8 && P.colp.fast_tail == 1;
+  const bool cpipe11 = (npen == 1 || (npen == 2 && P.pen[0] == 64)) && P.colp.L == 2 << kCPipeLogL && P.colp.T == 4 &&
+                       P.colp.fast_tail == 2;
+  if ((cpipe10 || cpipe11) && P.dtype == PFFT_C64 && !P.tc && P.colp.fast && P.colp.LB == P.colp.L &&
+      P.colp.nthreads == 256 && P.colp.fast_nmain == 2 && (d == 2 || d == 3) && P.nD % P.colp.T == 0) {
     int nsm = 0;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, P.device) != cudaSuccess || nsm < 1)
       return PFFT_ERR_CUDA;
