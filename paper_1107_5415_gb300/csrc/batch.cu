@@ -6,8 +6,9 @@
 // fft_mixed.cuh, whose tables are sub-allocated from one arena.  A schedule turns
 // the plans into grouped launches: for each pass, the patterns are grouped by
 // the threads of their tile into at most kMaxBuckets launches (so that small
-// tiles are not held to the occupancy of the largest one), those launches run concurrently on forked streams, and inside a
-// launch the CTAs of the costliest tiles come first.  The split level of every
+// tiles are not held to the occupancy of the largest one), those launches run
+// concurrently on forked streams, and inside a launch the CTAs of the costliest
+// tiles come first.  The split level of every
 // pattern is one more grouped launch.  The autotuner times candidate tile
 // budgets and orders on the real batch and keeps the fastest.
 #include <cuda_runtime.h>
@@ -28,8 +29,12 @@ namespace {
 constexpr int kMaxBuckets = 6;
 // Upper ends of the thread classes of a grouped pass launch: every CTA of a
 // launch has the threads of its largest tile, and a tile's idle warps hold
-// registers and wait at its barriers.
-constexpr int kThreadClass[kMaxBuckets] = {128, 256, 384, 512, 768, 1024};
+// registers and wait at its barriers.  The classes from 192 on are what 5, 4, 3, 2
+// and 1 CTAs share of the 1024 threads that an SM's registers hold (complex64): tiles
+// of 257 to 384 threads in one class of 384 left a quarter of them unused (a mix of
+// 512 patterns: 2.25 ms with {128, 256, 384, 512, 768, 1024}, 2.16 without the
+// class of 192, 2.15 so).
+constexpr int kThreadClass[kMaxBuckets] = {128, 192, 256, 320, 512, 1024};
 
 struct Bucket {
   int n = 0, nctas = 0, threads = 0, smem = 0;
