@@ -148,8 +148,7 @@ pfft_status build_schedule(pfft_batch_s& B) {
     // one tile per signal, or the row pass and the column pass
     const bool whole = P->mixed[MIX_WHOLE], single = whole || P->pen.empty();
     MixDesc r = P->mix[whole ? MIX_WHOLE : MIX_ROW];
-    r.load_mode = MAP_BOX_H;
-    r.store_mode = single ? MAP_BOX_G : MAP_WS;
+    mix_sides(r, MAP_BOX_H, single ? MAP_BOX_G : MAP_WS);
     r.scale = single ? scale : 1.0;
     r.in_sel = 0;
     r.out_sel = single ? 2 : 1;
@@ -158,8 +157,7 @@ pfft_status build_schedule(pfft_batch_s& B) {
     rows.push_back({r, i, tile_cost(r)});
     if (!single) {
       MixDesc c = P->mix[MIX_COL];
-      c.load_mode = MAP_WS;
-      c.store_mode = MAP_BOX_G;
+      mix_sides(c, MAP_WS, MAP_BOX_G);
       c.scale = scale;
       c.in_sel = 1;
       c.out_sel = 2;

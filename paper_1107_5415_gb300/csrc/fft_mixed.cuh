@@ -268,7 +268,7 @@ __device__ __forceinline__ void mix_stage(C* sm, const MixDesc& a, const MixStag
         for (int p = 0; p < NP; ++p) w[p] = __ldg(tab + p * s.Ns + k);
       }
       const int x = base + j * s.sig;
-      const C* src = sm + x + s.ipad * a.div_pad.div(x);
+      const C* src = sm + x + s.ipad * s.div_in.div(x);
 #pragma unroll
       for (int r = 0; r < R; ++r) v[q][r] = src[r * istep];
       if constexpr (kMixFused<C, R>) {
@@ -281,7 +281,7 @@ __device__ __forceinline__ void mix_stage(C* sm, const MixDesc& a, const MixStag
         mdft<C, R>(v[q]);
       }
       const int y = base + ((j - k) * R + k) * s.sig;
-      ob[q] = y + s.opad * a.div_pad.div(y);
+      ob[q] = y + s.opad * s.div_out.div(y);
     }
   }
   __syncthreads();
@@ -652,8 +652,7 @@ __device__ __forceinline__ void mix_row_box(const MixDesc& a, int tile, const C*
 }
 
 // Row tiles against the workspace, where rows are contiguous; an element's tile
-// position comes from the table of its column position (PIinv, or psout in the
-// padded tile).  The lanes run along a row; in a [element][row] tile of at least
+// position comes from the table of its column position (psin, psout).  The lanes run along a row; in a [element][row] tile of at least
 // four rows, over four adjacent elements of each row in turn, which are four
 // adjacent banks per row in the tile and one 32-byte sector in the workspace.
 // FS: a split last cycle, whose phase is applied here.
@@ -662,7 +661,7 @@ __device__ __forceinline__ void mix_row_ws(const MixDesc& a, int tile, const C* 
                                            C* sm) {
   using Rl = decltype(C::x);
   const int r0 = tile * a.T, nD = pinned(a.nD), rows = a.LB - r0;
-  const int* __restrict__ ps = LOAD ? a.PIinv : a.psout;
+  const int* __restrict__ ps = LOAD ? a.psin : a.psout;
   const Rl sy = (LOAD ? a.conj_in : 0) ? Rl(-1) : Rl(1);
   if constexpr (FS) {
     // blockDim.x is a multiple of 4 T (mix_configure): a thread keeps its row
@@ -683,7 +682,7 @@ __device__ __forceinline__ void mix_row_ws(const MixDesc& a, int tile, const C* 
           return cmul(v, mix_phase<C>(a, la, __ldg(mu + elem(w))));
         });
   } else {
-    const int pitch = LOAD ? nD : a.pitch, base = r0 * nD;
+    const int pitch = LOAD ? a.pitch_in : a.pitch_out, base = r0 * nD;
     const FastDiv dn = pinned(a.divnD);
     auto value = [&](C v, int) { return LOAD ? mix_scale(v, Rl(1), sy) : v; };
     auto ok = [](int) { return true; };

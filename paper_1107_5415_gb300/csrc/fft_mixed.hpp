@@ -47,12 +47,17 @@ constexpr int kMixThreadsC64 = 1024, kMixThreadsC128 = 512;
 // elements (one pencil position) follow every R1 of them from there.  R1 divides
 // every later step, so all accesses of a stage stay affine in r: istep and ostep
 // are the padded steps, ipad / opad the padding per pad unit (0: not padded).
+// The workspace side of a row tile visits the elements in the order of the column
+// positions, which may put every lane into the same bank: there the padding is by
+// a unit of its own (MixDesc::ws_in, ws_out), which divides the step of the first
+// stage's inputs or of the last one's outputs.
 struct MixStage {
   int R, aR, sig, Ns, blk;
   int istep, ostep, ipad, opad;
   int tw;       // twiddles of the stage in the stage table: [b][k] (MixTableArgs)
   int gen;      // direct stages: offset of g^t mod R (R - 1 ints) in the integer table
   int twstep;   // direct stages: step of the root table per unit of exp(-2 pi i / (Ns R))
+  FastDiv div_in, div_out;  // by the pad units of the inputs and of the outputs
   FastDiv div_sig, div_aR, div_Ns, div_nb;  // div_nb: direct stages, butterflies of the tile
 };
 
@@ -65,8 +70,9 @@ struct alignas(16) MixDesc {
   int nthreads, smem_bytes;
   int pad;            // padding of the finished tile: position x at x + pad (x / pad unit)
   FastDiv div_pad;    // by the pad unit (R1 positions of the fastest axis)
-  int pitch;          // row tiles in [row][element] order: distance of the finished rows
-  const int* psout;   // row tiles: padded element position of each column position (unpadded: PIinv)
+  int ws_in, ws_out;  // row tiles in [row][element] order: pad units of the workspace side (0: as without)
+  int pitch_in, pitch_out;  // their distances of the rows
+  const int *psin, *psout;  // row tiles: padded element position of each column position
   int dir_off;        // tables of the direct stages after the tile (elements)
   int nstages;
   int tw_n;           // order of the root table
@@ -107,6 +113,26 @@ struct MixTableArgs {
   int fused[kMixMaxStages];
   int R[kMixMaxStages], Ns[kMixMaxStages], off[kMixMaxStages + 1];
 };
+
+// Sets the sides of a call (load and store map) in a row tile's descriptor: the
+// workspace side has its own padding.
+inline void mix_sides(MixDesc& a, int load, int store) {
+  a.load_mode = load;
+  a.store_mode = store;
+  if (load == MAP_WS && a.ws_in) {
+    MixStage& s = a.st[0];
+    s.ipad = 1;
+    s.istep += s.istep / a.ws_in;
+    s.div_in.init(uint32_t(a.ws_in));
+  }
+  if (store == MAP_WS && a.ws_out) {
+    MixStage& s = a.st[a.nstages - 1];
+    s.opad = 1;
+    s.ostep = s.Ns * s.sig;
+    s.ostep += s.ostep / a.ws_out;
+    s.div_out.init(uint32_t(a.ws_out));
+  }
+}
 
 // Host-side launchers (fft_mixed_c64.cu, fft_mixed_c128.cu, fft_support.cu).
 int launch_mixed_c64(const MixDesc& a, cudaStream_t s);

@@ -18,7 +18,8 @@ struct MixStages {
   std::vector<pfft::MixStage> st;  // sig, blk and the divisors of a tile are set with its T
   void* stw = nullptr;
   int* gtab = nullptr;
-  int* psout = nullptr;
+  int ws_in = 0, ws_out = 0;  // row tiles: pad units of the workspace side
+  int *psin = nullptr, *psout = nullptr;
 };
 
 struct pfft_plan_s {

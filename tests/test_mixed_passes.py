@@ -203,3 +203,14 @@ def test_transposed_route(M):
     for f in ("forward", "inverse"):
         u, v = getattr(a, f)(x).cpu().numpy(), getattr(b, f)(x).cpu().numpy()
         assert rel_l2(v, u) <= TOL["c64"]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.complex64, torch.complex128], ids=["c64", "c128"])
+@pytest.mark.parametrize("M", [[[160, 150], [0, 270]], [[480, 60], [0, 540]], [[240, 48], [0, 216]],
+                               [[720, 16], [0, 720]], [[1200, 240], [0, 1080]]],
+                         ids=["step16", "step8", "rows", "several", "step40"])
+def test_strided_column_order(M, dtype):
+    """Rows whose column order steps by multiples of the banks: the workspace
+    side of a row tile is padded by a unit of its own (pad_unit)."""
+    test_mixed_passes(M, 2, dtype)
