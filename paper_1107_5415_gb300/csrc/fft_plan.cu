@@ -437,6 +437,12 @@ pfft_status mix_stages(pfft_plan_s& P, int kind) {
   return PFFT_OK;
 }
 
+// Points per thread of a launch that does not fill the chip.  [[64, 16], [-16,
+// 64]] x 1 there and back: 28.4 us with 16, 26.3 with 8, 29.7 with 5; [[300, 60],
+// [0, 240]] x 1: 31.1 and 28.2 us; [[60, 24], [0, 72]] x 1 in complex128: 62 and 50.6 us.
+constexpr int kMixFewPoints = 8;
+constexpr int kSMs = 152;
+
 // The descriptor of a kind of tile with T pencils (T a power of two; any T for
 // row tiles in [row][element] order and whole tiles).
 pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
@@ -490,6 +496,12 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
     if (s.R >= kMixMinDirect) rmax = std::max(rmax, s.R);
   }
   a.nthreads = mix_threads(rad, a.n, max_threads);
+  // a launch that leaves the chip idle gets twice the threads that its stages ask
+  // for, as long as all of it stays resident: half the turns of every load and store
+  const int more = (a.n + kMixFewPoints - 1) / kMixFewPoints;
+  const i64 ctas = i64(a.groups) * (kind == MIX_WHOLE ? 1 : P.batch);
+  if (!P.generic_only && more <= max_threads && ctas * more <= i64(kSMs) * max_threads)
+    a.nthreads = std::max(a.nthreads, (more + 31) / 32 * 32);
   // each thread keeps one column (or, of a [element][row] tile, one row in turns of four elements)
   const int keep = a.lay ? 4 * T : tstride;
   if (a.nthreads % keep) a.nthreads = (a.nthreads + keep - 1) / keep * keep;
