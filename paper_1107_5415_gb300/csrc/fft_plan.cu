@@ -538,7 +538,13 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
 // Pencils per tile: as many as `budget` points hold (at most `cap`), up to
 // `lanes` of them (the adjacent pencils that fill a 32-byte sector) even when
 // that takes `most` points; but no more than leave `ctas` tiles for the launch
-// once those lanes are there.
+// once those lanes are there.  A tile of more than half the threads of an SM has
+// it alone, every phase waiting for the one before: half the pencils are then the
+// better tile, and half of the last 16 bytes of a sector if that puts a quarter more
+// threads on the SM (there and back, columns of 1728 points in 576 threads, [[1728,
+// 1472], [0, 2048]] x 3: 0.414 and 0.365 ms; [[96, 87, 0], [0, 375, 201], [0, 0,
+// 243]] x 7, two columns of 3240 points in 544 threads: 3.60 and 3.24; a mix of 512
+// patterns: 2.14 and 2.11; but two of 3850 points in 704 threads lose 7%).
 pfft_status mix_choose(pfft_plan_s& P, int kind, int cap, int budget, int most, int lanes, int ctas) {
   pfft_status st = mix_stages(P, kind);
   if (st != PFFT_OK) return st;
@@ -554,7 +560,10 @@ pfft_status mix_choose(pfft_plan_s& P, int kind, int cap, int budget, int most, 
   }
   for (;; T /= 2) {
     st = mix_configure(P, kind, T);
-    if (st == PFFT_OK || T == 1) return st;
+    const int max = mix_max_threads(P.dtype), t = P.mix[kind].nthreads, half = (t / 2 + 31) / 32 * 32;
+    if (T == 1) return st;
+    if (st != PFFT_OK) continue;
+    if (t <= max / 2 || (T * elem_bytes(P.dtype) <= 16 && 4 * (max / half * half) < 5 * t)) return st;
   }
 }
 
