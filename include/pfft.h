@@ -334,7 +334,7 @@ pfft_status pwt_merge_general(int d, const int64_t* M, const int64_t* J, int64_t
  * only, else PFFT_ERR_UNSUPPORTED).  All patterns run together: grouped
  * launches (the row pass of every pattern, the column pass, the split
  * levels), each CTA finding its pattern in a device table, with patterns
- * grouped by shared-memory footprint into concurrent launches, replayed as
+ * grouped by the threads of their tiles into concurrent launches, replayed as
  * one CUDA graph.
  *
  * Data: the signals are concatenated, pattern i occupying elements
@@ -356,9 +356,9 @@ enum {
    * device queue in dependency order; a column tile waits (bounded) until
    * its pattern's row tiles are done, a split unit until the pattern's
    * coefficients are.  Results equal the grouped launches' up to rounding
-   * (every tile runs with 512 threads, which changes how the stage twiddle
-   * powers are formed).  All units share the largest tile's shared memory
-   * (fewer CTAs per SM when one pattern needs a large tile). */
+   * (the same tiles compiled into another kernel).  All units run with the
+   * largest tile's threads and shared memory (fewer CTAs per SM when one
+   * pattern needs a large tile). */
   PFFT_BATCH_ONE_LAUNCH = 8u
 };
 

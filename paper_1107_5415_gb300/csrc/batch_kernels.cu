@@ -13,6 +13,10 @@
 
 namespace pfft {
 
+// The single-launch kernel holds one descriptor of each kind.
+static_assert(sizeof(MixDesc) + sizeof(SplitItem) + sizeof(PrimeItem) + 256 <= 227 * 1024 - kMixGroupedSmem,
+              "static shared memory of a grouped kernel");
+
 // Largest k with cta0[k] <= b (cta0 ascending, cta0[0] = 0).
 __device__ __forceinline__ int find_item(const int* __restrict__ cta0, int n, int b) {
   int lo = 0, hi = n - 1;

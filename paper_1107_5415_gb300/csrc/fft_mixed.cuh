@@ -20,10 +20,14 @@
 // 1.993 -> 1.027 ms; [[64, 16], [-16, 64]] x 1: 0.089 -> 0.033 ms; a mix of 512
 // patterns: 3.65 -> 2.84 ms.  With the setups of a thread's loops trimmed (stage
 // tests by group, shears by multiply-high, one row per thread of a split tile):
-// 0.402, 0.964, 0.033 and, with the 32-bit splits, 2.33 ms.  Reading the workspace
+// 0.402, 0.964, 0.033 and, with the 32-bit splits, 2.33 ms.  With the padding of the
+// workspace side (pad_unit), eight points a thread in launches that leave the chip
+// idle and two or more tiles per SM wherever the pencils allow it: 0.388, 0.958,
+// 0.025 (0.029 with sixteen) and 2.20 ms.  Reading the workspace
 // straight into the first butterflies of a column tile and writing it from the last
-// ones saves instructions in such tiles but costs every other stage (0.415 for
-// the first).
+// ones saves instructions in such tiles but costs every other stage (0.415 ms for
+// the first), and so does a copy of the load and store loops without bounds checks
+// (0.393 against 0.389: the instruction cache).
 #pragma once
 #include <cuda_runtime.h>
 

@@ -34,8 +34,8 @@ constexpr int kMixOrder[15] = {15, 13, 11, 9, 16, 14, 12, 10, 8, 7, 6, 5, 4, 3, 
 template <typename C>
 constexpr int kMixThreads = sizeof(C) == 8 ? 1024 : 512;
 // Dynamic shared memory of a grouped tile: the 227 KB per CTA less room for the
-// static copy of its descriptor.
-constexpr int kMixGroupedSmem = 227 * 1024 - 4096;
+// static copies of the descriptors (batch_kernels.cu checks that they fit).
+constexpr int kMixGroupedSmem = 227 * 1024 - 8192;
 constexpr int kMixThreadsC64 = 1024, kMixThreadsC128 = 512;
 
 // One radix stage along one axis.  Tile positions of a butterfly (low, j, hi):
@@ -89,7 +89,7 @@ struct alignas(16) MixDesc {
   const void *fs_lo, *fs_hi;    // phases of a split last cycle (fft_plan.hpp)
   int fs_na;
   FastDiv fs_div;
-  FastDiv divT, divnD, divL;
+  FastDiv divnD, divL;
   int nsub, sub_n[kMaxSub], alpha[kMaxSub];
   FastDiv sub_div[kMaxSub];
   BoxDesc boxH, boxG;

@@ -458,7 +458,6 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
   a.n = T * a.L;
   const int count = kind == MIX_ROW ? P.LB : kind == MIX_COL ? P.nD : int(P.batch);
   a.groups = (count + T - 1) / T;
-  a.divT.init(uint32_t(T));
   a.divnD.init(uint32_t(P.nD));
   a.divL.init(uint32_t(a.L));
   a.stw = S.stw;

@@ -152,9 +152,6 @@ struct alignas(16) PassArgs {
   double scale;
   const void* in;
   void* out;
-  // grouped launches: in / out hold byte offsets into the launch's base
-  // pointer number in_sel / out_sel (see batch_kernels.cu)
-  int in_sel, out_sel;
   // tables (device, d int32 per entry)
   const int* Atab;   // [LB]  box(H) point of sum_{j<D} lambda_j g_j
   const int* Btab;   // [nD]  box(H) point of lambda_D g_D

@@ -40,7 +40,7 @@ struct pfft_plan_s {
   void* fs_tab = nullptr;   // exp(-2 pi i t / fs_N), two-level table
   // options (set before plan_device)
   pfft::Arena* arena = nullptr;  // sub-allocate device tables here (batch plans)
-  bool generic_only = false;     // shared-memory Stockham kernels only (grouped launches)
+  bool generic_only = false;     // mixed-radix passes only (grouped launches)
   bool own_workspace = true;     // allocate the LB x nD workspace
   bool tc = false;               // split-precision tensor-core radix-16 / 32 stages
   int max2 = 16;                 // largest power-of-two radix of the mixed-radix passes (16 or 8)
@@ -82,8 +82,8 @@ pfft_status plan_host(pfft_plan_s& P, int d, const int64_t* M);
 // Device tables and pass descriptors.
 pfft_status plan_device(pfft_plan_s& P);
 // Re-choose the tiles of both passes (pencils per CTA) under the given
-// element budgets and the largest power-of-two radix (16 or 8); generic
-// kernels only.  Tables are unchanged.
+// element budgets and the largest power-of-two radix (16 or 8); mixed-radix
+// passes only.  Tables are unchanged.
 pfft_status plan_retile(pfft_plan_s& P, int row_budget, int col_budget, int max2);
 void plan_release(pfft_plan_s* P);
 }  // namespace pfft
