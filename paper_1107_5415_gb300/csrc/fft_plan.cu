@@ -214,7 +214,9 @@ bool tc_tile_fits(int L, int row_max) {
 }
 
 // ------------------------------------------------ mixed-radix passes (fft_mixed.cuh)
-int mix_max_threads(int dtype) { return dtype == PFFT_C64 ? kMixThreadsC64 : kMixThreadsC128; }
+int mix_max_threads(const pfft_plan_s& P) {
+  return std::min(P.max_threads, P.dtype == PFFT_C64 ? kMixThreadsC64 : kMixThreadsC128);
+}
 int mix_points(int R) { return R * std::max(1, kMixPoints / R); }  // points a thread takes in a radix-R stage
 
 // Instructions a point costs in one stage: 8 for the shared-memory round trip,
@@ -272,7 +274,7 @@ bool mixed_radices(int n, int min_points, int max2, std::vector<int>& out, doubl
 }
 
 // Points per thread that every stage of a pencil of L points must reach.
-int mix_min_points(int L, int dtype) { return (L + mix_max_threads(dtype) - 1) / mix_max_threads(dtype); }
+int mix_min_points(int L, const pfft_plan_s& P) { return (L + mix_max_threads(P) - 1) / mix_max_threads(P); }
 
 // Threads of a mixed-radix tile of n points.
 int mix_threads(const std::vector<int>& radices, int n, int max_threads) {
@@ -293,17 +295,17 @@ int mix_threads(const std::vector<int>& radices, int n, int max_threads) {
 }
 
 // Whether a pencil of L points (one axis, or the axes of a column) fits a tile.
-bool mix_fits(const std::vector<int>& axes, int L, int dtype, double* cost = nullptr) {
-  if (L > (dtype == PFFT_C64 ? 16384 : 8192)) return false;
+bool mix_fits(const pfft_plan_s& P, const std::vector<int>& axes, int L, double* cost = nullptr) {
+  if (L > (P.dtype == PFFT_C64 ? 16384 : 8192)) return false;
   std::vector<int> all, rad;
   double c = 0, ca = 0;
   for (int a : axes) {
-    if (!mixed_radices(a, mix_min_points(L, dtype), 16, rad, &ca)) return false;
+    if (!mixed_radices(a, mix_min_points(L, P), 16, rad, &ca)) return false;
     all.insert(all.end(), rad.begin(), rad.end());
     c += ca;
   }
   if (cost) *cost = c;
-  return int(all.size()) <= kMixMaxStages && mix_threads(all, L, mix_max_threads(dtype)) <= mix_max_threads(dtype);
+  return int(all.size()) <= kMixMaxStages && mix_threads(all, L, mix_max_threads(P)) <= mix_max_threads(P);
 }
 
 // Pad unit u (element x at x + x / u) under which a walk over the elements in the
@@ -361,7 +363,7 @@ pfft_status mix_stages(pfft_plan_s& P, int kind) {
   std::vector<std::pair<int, int>> order;  // (radix, axis)
   std::vector<int> rad;
   for (size_t i = 0; i < axes.size(); ++i) {
-    if (!mixed_radices(axes[i].a, mix_min_points(L, P.dtype), P.max2, rad)) return PFFT_ERR_UNSUPPORTED;
+    if (!mixed_radices(axes[i].a, mix_min_points(L, P), P.max2, rad)) return PFFT_ERR_UNSUPPORTED;
     for (int R : rad) order.push_back({R, int(i)});
   }
   if (order.size() > size_t(kMixMaxStages)) return PFFT_ERR_UNSUPPORTED;
@@ -448,7 +450,7 @@ constexpr int kSMs = 152;
 pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
   MixDesc& a = P.mix[kind];  // its plan-wide fields are set (plan_device)
   const MixStages& S = P.stages[P.max2 == 16 ? 0 : 1][kind];
-  const int max_threads = mix_max_threads(P.dtype);
+  const int max_threads = mix_max_threads(P);
   a.kind = kind;
   a.lay = kind == MIX_ROW && P.fs_na > 1 ? 1 : 0;
   a.L = kind == MIX_ROW ? P.nD : kind == MIX_COL ? P.LB : int(P.m);
@@ -559,7 +561,7 @@ pfft_status mix_choose(pfft_plan_s& P, int kind, int cap, int budget, int most, 
   }
   for (;; T /= 2) {
     st = mix_configure(P, kind, T);
-    const int max = mix_max_threads(P.dtype), t = P.mix[kind].nthreads, half = (t / 2 + 31) / 32 * 32;
+    const int max = P.dtype == PFFT_C64 ? kMixThreadsC64 : kMixThreadsC128, t = P.mix[kind].nthreads, half = (t / 2 + 31) / 32 * 32;
     if (T == 1) return st;
     if (st != PFFT_OK) continue;
     if (t <= max / 2 || (T * elem_bytes(P.dtype) <= 16 && 4 * (max / half * half) < 5 * t)) return st;
@@ -788,7 +790,7 @@ pfft_status pfft::plan_host(pfft_plan_s& P, int d, const int64_t* Mv) {
   // and lambda_a becomes one more pencil axis of the column pass.
   const int row_max = P.dtype == PFFT_C64 ? 16384 : 8192;
   const i64 n = P.fs_N;
-  const bool split = n > 1 && (n > row_max || !(P.tc ? tc_tile_fits(int(n), row_max) : mix_fits({int(n)}, int(n), P.dtype)));
+  const bool split = n > 1 && (n > row_max || !(P.tc ? tc_tile_fits(int(n), row_max) : mix_fits(P, {int(n)}, int(n))));
   if (split) {
     const i64 other = P.m / n;
     int best = 0;
@@ -811,7 +813,7 @@ pfft_status pfft::plan_host(pfft_plan_s& P, int d, const int64_t* Mv) {
       double cr = 0, cc = 0;
       std::vector<int> pen(P.pen.begin(), P.pen.end());
       pen.push_back(int(na));
-      if (!mix_fits({int(nb)}, int(nb), P.dtype, &cr) || !mix_fits(pen, int(lb), P.dtype, &cc)) continue;
+      if (!mix_fits(P, {int(nb)}, int(nb), &cr) || !mix_fits(P, pen, int(lb), &cc)) continue;
       const int unit = P.dtype == PFFT_C64 ? 1024 : 512;
       auto long_tile = [&](i64 L) { return L > 8 * unit ? 60.0 : L > 4 * unit ? 30.0 : L > 2 * unit ? 12.0 : L > unit ? 3.0 : 0.0; };
       const double c = cr + cc + long_tile(nb) + long_tile(lb) + 3.0 * std::max<i64>(0, 8 - na);
@@ -1005,7 +1007,7 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
     const i64 half = P.dtype == PFFT_C64 ? 8192 : 4096;
     std::vector<int> axes(P.pen.begin(), P.pen.end());
     axes.push_back(nD);
-    P.mixed[MIX_WHOLE] = !P.tc && na == 1 && P.m <= (P.batch >= 64 ? 2 * half : half) && mix_fits(axes, int(P.m), P.dtype);
+    P.mixed[MIX_WHOLE] = !P.tc && na == 1 && P.m <= (P.batch >= 64 ? 2 * half : half) && mix_fits(P, axes, int(P.m));
   }
   if (npen >= 1 && P.own_workspace && !P.mixed[MIX_WHOLE])
     if (int e_ = P.alloc(&P.ws, size_t(P.m) * P.batch * eb)) return pfft_status(e_);

@@ -40,6 +40,7 @@ struct pfft_plan_s {
   void* fs_tab = nullptr;   // exp(-2 pi i t / fs_N), two-level table
   // options (set before plan_device)
   pfft::Arena* arena = nullptr;  // sub-allocate device tables here (batch plans)
+  int max_threads = 1024;        // of a mixed-radix tile (complex128: 512 at most)
   bool generic_only = false;     // mixed-radix passes only (grouped launches)
   bool own_workspace = true;     // allocate the LB x nD workspace
   bool tc = false;               // split-precision tensor-core radix-16 / 32 stages
