@@ -214,3 +214,24 @@ def test_strided_column_order(M, dtype):
     """Rows whose column order steps by multiples of the banks: the workspace
     side of a row tile is padded by a unit of its own (pad_unit)."""
     test_mixed_passes(M, 2, dtype)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.complex64, torch.complex128], ids=["c64", "c128"])
+def test_one_launch_tile_limit(dtype):
+    """A single-launch batch plans tiles of at most 512 threads; columns of 96^2
+    points have no such tile in complex64 and keep the larger one."""
+    n = 96 if dtype == torch.complex64 else 64
+    Ms = [[[n, 0, 0], [0, n, 0], [0, 0, n]], [[16, 3], [0, 30]], [[10800]]]
+    A = pf.PatternBatch(Ms, None, dtype=dtype)
+    Q = pf.PatternBatch(Ms, None, dtype=dtype, flags=pf.PFFT_BATCH_ONE_LAUNCH)
+    x = SI.complex_normal(1, A.total, seed=5, dtype=np.complex64 if dtype == torch.complex64 else np.complex128)
+    x = torch.from_numpy(x[0]).cuda()
+    want, got = A.forward(x), Q.forward(x)
+    Q.check_device_status()
+    tol = TOL["c64" if dtype == torch.complex64 else "c128"]
+    off = 0
+    for M in Ms:
+        m = abs(L.det(M))
+        assert rel_l2(got[off:off + m].cpu().numpy(), want[off:off + m].cpu().numpy()) <= tol
+        off += m
