@@ -1016,7 +1016,6 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
     if (int e_ = P.alloc(&P.fs_tab, size_t(2048 + nhi) * eb)) return pfft_status(e_);
     if (launch_phase_tables(P.fs_tab, P.fs_N, nhi, P.dtype, 0) != 0) return PFFT_ERR_CUDA;
   }
-  if (cudaDeviceSynchronize() != cudaSuccess) return PFFT_ERR_CUDA;
 
   // pass descriptors (data pointers and modes are filled per call)
   // arithmetic forms of PI and of the gather table (power-of-two cycles)
@@ -1350,22 +1349,25 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
       P.colp.smem_bytes = bytes;
     }
   }
+  int* didx = nullptr;
+  int rc = 0;
   if (!idx.empty()) {
-    int* didx = nullptr;
     if (int e_ = device_alloc((void**)&didx, idx.size() * sizeof(int))) return pfft_status(e_);
     if (int e_ = P.alloc(&P.stw, idx.size() * eb)) {
       cudaFree(didx);
       return pfft_status(e_);
     }
     cudaMemcpy(didx, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice);
-    const int rc = launch_twiddle_gather(P.stw, P.tw, didx, int(idx.size()), P.dtype, 0);
-    const cudaError_t ce = cudaDeviceSynchronize();
-    cudaFree(didx);
-    if (rc != 0 || ce != cudaSuccess) return PFFT_ERR_CUDA;
+    rc = launch_twiddle_gather(P.stw, P.tw, didx, int(idx.size()), P.dtype, 0);
     for (size_t i = 0; i < fastp.size(); ++i)
       fastp[i]->stw_g = static_cast<const char*>(P.stw) + base[i] * eb;
   }
-  return PFFT_OK;
+  // Every table above is built or copied on the default stream.  The first call
+  // may come on a stream that does not wait for that one (cudaStreamNonBlocking),
+  // so the host does, after the last of them.
+  const cudaError_t ce = cudaDeviceSynchronize();
+  if (didx) cudaFree(didx);
+  return rc == 0 && ce == cudaSuccess ? PFFT_OK : PFFT_ERR_CUDA;
 }
 
 pfft_status pfft::plan_retile(pfft_plan_s& P, int row_budget, int col_budget, int max2) {
