@@ -25,7 +25,9 @@
  *
  *  Data.  Complex interleaved (re, im): PFFT_C64 = 2 x float, PFFT_C128 =
  *  2 x double.  Buffers are DEVICE pointers owned by the caller, contiguous,
- *  batch outermost ([batch][m]).  All transform calls are asynchronous and
+ *  batch outermost ([batch][m]), aligned to one element (8 or 16 bytes); the
+ *  complex64 row passes by bulk copies want 16 bytes and are replaced by
+ *  element-wise ones, call by call, where a buffer has less.  All transform calls are asynchronous and
  *  stream-ordered on the given cudaStream_t (passed as void*, NULL = legacy
  *  default stream); nothing on the hot path synchronises with the host.
  *  Input and output must not overlap.
@@ -213,7 +215,8 @@ pfft_status pfft_last_device_status(pfft_plan p, void* stream);
  * waits with the default limit for its own copies, and returns without
  * transforming, so the output of such a call is undefined.  Host-side
  * setting, applies to later calls.  Returns PFFT_ERR_UNSUPPORTED for a plan
- * whose row pass does not stage through bulk copies (no such wait). */
+ * whose row pass does not stage through bulk copies (no such wait; nor has a
+ * call on a buffer that is not 16-byte aligned). */
 pfft_status pfft_set_wait_limit(pfft_plan p, int64_t spins);
 
 /* Per-kernel timing of a plan's launches (CUDA events recorded on the

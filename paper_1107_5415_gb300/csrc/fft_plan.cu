@@ -1541,6 +1541,12 @@ static pfft_status run_pass(pfft_plan_s* P, const pfft_plan_s* t, int kind, int 
     return PFFT_OK;
   }
   PassArgs a = kind == MIX_COL ? t->colp : t->rowp;
+  // Bulk copies start on 16 bytes.  The planner checked the rows' offsets inside a
+  // signal; a caller's array that starts 8 bytes past such an address (a slice of a
+  // tensor) is read and written element by element, by the kernel that rows
+  // without whole runs take.  Its exchange, L + L / 32 elements, ends before the
+  // stage table of either layout.
+  if (a.tma && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15)) a.tma = a.pipe = 0;
   a.load_mode = load;
   a.store_mode = store;
   a.conj_in = cin;

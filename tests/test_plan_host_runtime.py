@@ -71,6 +71,46 @@ def test_plan_tables_are_built_when_the_plan_is(fake, name, dtype, flags):
         fake.pfft_plan_destroy(h)
 
 
+ROWS = {2048: [[512, 128], [0, 512]], 4096: [[8, 0], [0, 4096]], 8192: [[4, 0], [0, 8192]], 16384: [[4, 0], [0, 16384]]}
+
+
+@pytest.mark.parametrize("inverse", [False, True], ids=["forward", "inverse"])
+@pytest.mark.parametrize("n", ROWS)
+def test_bulk_copies_only_where_they_are_aligned(fake, n, inverse):
+    """A bulk copy starts on 16 bytes: rows of a signal that begins 8 bytes past
+    such an address are read and written element by element."""
+    st, h = _create(fake, ROWS[n])
+    assert st == 0
+    f = fake.pfft_inverse if inverse else fake.pfft_forward
+    for src, dst, bulk in ((4096, 8192, True), (4104, 8192, inverse), (4096, 8200, not inverse), (4104, 8200, False)):
+        fake.fake_reset()
+        assert f(h, src, dst, None) == 0
+        rows = fake.fake_kernel(1 if inverse else 0).decode()
+        assert ("row_tma" in rows or "row_pipe" in rows) if bulk else "row_fast" in rows
+    fake.pfft_plan_destroy(h)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", ROWS)
+def test_transform_of_a_view_aligned_to_one_element(n):
+    M = ROWS[n]
+    m = abs(L.det(M))
+    plan = pf.PatternFFT(M, 2)
+    c = SI.complex_normal(2, m, seed=m % 83)
+
+    def view():
+        return torch.empty(2 * m + 1, dtype=torch.complex64, device="cuda")[1:].view(2, m)
+
+    x = view().copy_(torch.from_numpy(c))
+    y, z = view(), view()
+    assert x.data_ptr() % 16 == 8
+    plan.forward(x, out=y)
+    plan.inverse(y, out=z)
+    slots = SI.sample_slots(m, 1024, seed=3)
+    assert rel_l2(y.cpu().numpy()[:, slots], oracle.pattern_fft(M, c, out_slots=slots)) <= TOL["c64"]
+    assert rel_l2(z.cpu().numpy(), c) <= TOL["c64"]
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("name", ["whole", "whole-direct", "two-mixed", "split", "fast"])
 def test_first_call_on_a_side_stream(name):
