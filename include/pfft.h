@@ -48,8 +48,12 @@
  *  cycles but the last must be <= S; the last cycle n either fits (n <= S)
  *  or splits as n = n_a n_b with n_b <= S and P n_a <= S (four-step split
  *  inside the two passes).  Cycle lengths may contain any prime factor up to
- *  1021 (primes from 11 up are evaluated as direct sums: O(p) work per point
- *  for a factor p).  Anything else is rejected with PFFT_ERR_UNSUPPORTED at
+ *  1021 (primes from 17 up, and 11 and 13 in long PFFT_C128 tiles, are
+ *  evaluated as direct sums: O(p) work per point for a factor p).  A tile whose
+ *  length is no power of two holds fewer points by its factors, in the threads
+ *  of one CTA: 15/16 S with a factor 3 or 5, 7/8 S with 7 and, PFFT_C64 only,
+ *  13/16 S with 13 and 11/16 S with 11 (a last cycle beyond that is
+ *  split if it can be).  Anything else is rejected with PFFT_ERR_UNSUPPORTED at
  *  plan time.
  */
 #ifndef PFFT_H

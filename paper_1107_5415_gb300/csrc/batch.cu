@@ -96,7 +96,7 @@ double tile_cost(const MixDesc& a) {
   double w = 0;
   for (int i = 0; i < a.nstages; ++i) {
     const int R = a.st[i].R;
-    w += R >= kMixMinDirect ? R / 4.0 : std::log2(double(R));
+    w += i < a.ndirect ? R / 4.0 : std::log2(double(R));
   }
   return double(a.T) * a.L * (w + 2.0);
 }

@@ -298,7 +298,7 @@ __device__ __forceinline__ void mix_stage(C* sm, const MixDesc& a, const MixStag
   __syncthreads();
 }
 
-// ---- a prime radix R >= 17, in the order of a primitive root g of R.  With
+// ---- a prime radix R >= 11, in the order of a primitive root g of R.  With
 // x'_r the twiddled inputs, h = (R - 1) / 2 and r_m = g^m mod R, so that
 // R - r_m = r_{m+h}, a pre-pass stores a_m = x'_{r_m} + x'_{R - r_m} and b_m =
 // x'_{r_m} - x'_{R - r_m} at slots 1 + m and 1 + h + m of the butterfly (slot 0
@@ -472,13 +472,10 @@ __device__ __forceinline__ void mix_stages_of4(C* sm, const MixDesc& a, int& i, 
 
 template <typename C>
 __device__ __forceinline__ void mix_stages(C* sm, const MixDesc& a) {
-  int i = 0, R = a.nstages ? a.st[0].R : 0;
+  int i = 0;
 #pragma unroll 1
-  while (R >= kMixMinDirect) {
-    mix_direct<C>(sm, a, a.st[i]);
-    ++i;
-    R = i < a.nstages ? a.st[i].R : 0;
-  }
+  for (; i < a.ndirect; ++i) mix_direct<C>(sm, a, a.st[i]);
+  int R = i < a.nstages ? a.st[i].R : 0;
   mix_stages_of4<C, 15, 13, 11, 9>(sm, a, i, R);
   mix_stages_of4<C, 16, 14, 12, 10>(sm, a, i, R);
   mix_stages_of4<C, 8, 7, 6, 5>(sm, a, i, R);

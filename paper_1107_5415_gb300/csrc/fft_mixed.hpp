@@ -24,7 +24,8 @@ enum MixKind { MIX_ROW = 0, MIX_COL = 1, MIX_WHOLE = 2 };
 
 constexpr int kMixMaxStages = 16;
 constexpr int kMixPoints = 16;  // points a thread holds between the barriers of a stage, at most
-// Register butterflies reach radix 16; primes from 17 up are direct stages.
+// Register butterflies reach radix 16; primes from 17 up are direct stages, and so
+// are 11 and 13 in a complex128 pencil that needs more than 11 or 13 points a thread.
 constexpr int kMixMinDirect = 17;
 // Outputs pairs of one work item of a direct stage: kMixWide when every item
 // has a thread of its own, else kMixNarrow with at most kMixItems per thread.
@@ -74,7 +75,7 @@ struct alignas(16) MixDesc {
   int pitch_in, pitch_out;  // their distances of the rows
   const int *psin, *psout;  // row tiles: padded element position of each column position
   int dir_off;        // tables of the direct stages after the tile (elements)
-  int nstages;
+  int nstages, ndirect;  // the first ndirect stages are direct sums
   int tw_n;           // order of the root table
   int load_mode, store_mode, conj_in, conj_out;
   int in_sel, out_sel;  // grouped launches: in / out are byte offsets into base[in_sel] / base[out_sel]

@@ -223,15 +223,24 @@ int mix_points(int R) { return R * std::max(1, kMixPoints / R); }  // points a t
 // about 40 per butterfly for its indices, the butterfly and the twiddles
 // (operation counts of fft_mixed.cuh); a direct stage about 1.2 per unit of R
 // on top of its pre-pass.
-double radix_cost(int R) {
+double radix_cost(int R, bool direct = false) {
   static const double flops[17] = {0, 0, 4, 6.7, 8, 11.2, 11, 14.4, 13, 15.6, 15.2, 19.6, 14.3, 21.7, 17.7, 17.6, 16.8};
-  return R >= kMixMinDirect ? 40 + 1.2 * R : 8 + 40.0 / R + flops[R];
+  return direct ? 40 + 1.2 * R : 8 + 40.0 / R + flops[R];
 }
+
+// A radix and how its stages run: as register butterflies or as direct sums.
+struct Radix {
+  int R;
+  bool direct;
+};
 
 // Cheapest radices covering n (factors 2, 3, 5, 7, 11, 13 through the register
 // butterflies, larger primes as direct stages, smallest first and before all
-// others), every one taking at least min_points points per thread.  cost: the
-// sum of radix_cost.  False when n has no such cover.
+// others), every register radix taking at least min_points points per thread.
+// small_direct: 11 and 13, whose butterflies are 11 and 13 points, run as direct
+// stages where min_points is more: complex128 pencils of more than 5632 and 6656
+// points (512 threads), such as the columns of diag(77, 77, 77).  cost: the sum of
+// radix_cost.  False when n has no such cover.
 struct RadixCover {
   double cost;
   int R;  // first radix (0: none)
@@ -249,23 +258,24 @@ RadixCover cover_smooth(int n, int min_points, int max2, std::map<int, RadixCove
   memo[n] = best;
   return best;
 }
-bool mixed_radices(int n, int min_points, int max2, std::vector<int>& out, double* cost = nullptr) {
+bool mixed_radices(int n, int min_points, int max2, bool small_direct, std::vector<Radix>& out, double* cost = nullptr) {
   out.clear();
   double c = 0;
-  for (int p = kMixMinDirect; p <= kMaxDirectRadix && p <= n; p += 2) {
-    bool prime = p % 3 && p % 5 && p % 7 && p % 11 && p % 13;
+  for (int p = 11; p <= kMaxDirectRadix && p <= n; p += 2) {
+    if (p < kMixMinDirect && !(small_direct && mix_points(p) < min_points)) continue;
+    bool prime = p % 3 && p % 5 && p % 7 && (p == 11 || p % 11) && (p == 13 || p % 13);
     for (int q = 17; prime && q * q <= p; q += 2) prime = p % q != 0;
     if (!prime) continue;
     for (; n % p == 0; n /= p) {
-      out.push_back(p);
-      c += radix_cost(p);
+      out.push_back({p, true});
+      c += radix_cost(p, true);
     }
   }
   std::map<int, RadixCover> memo;
   for (int x = n; x > 1;) {
     const RadixCover r = cover_smooth(x, min_points, max2, memo);
     if (!r.R) return false;
-    out.push_back(r.R);
+    out.push_back({r.R, false});
     c += radix_cost(r.R);
     x /= r.R;
   }
@@ -277,11 +287,11 @@ bool mixed_radices(int n, int min_points, int max2, std::vector<int>& out, doubl
 int mix_min_points(int L, const pfft_plan_s& P) { return (L + mix_max_threads(P) - 1) / mix_max_threads(P); }
 
 // Threads of a mixed-radix tile of n points.
-int mix_threads(const std::vector<int>& radices, int n, int max_threads) {
+int mix_threads(const std::vector<Radix>& radices, int n, int max_threads) {
   int need = (n + kMixPoints - 1) / kMixPoints;
-  for (int R : radices) {
-    const int nbf = n / R;
-    if (R >= kMixMinDirect) {  // pre-pass pairs, then wide items or up to kMixItems narrow ones (mix_direct)
+  for (const Radix& r : radices) {
+    const int R = r.R, nbf = n / R;
+    if (r.direct) {  // pre-pass pairs, then wide items or up to kMixItems narrow ones (mix_direct)
       const int h = (R - 1) / 2;
       const int wide = nbf * ((h + kMixWide - 1) / kMixWide), narrow = nbf * ((h + kMixNarrow - 1) / kMixNarrow);
       need = std::max(need, (nbf * h + kMixPoints / 2 - 1) / (kMixPoints / 2));
@@ -295,12 +305,13 @@ int mix_threads(const std::vector<int>& radices, int n, int max_threads) {
 }
 
 // Whether a pencil of L points (one axis, or the axes of a column) fits a tile.
-bool mix_fits(const pfft_plan_s& P, const std::vector<int>& axes, int L, double* cost = nullptr) {
+bool mix_fits(const pfft_plan_s& P, const std::vector<int>& axes, int L, bool small_direct = false,
+              double* cost = nullptr) {
   if (L > (P.dtype == PFFT_C64 ? 16384 : 8192)) return false;
-  std::vector<int> all, rad;
+  std::vector<Radix> all, rad;
   double c = 0, ca = 0;
   for (int a : axes) {
-    if (!mixed_radices(a, mix_min_points(L, P), 16, rad, &ca)) return false;
+    if (!mixed_radices(a, mix_min_points(L, P), 16, small_direct, rad, &ca)) return false;
     all.insert(all.end(), rad.begin(), rad.end());
     c += ca;
   }
@@ -360,18 +371,18 @@ pfft_status mix_stages(pfft_plan_s& P, int kind) {
       axes.push_back({P.pen[s], sigma, 1});
       sigma *= P.pen[s];
     }
-  std::vector<std::pair<int, int>> order;  // (radix, axis)
-  std::vector<int> rad;
+  std::vector<std::pair<Radix, int>> order;  // (radix, axis)
+  std::vector<Radix> rad;
   for (size_t i = 0; i < axes.size(); ++i) {
-    if (!mixed_radices(axes[i].a, mix_min_points(L, P), P.max2, rad)) return PFFT_ERR_UNSUPPORTED;
-    for (int R : rad) order.push_back({R, int(i)});
+    if (!mixed_radices(axes[i].a, mix_min_points(L, P), P.max2, P.dtype == PFFT_C128, rad)) return PFFT_ERR_UNSUPPORTED;
+    for (const Radix& r : rad) order.push_back({r, int(i)});
   }
   if (order.size() > size_t(kMixMaxStages)) return PFFT_ERR_UNSUPPORTED;
-  std::stable_sort(order.begin(), order.end(), [](const std::pair<int, int>& x, const std::pair<int, int>& y) {
-    const bool dx = x.first >= kMixMinDirect, dy = y.first >= kMixMinDirect;
-    if (dx || dy) return dx != dy ? dx : x.first < y.first;
+  std::stable_sort(order.begin(), order.end(), [](const std::pair<Radix, int>& x, const std::pair<Radix, int>& y) {
+    const Radix &a = x.first, &b = y.first;
+    if (a.direct || b.direct) return a.direct != b.direct ? a.direct : a.R < b.R;
     auto rank = [](int R) { return std::find(kMixOrder, kMixOrder + 15, R) - kMixOrder; };
-    return rank(x.first) < rank(y.first);
+    return rank(a.R) < rank(b.R);
   });
   MixTableArgs t;
   std::memset(&t, 0, sizeof(t));
@@ -380,14 +391,15 @@ pfft_status mix_stages(pfft_plan_s& P, int kind) {
     Axis& ax = axes[o.second];
     MixStage s;
     std::memset(&s, 0, sizeof(s));
-    s.R = o.first;
+    s.R = o.first.R;
     s.aR = ax.a / s.R;
     s.sig = ax.sigma;
     s.Ns = ax.Ns;
     s.twstep = tw_n / (s.Ns * s.R);
     s.div_aR.init(uint32_t(s.aR));
     s.div_Ns.init(uint32_t(s.Ns));
-    if (s.R >= kMixMinDirect) {
+    if (o.first.direct) {
+      ++S.ndirect;
       s.gen = int(g.size());
       const int r = primitive_root(s.R);
       for (int e = 0, x = 1; e < s.R - 1; ++e, x = x * r % s.R) g.push_back(x);
@@ -419,9 +431,9 @@ pfft_status mix_stages(pfft_plan_s& P, int kind) {
       if (s.Ns == 1 && s.R % 2 == 0) R1 = s.R;
     if (P.fs_na == 1 && !S.st.empty()) {
       const int lanes = 128 / int(elem_bytes(P.dtype));
-      if (S.st[0].R < kMixMinDirect) S.ws_in = pad_unit(P.PIinv, S.st[0].aR, 0, lanes);
+      if (S.ndirect == 0) S.ws_in = pad_unit(P.PIinv, S.st[0].aR, 0, lanes);
       const MixStage& z = S.st.back();
-      if (z.R < kMixMinDirect) S.ws_out = pad_unit(P.PIinv, z.Ns, R1, lanes);
+      if (S.ndirect < int(S.st.size())) S.ws_out = pad_unit(P.PIinv, z.Ns, R1, lanes);
     }
     auto padded = [&](int unit, int** out) {
       if (!unit) return 0;
@@ -468,7 +480,8 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
   a.tw_n = kind == MIX_COL && P.tw_col ? P.col_n : P.nD;
   const int tstride = kind == MIX_COL || a.lay ? T : 1;  // stride of the pencil index in the tile
   a.nstages = int(S.st.size());
-  std::vector<int> rad;
+  a.ndirect = S.ndirect;
+  std::vector<Radix> rad;
   int rmax = 0;
   int unit = 0;  // pad unit, once padded
   for (int i = 0; i < a.nstages; ++i) {
@@ -493,8 +506,8 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
     s.div_sig.init(uint32_t(s.sig));
     s.div_nb.init(uint32_t(std::max(1, a.n / s.R)));
     a.st[i] = s;
-    rad.push_back(s.R);
-    if (s.R >= kMixMinDirect) rmax = std::max(rmax, s.R);
+    rad.push_back({s.R, i < a.ndirect});
+    if (i < a.ndirect) rmax = std::max(rmax, s.R);
   }
   a.nthreads = mix_threads(rad, a.n, max_threads);
   // a launch that leaves the chip idle gets twice the threads that its stages ask
@@ -790,8 +803,12 @@ pfft_status pfft::plan_host(pfft_plan_s& P, int d, const int64_t* Mv) {
   // and lambda_a becomes one more pencil axis of the column pass.
   const int row_max = P.dtype == PFFT_C64 ? 16384 : 8192;
   const i64 n = P.fs_N;
-  const bool split = n > 1 && (n > row_max || !(P.tc ? tc_tile_fits(int(n), row_max) : mix_fits(P, {int(n)}, int(n))));
-  if (split) {
+  // A cycle that fits only with radices 11 or 13 as direct stages is split if it
+  // can be without them, and stays whole if not; splits that need them come last.
+  const bool whole = n <= row_max && (P.tc ? tc_tile_fits(int(n), row_max) : mix_fits(P, {int(n)}, int(n)));
+  const bool small_direct = P.dtype == PFFT_C128;
+  const bool whole_direct = small_direct && !whole && n <= row_max && mix_fits(P, {int(n)}, int(n), true);
+  auto split_cycle = [&](bool direct) {
     const i64 other = P.m / n;
     int best = 0;
     double best_cost = 1e30;
@@ -813,7 +830,7 @@ pfft_status pfft::plan_host(pfft_plan_s& P, int d, const int64_t* Mv) {
       double cr = 0, cc = 0;
       std::vector<int> pen(P.pen.begin(), P.pen.end());
       pen.push_back(int(na));
-      if (!mix_fits(P, {int(nb)}, int(nb), &cr) || !mix_fits(P, pen, int(lb), &cc)) continue;
+      if (!mix_fits(P, {int(nb)}, int(nb), direct, &cr) || !mix_fits(P, pen, int(lb), direct, &cc)) continue;
       const int unit = P.dtype == PFFT_C64 ? 1024 : 512;
       auto long_tile = [&](i64 L) { return L > 8 * unit ? 60.0 : L > 4 * unit ? 30.0 : L > 2 * unit ? 12.0 : L > unit ? 3.0 : 0.0; };
       const double c = cr + cc + long_tile(nb) + long_tile(lb) + 3.0 * std::max<i64>(0, 8 - na);
@@ -822,10 +839,17 @@ pfft_status pfft::plan_host(pfft_plan_s& P, int d, const int64_t* Mv) {
         best = int(nb);
       }
     }
-    if (!best) return PFFT_ERR_UNSUPPORTED;
-    P.nD = best;
-    P.fs_na = int(n / best);
-    P.pen.push_back(P.fs_na);
+    return best;
+  };
+  if (n > 1 && !whole) {
+    int best = split_cycle(false);
+    if (!best && !whole_direct && small_direct) best = split_cycle(true);
+    if (!best && !whole_direct) return PFFT_ERR_UNSUPPORTED;
+    if (best) {
+      P.nD = best;
+      P.fs_na = int(n / best);
+      P.pen.push_back(P.fs_na);
+    }
   }
   if (P.pen.size() > size_t(kMaxSub)) return PFFT_ERR_UNSUPPORTED;
   P.LB = int(P.m / P.nD);

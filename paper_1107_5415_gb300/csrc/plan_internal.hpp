@@ -16,6 +16,7 @@
 struct MixStages {
   bool ready = false;
   std::vector<pfft::MixStage> st;  // sig, blk and the divisors of a tile are set with its T
+  int ndirect = 0;                 // the first ones, run as direct sums
   void* stw = nullptr;
   int* gtab = nullptr;
   int ws_in = 0, ws_out = 0;  // row tiles: pad units of the workspace side

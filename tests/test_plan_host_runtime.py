@@ -1,10 +1,13 @@
 """Host side of plan creation against a stand-in for the CUDA runtime
-(fake_cudart.cpp): what is still in flight when a plan is handed out."""
+(fake_cudart.cpp): what is still in flight when a plan is handed out, which
+kernels a call launches, which lengths have a plan; and on a GPU the calls that
+these decide."""
 import ctypes
 import os
 import shutil
 import subprocess
 
+import numpy as np
 import pytest
 import torch
 
@@ -88,6 +91,47 @@ def test_bulk_copies_only_where_they_are_aligned(fake, n, inverse):
         rows = fake.fake_kernel(1 if inverse else 0).decode()
         assert ("row_tma" in rows or "row_pipe" in rows) if bulk else "row_fast" in rows
     fake.pfft_plan_destroy(h)
+
+
+def test_complex128_cycles_with_factors_11_and_13(fake):
+    """Two equal cycles of n points, 11 or 13 dividing n: the row and the column
+    each take a tile of 512 threads, 16 points a thread, wherever the other
+    factors do (15 points in radices 3 and 5, 14 in radix 7)."""
+    tried = 0
+    for n in range(11 * 400, 8193):
+        if n % 11 and n % 13:
+            continue
+        primes = [p for p in range(2, 1022) if n % p == 0 and all(p % q for q in range(2, p))]
+        rest = n
+        for p in primes:
+            while rest % p == 0:
+                rest //= p
+        if rest > 1 or n > 512 * min([16] + [{3: 15, 5: 15, 7: 14}[p] for p in primes if p in (3, 5, 7)]):
+            continue
+        tried += 1
+        st, h = _create(fake, [[n, 0], [0, n]], 1, 1)
+        assert st == 0, n
+        fake.pfft_plan_destroy(h)
+    assert tried > 300
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,batch", [([[77, 0, 0], [0, 77, 0], [0, 0, 77]], 2),      # column 7 7 11 11
+                                     ([[26, 0, 0], [0, 286, 0], [0, 0, 286]], 1),   # column 2 2 11 13 13
+                                     ([[88, 0, 0], [0, 88, 0], [0, 0, 88]], 1),     # column 2^6 11 11
+                                     ([[6006, 0], [0, 6006]], 1)],                  # row and column
+                         ids=["77", "26-286", "88", "6006"])
+def test_complex128_direct_11_and_13(M, batch):
+    m = abs(L.det(M))
+    plan = pf.PatternFFT(M, batch, torch.complex128)
+    c = SI.complex_normal(batch, m, seed=m % 79, dtype=np.complex128)
+    y = plan.forward(torch.from_numpy(c).cuda())
+    yh = y.cpu().numpy()
+    slots = SI.sample_slots(m, 16 if m > 1 << 24 else 256, seed=3)
+    assert rel_l2(yh[:, slots], oracle.pattern_fft(M, c, out_slots=slots)) <= TOL["c128"]
+    assert rel_l2(plan.inverse(y).cpu().numpy(), c) <= TOL["c128"]
+    ref = oracle.pattern_fft(M, yh, inverse=True, out_slots=slots)
+    assert rel_l2(c[:, slots], ref) <= TOL["c128"]
 
 
 @pytest.mark.gpu
