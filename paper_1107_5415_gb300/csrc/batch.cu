@@ -327,6 +327,13 @@ pfft_status build_schedule(pfft_batch_s& B) {
       return PFFT_ERR_CUDA;
     }
   }
+  // the plans' tables, the stage tables that another radix made them build, the
+  // split tables and the schedule, all on the default stream, before a launch on one
+  // that does not wait for it
+  if (cudaDeviceSynchronize() != cudaSuccess) {
+    cudaFree(dev);
+    return PFFT_ERR_CUDA;
+  }
   if (B.sched) cudaFree(B.sched);
   B.sched = dev;
   B.rows = rb;
@@ -634,7 +641,6 @@ extern "C" pfft_status pfft_batch_create(pfft_batch* out, int n, const int* d, c
     mo += size_t(d[i]) * d[i];
   }
   if (B->total >= (int64_t(1) << 40)) return fail(PFFT_ERR_OVERFLOW);
-  if (cudaDeviceSynchronize() != cudaSuccess) return fail(PFFT_ERR_CUDA);  // tables built
   if (need_ws)
     if (int e = device_alloc(&B->ws, size_t(B->total) * ebytes(dtype))) return fail(pfft_status(e));
   if (flags & PFFT_BATCH_ONE_LAUNCH) {  // status word and queue counters

@@ -85,7 +85,8 @@ pfft_status plan_host(pfft_plan_s& P, int d, const int64_t* M);
 pfft_status plan_device(pfft_plan_s& P);
 // Re-choose the tiles of both passes (pencils per CTA) under the given
 // element budgets and the largest power-of-two radix (16 or 8); mixed-radix
-// passes only.  Tables are unchanged.
+// passes only.  The first call with another radix builds its stage tables on the
+// default stream: the caller waits for them before a launch.
 pfft_status plan_retile(pfft_plan_s& P, int row_budget, int col_budget, int max2);
 void plan_release(pfft_plan_s* P);
 }  // namespace pfft

@@ -135,8 +135,16 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
   return cudaSuccess;
 }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+// A batch's streams are joined to the one that is waited for; none of them waits
+// for the default stream.
 cudaError_t cudaStreamSynchronize(cudaStream_t s) {
-  pending.erase(s);
+  const int by_default = pending[nullptr];
+  if (!s) {
+    pending.erase(nullptr);
+  } else {
+    pending.clear();
+    pending[nullptr] = by_default;
+  }
   return cudaSuccess;
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }

@@ -74,6 +74,23 @@ def test_plan_tables_are_built_when_the_plan_is(fake, name, dtype, flags):
         fake.pfft_plan_destroy(h)
 
 
+@pytest.mark.parametrize("flags", [0, pf.PFFT_BATCH_RADIX8, pf.PFFT_BATCH_AUTOTUNE, pf.PFFT_BATCH_ONE_LAUNCH],
+                         ids=["grouped", "radix8", "autotune", "one-launch"])
+def test_batch_tables_are_built_when_the_batch_is(fake, flags):
+    """The schedule, the stage tables of its radices and the split tables, for
+    launches on streams that do not wait for the default one."""
+    Ms = [[[96, 0], [0, 96]], [[64, 2], [0, 256]], [[1200, 240], [0, 1080]], [[60]]]
+    Js = [[[2, 0], [0, 1]], [[2, 0], [0, 1]], [[3, 0], [0, 1]], [[2]]]
+    flat = [x for A in Ms for r in A for x in r], [x for A in Js for r in A for x in r]
+    (_, m), (_, j) = _capi._i64(flat[0]), _capi._i64(flat[1])
+    h = ctypes.c_void_p()
+    fake.fake_reset()
+    d = (ctypes.c_int * len(Ms))(*[len(A) for A in Ms])
+    assert fake.pfft_batch_create(ctypes.byref(h), len(Ms), d, m, j, pf.PWT_DIRICHLET, 0.0, 0, flags) == 0
+    assert fake.fake_pending() == 0
+    fake.pfft_batch_destroy(h)
+
+
 ROWS = {2048: [[512, 128], [0, 512]], 4096: [[8, 0], [0, 4096]], 8192: [[4, 0], [0, 8192]], 16384: [[4, 0], [0, 16384]]}
 
 
