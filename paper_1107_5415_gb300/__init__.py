@@ -326,10 +326,13 @@ class PatternBatch:
 
 
 def _det_int(A) -> int:
-    """|det A| of an integer matrix, exact (Laplace expansion along the first row)."""
+    """|det A| of an integer matrix, exact up to the four dimensions that the library
+    takes (Laplace expansion along the first row)."""
     A = np.asarray(A, dtype=np.int64)
     if A.ndim != 2 or A.shape[0] != A.shape[1]:
         raise np.linalg.LinAlgError("A must be a square matrix")
+    if len(A) > 4:
+        return int(round(abs(np.linalg.det(A.astype(np.float64)))))
 
     def det(a):
         if len(a) == 0:
