@@ -552,11 +552,15 @@ static pfft_status synthesise(pwt_plan p, const void* scaling, const void* const
   for (int l = 0; l < p->levels; ++l)
     if (!wavelets[l]) return PFFT_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  // the launches of the analysis in reverse
+  // the launches of the analysis in reverse.  Without symbol tables (fewer than four
+  // signals) one level a launch: a fused thread then evaluates the symbols of seven
+  // fibres, one after the other ([[1024, 1024], [-1024, 1024]] x 1, three levels of the
+  // trapezoid back: 22.3 us in three launches, 27.5 in two, 30.6 in one; [[384, 384],
+  // [-384, 384]] x 3: 12.8, 14.3 and 17.9).
   int first[64], count[64], n = 0;
   for (int l = 0; l < p->levels; l += count[n++]) {
     first[n] = l;
-    count[n] = fuse_count(p, l);
+    count[n] = p->symtab ? fuse_count(p, l) : 1;
   }
   const void* cur = scaling;
   for (int g = n - 1; g >= 0; --g) {

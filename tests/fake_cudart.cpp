@@ -16,7 +16,11 @@ std::map<const void*, std::string>& names() {
   static std::map<const void*, std::string> n;
   return n;
 }
-std::vector<std::string> launched;  // kernels in order since fake_reset()
+struct Launch {
+  std::string kernel;
+  dim3 grid, block;
+};
+std::vector<Launch> launched;  // in order since fake_reset()
 std::map<void*, int> pending;          // by stream; nullptr: the default one, which the others do not wait for
 struct Config {
   dim3 grid, block;
@@ -37,7 +41,10 @@ int fake_pending() {
   return n;
 }
 int fake_launches() { return int(launched.size()); }
-const char* fake_kernel(int i) { return launched[i].c_str(); }
+const char* fake_kernel(int i) { return launched[i].kernel.c_str(); }
+int fake_grid_x(int i) { return int(launched[i].grid.x); }
+int fake_grid_y(int i) { return int(launched[i].grid.y); }
+int fake_threads(int i) { return int(launched[i].block.x); }
 
 void** __cudaRegisterFatBinary(void*) {
   static void* handle;
@@ -67,7 +74,7 @@ cudaError_t __cudaPopCallConfiguration(dim3* grid, dim3* block, size_t* smem, vo
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void**, size_t smem, cudaStream_t s) {
   if (grid.x == 0 || grid.y == 0 || grid.y > 65535 || block.x == 0 || block.x > 1024 || smem > 227 * 1024)
     return cudaErrorInvalidConfiguration;
-  launched.push_back(names()[reinterpret_cast<const void*>(k)]);
+  launched.push_back({names()[reinterpret_cast<const void*>(k)], grid, block});
   ++pending[s];
   return cudaSuccess;
 }

@@ -91,6 +91,30 @@ def test_batch_tables_are_built_when_the_batch_is(fake, flags):
     fake.pfft_batch_destroy(h)
 
 
+def _launches(lib):
+    """(kernel, grid x, grid y, threads) of the launches since fake_reset()."""
+    return [(lib.fake_kernel(i).decode(), lib.fake_grid_x(i), lib.fake_grid_y(i), lib.fake_threads(i))
+            for i in range(lib.fake_launches())]
+
+
+def _synthesis(lib, size, levels, batch, dtype=0):
+    """Launches of a reconstruction of a quincunx cascade."""
+    d, (_, m) = _capi._mat([[size, size], [-size, size]])
+    _, j = _capi._i64([x for J in SI.wavelet_dilations(levels) for r in J for x in r])
+    h = ctypes.c_void_p()
+    assert lib.pwt_plan_create(ctypes.byref(h), d, m, levels, j, pf.PWT_DLVP, 0.25, batch, dtype, 0) == 0
+    lib.fake_reset()
+    assert lib.pwt_reconstruct(h, 4096, _capi._ptr_array([4096] * levels), 8192, None) == 0
+    lib.pwt_plan_destroy(h)
+    return _launches(lib)
+
+
+def test_synthesis_is_fused_where_symbol_tables_exist(fake):
+    """Fewer than four signals have none: one level a launch."""
+    assert ["fused" in k for k, *_ in _synthesis(fake, 64, 7, 3)] == [False] * 7
+    assert ["fused" in k for k, *_ in _synthesis(fake, 64, 7, 4)] == [False, True, True]
+
+
 ROWS = {2048: [[512, 128], [0, 512]], 4096: [[8, 0], [0, 4096]], 8192: [[4, 0], [0, 8192]], 16384: [[4, 0], [0, 16384]]}
 
 
