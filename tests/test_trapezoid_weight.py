@@ -10,7 +10,7 @@ def _sum(t, q, eta, odd):
     u = F(0)
     for n in range(-3, 2):
         b = (F(1, 2) * (1 + eta) - abs(F(t, q) + n)) / eta
-        u += min(max(b, F(0)), F(1)) * (-1) ** (odd * n)
+        u += min(max(b, F(0)), F(1)) * (-1 if odd * n % 2 else 1)
     return u
 
 
