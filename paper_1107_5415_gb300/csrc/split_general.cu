@@ -97,8 +97,11 @@ __global__ void __launch_bounds__(256) split_general_kernel(GeneralDesc G, int b
 }
 
 // Built-in band system (split_prime.cuh): one work item per fibre and chunk
-// of band outputs, blockIdx.y the signal.  parts: [p][batch][mN].
-template <typename C, int MODE>
+// of band outputs, blockIdx.y the signal.  parts: [p][batch][mN].  WIDE: primes and
+// numerators beyond the multiply-high path (P.small = 0), in a kernel of its own:
+// beside the small fibres' code its loop took 5 to 13% more ([[16424, 0, 0], [0, 64,
+// 0], [0, 0, 128]] x 8 by diag(2053, 1, 1), merged: 14.7 against 13.0 ms).
+template <typename C, int MODE, bool WIDE>
 __global__ void __launch_bounds__(256) split_prime_kernel(PrimeDesc P, int batch, const C* __restrict__ cin,
                                                           C* __restrict__ cout, const C* __restrict__ din,
                                                           C* __restrict__ dout) {
@@ -109,11 +112,29 @@ __global__ void __launch_bounds__(256) split_prime_kernel(PrimeDesc P, int batch
        w += (long long)gridDim.x * blockDim.x) {
     const int ch = int(w / P.mN), gs = int(w - (long long)ch * P.mN);
     const long long off = (long long)b * P.mN + gs;
-    prime_item<C, MODE>(P, gs, ch * kPrimeChunk, MODE == 0 ? cin + (long long)b * P.mM : nullptr,
-                        MODE == 0 ? nullptr : cout + (long long)b * P.mM, MODE == 0 ? nullptr : din + off,
-                        MODE == 0 ? nullptr : din + off + dstride, MODE == 0 ? dout + off : nullptr,
-                        MODE == 0 ? dout + off + dstride : nullptr, dstride);
+    const C* ci = MODE == 0 ? cin + (long long)b * P.mM : nullptr;
+    C* co = MODE == 0 ? nullptr : cout + (long long)b * P.mM;
+    const C *d0 = MODE == 0 ? nullptr : din + off, *dw = MODE == 0 ? nullptr : din + off + dstride;
+    C *o0 = MODE == 0 ? dout + off : nullptr, *ow = MODE == 0 ? dout + off + dstride : nullptr;
+    if constexpr (WIDE)
+      prime_split_item<C, MODE>(P, gs, ch * kPrimeChunk, ci, co, d0, dw, o0, ow, dstride);
+    else
+      prime_item<C, MODE>(P, gs, ch * kPrimeChunk, ci, co, d0, dw, o0, ow, dstride);
   }
+}
+
+template <typename C>
+static void launch_prime(const PrimeDesc& P, dim3 grid, int batch, int mode, const void* src, void* dst, cudaStream_t s) {
+  const C* in = static_cast<const C*>(src);
+  C* out = static_cast<C*>(dst);
+  if (mode == 0 && P.small)
+    split_prime_kernel<C, 0, false><<<grid, 256, 0, s>>>(P, batch, in, nullptr, nullptr, out);
+  else if (mode == 0)
+    split_prime_kernel<C, 0, true><<<grid, 256, 0, s>>>(P, batch, in, nullptr, nullptr, out);
+  else if (P.small)
+    split_prime_kernel<C, 1, false><<<grid, 256, 0, s>>>(P, batch, nullptr, out, in, nullptr);
+  else
+    split_prime_kernel<C, 1, true><<<grid, 256, 0, s>>>(P, batch, nullptr, out, in, nullptr);
 }
 
 // Small primes on the int32 index path: one thread per fibre, which keeps its
@@ -369,23 +390,10 @@ static pfft_status prime_run(int mode, int d, const int64_t* M, const int64_t* J
   const long long cap = (152LL * 16 + batch - 1) / batch;
   if (gx > cap) gx = cap;
   dim3 grid(unsigned(gx < 1 ? 1 : gx), unsigned(batch));
-  if (dtype == PFFT_C64) {
-    using C = float2;
-    if (mode == 0)
-      split_prime_kernel<C, 0><<<grid, blk, 0, s>>>(P, int(batch), static_cast<const C*>(src), nullptr, nullptr,
-                                                     static_cast<C*>(dst));
-    else
-      split_prime_kernel<C, 1><<<grid, blk, 0, s>>>(P, int(batch), nullptr, static_cast<C*>(dst),
-                                                     static_cast<const C*>(src), nullptr);
-  } else {
-    using C = double2;
-    if (mode == 0)
-      split_prime_kernel<C, 0><<<grid, blk, 0, s>>>(P, int(batch), static_cast<const C*>(src), nullptr, nullptr,
-                                                     static_cast<C*>(dst));
-    else
-      split_prime_kernel<C, 1><<<grid, blk, 0, s>>>(P, int(batch), nullptr, static_cast<C*>(dst),
-                                                     static_cast<const C*>(src), nullptr);
-  }
+  if (dtype == PFFT_C64)
+    launch_prime<float2>(P, grid, int(batch), mode, src, dst, s);
+  else
+    launch_prime<double2>(P, grid, int(batch), mode, src, dst, s);
   return cudaGetLastError() == cudaSuccess ? PFFT_OK : PFFT_ERR_CUDA;
 }
 

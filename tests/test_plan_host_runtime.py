@@ -115,6 +115,25 @@ def test_synthesis_is_fused_where_symbol_tables_exist(fake):
     assert ["fused" in k for k, *_ in _synthesis(fake, 64, 7, 4)] == [False, True, True]
 
 
+def _band_kernel(lib, p, mode, dtype=0):
+    """The kernel that splits (0) or merges (1) a pattern by diag(p, 1)."""
+    d, (_, m) = _capi._mat([[8 * p, 0], [0, 64]])
+    _, j = _capi._i64([p, 0, 0, 1])
+    lib.fake_reset()
+    f = lib.pwt_merge_general if mode else lib.pwt_split_general
+    assert f(d, m, j, 4, dtype, None, 4096, 8192, None) == 0
+    (k, *_), = _launches(lib)
+    return k
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["split", "merge"])
+def test_large_primes_run_in_a_kernel_of_their_own(fake, mode):
+    """Beside the code of the small fibres their loop is slower."""
+    assert "split_prime_small" in _band_kernel(fake, 5, mode)
+    small, wide = _band_kernel(fake, 1021, mode), _band_kernel(fake, 1031, mode)
+    assert "split_prime_kernel" in small and "split_prime_kernel" in wide and small != wide
+
+
 ROWS = {2048: [[512, 128], [0, 512]], 4096: [[8, 0], [0, 4096]], 8192: [[4, 0], [0, 8192]], 16384: [[4, 0], [0, 16384]]}
 
 
