@@ -134,6 +134,12 @@ def test_large_primes_run_in_a_kernel_of_their_own(fake, mode):
     assert "split_prime_kernel" in small and "split_prime_kernel" in wide and small != wide
 
 
+def test_fibres_of_seven_in_registers_where_they_fit(fake):
+    """A split by seven in double precision takes the chunks of the larger primes."""
+    assert "split_prime_small" in _band_kernel(fake, 7, 0) and "split_prime_small" in _band_kernel(fake, 7, 1, 1)
+    assert "split_prime_kernel" in _band_kernel(fake, 7, 0, 1)
+
+
 ROWS = {2048: [[512, 128], [0, 512]], 4096: [[8, 0], [0, 4096]], 8192: [[4, 0], [0, 8192]], 16384: [[4, 0], [0, 16384]]}
 
 
