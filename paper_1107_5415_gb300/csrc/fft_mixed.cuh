@@ -311,6 +311,14 @@ __device__ __forceinline__ void mix_stage(C* sm, const MixDesc& a, const MixStag
 // three shared-memory reads for 4 Q multiply-adds (in 2 Q packed instructions);
 // the reads bound it, hence the wide items wherever every item has a thread (six
 // pairs: eight spill, 2.36 against 2.33 ms for the mix below).
+//
+// In complex128 the two multiply-adds a clock of an SM bound it.  Items of four
+// pairs pad h less; y_0 is summed by the first item of a butterfly alone, after its
+// pairs (two additions beside sixteen multiply-adds in the step of every item were an
+// eighth of the work); and the planner picks the threads and pencils whose warps the
+// schedulers share evenly (direct_time of fft_plan.cu).  [[1021, 0], [0, 1021]] x 4, one
+// direction: 17.75 ms with six pairs an item and y_0 in each, 14.58 now (0.95 of the
+// multiply-add rate); a mix of 256 patterns of sides up to 512: 10.2 -> 9.4 ms.
 template <typename C>
 __device__ __forceinline__ void mix_locate(const MixStage& s, int b, int& base, int& j, int& k) {
   const int t = s.div_sig.div(b), low = b - t * s.sig;
@@ -360,12 +368,17 @@ __device__ __noinline__ void mix_direct_pairs(C* sm, const MixStage& s, int nbf,
         const C av = *pa, bv = *pb;
         pa += istep;
         pb += istep;
-        y0[u] = bsum<true>(y0[u], av);
+        if constexpr (sizeof(C) == 8) y0[u] = bsum<true>(y0[u], av);
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
           A[u][i] = cfma_r(av, wv[i].x, A[u][i]);
           B[u][i] = cfma_r(bv, wv[i].y, B[u][i]);
         }
+      }
+      if (sizeof(C) == 16 && blk == 0) {
+        pa = sm + base + j * s.sig + istep;
+#pragma unroll 4
+        for (int m = 0; m < h; ++m, pa += istep) y0[u] = cadd(y0[u], *pa);
       }
       ob[u] = base + ((j - k) * R + k) * s.sig;
       n0[u] = blk * Q;
@@ -440,8 +453,9 @@ __device__ __noinline__ void mix_direct(C* sm, const MixDesc& a, const MixStage&
       }
     __syncthreads();
   }
-  if (nbf * ((h + kMixWide - 1) / kMixWide) <= nthr)
-    mix_direct_pairs<C, 1, kMixWide>(sm, s, nbf, P, gp);
+  constexpr int W = sizeof(C) == 8 ? kMixWide : kMixNarrow;
+  if (nbf * ((h + W - 1) / W) <= nthr)
+    mix_direct_pairs<C, 1, W>(sm, s, nbf, P, gp);
   else
     mix_direct_pairs<C, kMixItems, kMixNarrow>(sm, s, nbf, P, gp);
 }

@@ -27,8 +27,9 @@ constexpr int kMixPoints = 16;  // points a thread holds between the barriers of
 // Register butterflies reach radix 16; primes from 17 up are direct stages, and so
 // are 11 and 13 in a complex128 pencil that needs more than 11 or 13 points a thread.
 constexpr int kMixMinDirect = 17;
-// Outputs pairs of one work item of a direct stage: kMixWide when every item
-// has a thread of its own, else kMixNarrow with at most kMixItems per thread.
+// Output pairs of one work item of a direct stage: kMixWide when every item
+// has a thread of its own, else kMixNarrow with at most kMixItems per thread;
+// kMixNarrow either way in complex128 (mix_direct_pairs).
 constexpr int kMixWide = 6, kMixNarrow = 4, kMixItems = 3;
 // Order in which the stages of the register radices run (mix_stages).
 constexpr int kMixOrder[15] = {15, 13, 11, 9, 16, 14, 12, 10, 8, 7, 6, 5, 4, 3, 2};

@@ -286,22 +286,49 @@ bool mixed_radices(int n, int min_points, int max2, bool small_direct, std::vect
 // Points per thread that every stage of a pencil of L points must reach.
 int mix_min_points(int L, const pfft_plan_s& P) { return (L + mix_max_threads(P) - 1) / mix_max_threads(P); }
 
+// Time of the direct stages of a complex128 tile of n points with t threads, per
+// SM: their multiply-adds bound it, so it is the turns that the busiest of the
+// SM's four schedulers gives to warps with items, over the tiles resident at a time
+// (128 registers a thread).  Tiles of a multiple of four warps put the warps of a
+// last, partial turn on the same schedulers, others spread them.  A tile alone on
+// its SM loads and stores beside no other's sums (4%).
+double direct_time(const std::vector<Radix>& radices, int n, int t) {
+  const int tiles = kMixThreadsC128 / t, per_tile = t / 32;
+  double time = 0;
+  for (const Radix& r : radices) {
+    if (!r.direct) continue;
+    const int h = (r.R - 1) / 2, items = n / r.R * ((h + kMixNarrow - 1) / kMixNarrow);
+    for (int left = items; left > 0; left -= t) {
+      const int warps = (std::min(left, t) + 31) / 32;
+      time += double(h) * (per_tile % 4 ? (tiles * warps + 3) / 4 : tiles * ((warps + 3) / 4));
+    }
+  }
+  return time / tiles * (tiles == 1 ? 1.04 : 1.0);
+}
+
 // Threads of a mixed-radix tile of n points.
-int mix_threads(const std::vector<Radix>& radices, int n, int max_threads) {
+int mix_threads(const std::vector<Radix>& radices, int n, int max_threads, int dtype) {
   int need = (n + kMixPoints - 1) / kMixPoints;
+  bool sums = false;
   for (const Radix& r : radices) {
     const int R = r.R, nbf = n / R;
     if (r.direct) {  // pre-pass pairs, then wide items or up to kMixItems narrow ones (mix_direct)
       const int h = (R - 1) / 2;
       const int wide = nbf * ((h + kMixWide - 1) / kMixWide), narrow = nbf * ((h + kMixNarrow - 1) / kMixNarrow);
       need = std::max(need, (nbf * h + kMixPoints / 2 - 1) / (kMixPoints / 2));
-      need = std::max(need, wide <= max_threads ? wide : (narrow + kMixItems - 1) / kMixItems);
+      need = std::max(need, dtype == PFFT_C64 && wide <= max_threads ? wide : (narrow + kMixItems - 1) / kMixItems);
+      sums = true;
     } else {
       const int nb = std::max(1, kMixPoints / R);
       need = std::max(need, (nbf + nb - 1) / nb);
     }
   }
-  return (need + 31) / 32 * 32;
+  need = (need + 31) / 32 * 32;
+  if (dtype == PFFT_C64 || !sums) return need;
+  int best = need;
+  for (int t = need; t <= max_threads; t += 32)
+    if (direct_time(radices, n, t) <= direct_time(radices, n, best)) best = t;
+  return best;
 }
 
 // Whether a pencil of L points (one axis, or the axes of a column) fits a tile.
@@ -316,7 +343,7 @@ bool mix_fits(const pfft_plan_s& P, const std::vector<int>& axes, int L, bool sm
     c += ca;
   }
   if (cost) *cost = c;
-  return int(all.size()) <= kMixMaxStages && mix_threads(all, L, mix_max_threads(P)) <= mix_max_threads(P);
+  return int(all.size()) <= kMixMaxStages && mix_threads(all, L, mix_max_threads(P), P.dtype) <= mix_max_threads(P);
 }
 
 // Pad unit u (element x at x + x / u) under which a walk over the elements in the
@@ -509,7 +536,7 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
     rad.push_back({s.R, i < a.ndirect});
     if (i < a.ndirect) rmax = std::max(rmax, s.R);
   }
-  a.nthreads = mix_threads(rad, a.n, max_threads);
+  a.nthreads = mix_threads(rad, a.n, max_threads, P.dtype);
   // a launch that leaves the chip idle gets twice the threads that its stages ask
   // for, as long as all of it stays resident: half the turns of every load and store
   const int more = (a.n + kMixFewPoints - 1) / kMixFewPoints;
@@ -559,6 +586,8 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
 // 1472], [0, 2048]] x 3: 0.414 and 0.365 ms; [[96, 87, 0], [0, 375, 201], [0, 0,
 // 243]] x 7, two columns of 3240 points in 544 threads: 3.60 and 3.24; a mix of 512
 // patterns: 2.14 and 2.11; but two of 3850 points in 704 threads lose 7%).
+// Complex128 tiles with direct sums hold another number of pencils, up to `most`
+// points, where that takes the launch at least 3% less by direct_time.
 pfft_status mix_choose(pfft_plan_s& P, int kind, int cap, int budget, int most, int lanes, int ctas) {
   pfft_status st = mix_stages(P, kind);
   if (st != PFFT_OK) return st;
@@ -571,6 +600,26 @@ pfft_status mix_choose(pfft_plan_s& P, int kind, int cap, int budget, int most, 
     const bool few = (count + 2 * T - 1) / (2 * T) * signals < ctas;
     if (n > (2 * T <= lanes ? std::max(most, budget) : budget) || (few && 2 * T > lanes && n > 256)) break;
     T *= 2;
+  }
+  const MixStages& S = P.stages[P.max2 == 16 ? 0 : 1][kind];
+  if (P.dtype == PFFT_C128 && S.ndirect) {
+    std::vector<Radix> rad;
+    for (int i = 0; i < int(S.st.size()); ++i) rad.push_back({S.st[i].R, i < S.ndirect});
+    auto time = [&](int x) {  // a pencil
+      return mix_configure(P, kind, x) == PFFT_OK ? direct_time(rad, x * L, P.mix[kind].nthreads) / x : 1e30;
+    };
+    // adjacent columns first as many as there may be, rows and signals as above
+    int best = T;
+    double least = lanes > 1 ? 1e30 : time(T);
+    for (int x = 16; x >= 1; x /= 2) {
+      if (x > cap || x > count || (x > 1 && (i64(x) * L > most || (count + x - 1) / x * signals < ctas))) continue;
+      const double c = time(x);
+      if (c < 0.97 * least) {
+        least = c;
+        best = x;
+      }
+    }
+    return mix_configure(P, kind, best);
   }
   for (;; T /= 2) {
     st = mix_configure(P, kind, T);

@@ -200,6 +200,36 @@ def test_complex128_direct_11_and_13(M, batch):
     assert rel_l2(c[:, slots], ref) <= TOL["c128"]
 
 
+@pytest.mark.parametrize("n,batch", [(1021, 4), (1004, 8), (1124, 1), (727, 4)])
+def test_complex128_direct_sums_share_an_sm(fake, n, batch):
+    """A tile of direct sums has its SM alone only when it must: at 128 registers a
+    thread, 256 threads leave room for a second one."""
+    st, h = _create(fake, [[n, 0], [0, n]], batch, 1)
+    assert st == 0
+    fake.fake_reset()
+    assert fake.pfft_forward(h, 4096, 8192, None) == 0
+    assert [t <= 256 for *_, t in _launches(fake)] == [True, True]
+    fake.pfft_plan_destroy(h)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.complex64, torch.complex128], ids=["c64", "c128"])
+@pytest.mark.parametrize("M,batch", [([[37, 0], [0, 74]], 5), ([[101, 0], [0, 101]], 3), ([[281, 0], [0, 1124]], 1),
+                                     ([[997]], 5), ([[643, 0], [0, 283]], 2), ([[1021, 0], [0, 127]], 1),
+                                     ([[17, 0], [0, 323]], 2), ([[29, 1], [0, 4 * 29 * 31]], 1)],
+                         ids=["37", "101", "281", "997", "643-283", "1021-127", "17-19", "29-31"])
+def test_direct_sums(M, batch, dtype):
+    """One to three turns of items, one to sixteen pencils a tile."""
+    m = abs(L.det(M))
+    plan = pf.PatternFFT(M, batch, dtype)
+    tol = TOL["c64" if dtype == torch.complex64 else "c128"]
+    c = SI.complex_normal(batch, m, seed=m % 73, dtype=np.complex64 if dtype == torch.complex64 else np.complex128)
+    y = plan.forward(torch.from_numpy(c).cuda())
+    slots = SI.sample_slots(m, min(m, 512), seed=3)
+    assert rel_l2(y.cpu().numpy()[:, slots], oracle.pattern_fft(M, c, out_slots=slots)) <= tol
+    assert rel_l2(plan.inverse(y).cpu().numpy(), c) <= tol
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n", ROWS)
 def test_transform_of_a_view_aligned_to_one_element(n):
