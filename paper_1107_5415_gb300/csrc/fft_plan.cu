@@ -944,10 +944,42 @@ static pfft_status mix_tile(pfft_plan_s& P, int kind, int budget, int ctas) {
                     ctas);
 }
 
+// Whether whole signals share tiles: one launch, no workspace.  Two tiles of 8192
+// complex64 (4096 complex128) points share an SM; one of twice that takes the SM,
+// worth it once the batch alone nearly fills the chip, as two passes use more SMs.
+// The register-resident passes are the better ones, one direction in us against
+// whole tiles,
+//   for a single complex64 cycle: 1024 points x 4096 signals 15.0 and 21.6, 4096 x 512
+//     12.1 and 13.8, 8192 x 16 8.2 and 10.8 (but 2048 x 64 5.8 and 5.3, 512 x 2048 4%
+//     apart), so from 4096 points on, or from 1024 in more than two signals an SM;
+//   for a batch that leaves a third of the chip idle, both passes resident: [[128, 0],
+//     [0, 128]] x 64 12.5 and 17.1 (x 100: 13% apart, x 152: whole tiles by 6%); in
+//     complex128 above 2048 points [[64, 0], [0, 64]] x 1 39 and 47 (x 100: 2% apart);
+//   for more than 4096 complex128 points, one such pass being enough: [[64, 0], [0,
+//     128]] x 64 54 and 99, x 200 147 and 197, x 512 338 and 406; [[16, 0, 0], [0, 16,
+//     0], [0, 0, 32]] x 64 54 and 94, x 512 333 and 383 (x 152 and x 304: whole tiles by
+//     5%).
+static bool whole_tile(const pfft_plan_s& P, int resident) {
+  const bool c64 = P.dtype == PFFT_C64;
+  const i64 half = c64 ? 8192 : 4096;
+  std::vector<int> axes(P.pen.begin(), P.pen.end());
+  axes.push_back(P.nD);
+  if (P.m > 2 * half || !mix_fits(P, axes, int(P.m))) return false;
+  const i64 most_sms = 2 * i64(P.nsm) / 3;
+  if (P.pen.empty()) {
+    if (resident && c64 && (P.m >= 4096 || (P.m >= 1024 && P.batch > 2 * i64(P.nsm)))) return false;
+  } else if (!c64) {
+    if (P.m > half ? resident > 0 : resident == 2 && P.m > half / 2 && P.batch < most_sms) return false;
+  }
+  return P.m <= half || P.batch >= (resident == 2 ? most_sms : 64);
+}
+
 pfft_status pfft::plan_device(pfft_plan_s& P) {
   const int d = P.d, D = P.D;
   if (cudaGetDevice(&P.device) != cudaSuccess) return PFFT_ERR_CUDA;
   if (D == 0) return PFFT_OK;  // m == 1: the transform is the identity
+  if (cudaDeviceGetAttribute(&P.nsm, cudaDevAttrMultiProcessorCount, P.device) != cudaSuccess || P.nsm < 1)
+    return PFFT_ERR_CUDA;
   // generators of the cycles
   std::vector<std::vector<i64>> g(D), h(D);
   for (int j = 0; j < D; ++j) {
@@ -1072,18 +1104,6 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
       if (launch_twiddles(P.tw_col, col_n, P.dtype, 0) != 0) return PFFT_ERR_CUDA;
     }
   }
-  // Whole signals in one tile: one launch, no workspace.  Up to 8192 complex64
-  // points two such tiles share an SM; up to 16384 one tile takes the SM, worth
-  // it once the batch alone nearly fills the chip (otherwise two passes use
-  // more SMs).
-  {
-    const i64 half = P.dtype == PFFT_C64 ? 8192 : 4096;
-    std::vector<int> axes(P.pen.begin(), P.pen.end());
-    axes.push_back(nD);
-    P.mixed[MIX_WHOLE] = !P.tc && na == 1 && P.m <= (P.batch >= 64 ? 2 * half : half) && mix_fits(P, axes, int(P.m));
-  }
-  if (npen >= 1 && P.own_workspace && !P.mixed[MIX_WHOLE])
-    if (int e_ = P.alloc(&P.ws, size_t(P.m) * P.batch * eb)) return pfft_status(e_);
   if (na > 1) {  // exp(-2 pi i t / n) for t < n, as lo[t & 2047] * hi[t >> 11]
     const int nhi = int((P.fs_N + 2047) >> 11);
     if (int e_ = P.alloc(&P.fs_tab, size_t(2048 + nhi) * eb)) return pfft_status(e_);
@@ -1192,26 +1212,21 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
   // is not split, whose box loads need no lanes across rows); the mixed-radix
   // ones everything else.
   auto no_pass = [](PassArgs& p) { p.fast = p.tc = 0; };
-  if (P.mixed[MIX_WHOLE]) {
-    no_pass(P.rowp);
-    no_pass(P.colp);
-  } else {
-    pfft_status st = PFFT_ERR_UNSUPPORTED;
-    if (P.tc || na == 1) st = choose_and_configure(P.rowp, P, false, 64, std::max(row_budget, nD));
-    if (st != PFFT_OK) {
-      if (P.tc) return st;
-      no_pass(P.rowp);
-      P.mixed[MIX_ROW] = true;
-    }
-    if (npen >= 1) {
-      st = choose_and_configure(P.colp, P, true, P.generic_only ? 512 : 16, std::max(budget, LB));
-      if (st != PFFT_OK) {
-        if (P.tc) return st;
-        no_pass(P.colp);
-        P.mixed[MIX_COL] = true;
-      }
-    }
+  {
+    pfft_status row = PFFT_ERR_UNSUPPORTED, col = PFFT_ERR_UNSUPPORTED;
+    if (P.tc || na == 1) row = choose_and_configure(P.rowp, P, false, 64, std::max(row_budget, nD));
+    if (npen >= 1) col = choose_and_configure(P.colp, P, true, P.generic_only ? 512 : 16, std::max(budget, LB));
+    if (P.tc && row != PFFT_OK) return row;
+    if (P.tc && npen >= 1 && col != PFFT_OK) return col;
+    const int resident = (row == PFFT_OK) + (col == PFFT_OK);  // register-resident passes
+    P.mixed[MIX_WHOLE] = !P.tc && na == 1 && whole_tile(P, resident);
+    P.mixed[MIX_ROW] = !P.mixed[MIX_WHOLE] && row != PFFT_OK;
+    P.mixed[MIX_COL] = !P.mixed[MIX_WHOLE] && npen >= 1 && col != PFFT_OK;
+    if (P.mixed[MIX_WHOLE] || P.mixed[MIX_ROW]) no_pass(P.rowp);
+    if (P.mixed[MIX_WHOLE] || P.mixed[MIX_COL]) no_pass(P.colp);
   }
+  if (npen >= 1 && P.own_workspace && !P.mixed[MIX_WHOLE])
+    if (int e_ = P.alloc(&P.ws, size_t(P.m) * P.batch * eb)) return pfft_status(e_);
   for (int kind = 0; kind < 3; ++kind) {
     if (!P.mixed[kind]) continue;
     MixDesc& a = P.mix[kind];
@@ -1367,9 +1382,6 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
         const int x_off = (s_el + 15) & ~15;
         const int stw_off = (x_off + kPipeX + 15) & ~15;
         const int bar_off = ((stw_off + P.rowp.stw_n) * 8 + 15) & ~15;
-        int nsm = 0;
-        if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, P.device) != cudaSuccess || nsm < 1)
-          return PFFT_ERR_CUDA;
         if (bar_off + 16 <= 227 * 1024) {
           // outputs stored from registers: the workspace when the permutation
           // multiplier is 1 and lanes form runs of >= 4 elements (32 B); the
@@ -1392,7 +1404,7 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
           P.rowp.pipe_lrun = lrun;
           P.rowp.pipe = 1;
           P.rowp.pipe_x_off = x_off;
-          P.rowp.pipe_grid = nsm;
+          P.rowp.pipe_grid = P.nsm;
           P.rowp.stw_smem_off = stw_off;
           P.rowp.bar_smem_off = bar_off;
           P.rowp.smem_bytes = bar_off + 16;
@@ -1407,9 +1419,6 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
                        P.colp.fast_tail == 2;
   if ((cpipe10 || cpipe11) && P.dtype == PFFT_C64 && !P.tc && P.colp.fast && P.colp.LB == P.colp.L &&
       P.colp.nthreads == 256 && P.colp.fast_nmain == 2 && (d == 2 || d == 3) && P.nD % P.colp.T == 0) {
-    int nsm = 0;
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, P.device) != cudaSuccess || nsm < 1)
-      return PFFT_ERR_CUDA;
     const int e_off = kCPipeS + kCPipeX;  // 2 x 8 column points of up to 4 int32: 32 elements
     const int stw_off = e_off + 32;
     const int bytes = (stw_off + P.colp.stw_n) * 8;
@@ -1417,7 +1426,7 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
       P.colp.cpipe = 1;
       P.colp.cpipe_x_off = kCPipeS;
       P.colp.cpipe_e_off = e_off;
-      P.colp.cpipe_grid = 2 * nsm;
+      P.colp.cpipe_grid = 2 * P.nsm;
       P.colp.stw_smem_off = stw_off;
       P.colp.smem_bytes = bytes;
     }

@@ -48,6 +48,7 @@ struct pfft_plan_s {
   int max2 = 16;                 // largest power-of-two radix of the mixed-radix passes (16 or 8)
   // device state
   int device = 0;
+  int nsm = 0;  // multiprocessors
   int* dtab = nullptr;
   void* tw = nullptr;
   int col_n = 0;           // order of tw_col

@@ -159,6 +159,40 @@ def test_bulk_copies_only_where_they_are_aligned(fake, n, inverse):
     fake.pfft_plan_destroy(h)
 
 
+# matrix, signals, complex128, whole signals in one tile
+WHOLE = [([[512]], 4096, 0, True), ([[1024]], 304, 0, True), ([[1024]], 305, 0, False), ([[4096]], 1, 0, False),
+         ([[16384]], 70, 0, False), ([[8192]], 1, 0, False), ([[4096]], 1, 1, True), ([[90, 0], [0, 90]], 1, 0, True),
+         ([[64, 0], [0, 128]], 1, 0, True), ([[128, 0], [0, 128]], 100, 0, False), ([[128, 0], [0, 128]], 101, 0, True),
+         ([[120, 0], [0, 120]], 64, 0, True), ([[120, 0], [0, 120]], 63, 0, False), ([[8, 0], [0, 2048]], 64, 0, True),
+         ([[64, 0], [0, 64]], 100, 1, False), ([[64, 0], [0, 64]], 101, 1, True), ([[32, 0], [0, 64]], 1, 1, True),
+         ([[64, 0], [0, 128]], 64, 1, False), ([[16, 0, 0], [0, 16, 0], [0, 0, 32]], 200, 1, False),
+         ([[60, 0], [0, 72]], 64, 1, True), ([[8192]], 64, 1, True)]
+
+
+@pytest.mark.parametrize("M,batch,c128,whole", WHOLE)
+def test_whole_signals_in_a_tile(fake, M, batch, c128, whole):
+    st, h = _create(fake, M, batch, c128)
+    assert st == 0
+    fake.fake_reset()
+    assert fake.pfft_forward(h, 4096, 8192, None) == 0
+    kernels = [k for k, *_ in _launches(fake)]
+    assert (len(kernels) == 1 and "mixed_kernel" in kernels[0]) == whole
+    fake.pfft_plan_destroy(h)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,batch,c128,whole", WHOLE)
+def test_transform_of_many_signals(M, batch, c128, whole):
+    m = abs(L.det(M))
+    plan = pf.PatternFFT(M, batch, torch.complex128 if c128 else torch.complex64)
+    tol = TOL["c128" if c128 else "c64"]
+    c = SI.complex_normal(batch, m, seed=m % 71, dtype=np.complex128 if c128 else np.complex64)
+    y = plan.forward(torch.from_numpy(c).cuda())
+    slots = SI.sample_slots(m, 64, seed=3)
+    assert rel_l2(y.cpu().numpy()[-2:, slots], oracle.pattern_fft(M, c[-2:], out_slots=slots)) <= tol
+    assert rel_l2(plan.inverse(y).cpu().numpy(), c) <= tol
+
+
 def test_complex128_cycles_with_factors_11_and_13(fake):
     """Two equal cycles of n points, 11 or 13 dividing n: the row and the column
     each take a tile of 512 threads, 16 points a thread, wherever the other
