@@ -95,8 +95,8 @@ size_t ebytes(int dtype) { return dtype == PFFT_C64 ? 8 : 16; }
 double tile_cost(const MixDesc& a) {
   double w = 0;
   for (int i = 0; i < a.nstages; ++i) {
-    const int R = a.st[i].R;
-    w += i < a.ndirect ? R / 4.0 : std::log2(double(R));
+    const MixStage& s = a.st[i];
+    w += s.R >= kMixMinDirect ? s.tw / 4.0 : std::log2(double(s.R));
   }
   return double(a.T) * a.L * (w + 2.0);
 }

@@ -331,7 +331,7 @@ __device__ __forceinline__ void mix_locate(const MixStage& s, int b, int& base, 
 template <typename C, int NQ, int Q>
 __device__ __noinline__ void mix_direct_pairs(C* sm, const MixStage& s, int nbf, const C* P, const int* gp) {
   using Rl = decltype(C::x);
-  const int R = s.R, h = (R - 1) / 2;
+  const int R = s.tw, h = (R - 1) / 2;
   const int istep = s.aR * s.sig, ostep = s.Ns * s.sig;
   const int items = nbf * ((h + Q - 1) / Q);
   C A[NQ][Q], B[NQ][Q], y0[NQ];
@@ -405,7 +405,7 @@ __device__ __noinline__ void mix_direct_pairs(C* sm, const MixStage& s, int nbf,
 template <typename C>
 __device__ __noinline__ void mix_direct(C* sm, const MixDesc& a, const MixStage& s) {
   constexpr int NA = kMixPoints / 2;
-  const int R = s.R, h = (R - 1) / 2;
+  const int R = s.tw, h = (R - 1) / 2;
   const int nbf = a.n / R;
   const int nthr = blockDim.x;
   const int istep = s.aR * s.sig;
@@ -486,10 +486,13 @@ __device__ __forceinline__ void mix_stages_of4(C* sm, const MixDesc& a, int& i, 
 
 template <typename C>
 __device__ __forceinline__ void mix_stages(C* sm, const MixDesc& a) {
-  int i = 0;
+  int i = 0, R = a.nstages ? a.st[0].R : 0;
 #pragma unroll 1
-  for (; i < a.ndirect; ++i) mix_direct<C>(sm, a, a.st[i]);
-  int R = i < a.nstages ? a.st[i].R : 0;
+  while (R >= kMixMinDirect) {
+    mix_direct<C>(sm, a, a.st[i]);
+    ++i;
+    R = i < a.nstages ? a.st[i].R : 0;
+  }
   mix_stages_of4<C, 15, 13, 11, 9>(sm, a, i, R);
   mix_stages_of4<C, 16, 14, 12, 10>(sm, a, i, R);
   mix_stages_of4<C, 8, 7, 6, 5>(sm, a, i, R);

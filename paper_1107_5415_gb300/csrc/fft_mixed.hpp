@@ -27,6 +27,7 @@ constexpr int kMixPoints = 16;  // points a thread holds between the barriers of
 // Register butterflies reach radix 16; primes from 17 up are direct stages, and so
 // are 11 and 13 in a complex128 pencil that needs more than 11 or 13 points a thread.
 constexpr int kMixMinDirect = 17;
+constexpr int kMixDirect = 2048;  // marks the radix of such a stage (one comparison tells the kernel)
 // Output pairs of one work item of a direct stage: kMixWide when every item
 // has a thread of its own, else kMixNarrow with at most kMixItems per thread;
 // kMixNarrow either way in complex128 (mix_direct_pairs).
@@ -54,9 +55,10 @@ constexpr int kMixThreadsC64 = 1024, kMixThreadsC128 = 512;
 // a unit of its own (MixDesc::ws_in, ws_out), which divides the step of the first
 // stage's inputs or of the last one's outputs.
 struct MixStage {
-  int R, aR, sig, Ns, blk;
+  int R;        // plus kMixDirect for a direct stage of a radix below kMixMinDirect
+  int aR, sig, Ns, blk;
   int istep, ostep, ipad, opad;
-  int tw;       // twiddles of the stage in the stage table: [b][k] (MixTableArgs)
+  int tw;       // twiddles of the stage in the stage table: [b][k] (MixTableArgs); direct stages: the radix
   int gen;      // direct stages: offset of g^t mod R (R - 1 ints) in the integer table
   int twstep;   // direct stages: step of the root table per unit of exp(-2 pi i / (Ns R))
   FastDiv div_in, div_out;  // by the pad units of the inputs and of the outputs
@@ -76,7 +78,7 @@ struct alignas(16) MixDesc {
   int pitch_in, pitch_out;  // their distances of the rows
   const int *psin, *psout;  // row tiles: padded element position of each column position
   int dir_off;        // tables of the direct stages after the tile (elements)
-  int nstages, ndirect;  // the first ndirect stages are direct sums
+  int nstages;
   int tw_n;           // order of the root table
   int load_mode, store_mode, conj_in, conj_out;
   int in_sel, out_sel;  // grouped launches: in / out are byte offsets into base[in_sel] / base[out_sel]

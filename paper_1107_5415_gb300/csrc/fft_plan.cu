@@ -507,7 +507,6 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
   a.tw_n = kind == MIX_COL && P.tw_col ? P.col_n : P.nD;
   const int tstride = kind == MIX_COL || a.lay ? T : 1;  // stride of the pencil index in the tile
   a.nstages = int(S.st.size());
-  a.ndirect = S.ndirect;
   std::vector<Radix> rad;
   int rmax = 0;
   int unit = 0;  // pad unit, once padded
@@ -532,9 +531,13 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
     s.div_out.init(uint32_t(s.opad ? unit : 1 << 30));
     s.div_sig.init(uint32_t(s.sig));
     s.div_nb.init(uint32_t(std::max(1, a.n / s.R)));
+    rad.push_back({s.R, i < S.ndirect});
+    if (i < S.ndirect) {
+      rmax = std::max(rmax, s.R);
+      s.tw = s.R;
+      if (s.R < kMixMinDirect) s.R += kMixDirect;
+    }
     a.st[i] = s;
-    rad.push_back({s.R, i < a.ndirect});
-    if (i < a.ndirect) rmax = std::max(rmax, s.R);
   }
   a.nthreads = mix_threads(rad, a.n, max_threads, P.dtype);
   // a launch that leaves the chip idle gets twice the threads that its stages ask
