@@ -292,8 +292,8 @@ int mix_min_points(int L, const pfft_plan_s& P) { return (L + mix_max_threads(P)
 // (128 registers a thread).  Tiles of a multiple of four warps put the warps of a
 // last, partial turn on the same schedulers, others spread them.  A tile alone on
 // its SM loads and stores beside no other's sums (4%).
-double direct_time(const std::vector<Radix>& radices, int n, int t) {
-  const int tiles = kMixThreadsC128 / t, per_tile = t / 32;
+double direct_time(const std::vector<Radix>& radices, int n, int t, bool alone = false) {
+  const int tiles = alone ? 1 : kMixThreadsC128 / t, per_tile = t / 32;
   double time = 0;
   for (const Radix& r : radices) {
     if (!r.direct) continue;
@@ -303,11 +303,11 @@ double direct_time(const std::vector<Radix>& radices, int n, int t) {
       time += double(h) * (per_tile % 4 ? (tiles * warps + 3) / 4 : tiles * ((warps + 3) / 4));
     }
   }
-  return time / tiles * (tiles == 1 ? 1.04 : 1.0);
+  return time / tiles * (tiles == 1 && !alone ? 1.04 : 1.0);
 }
 
-// Threads of a mixed-radix tile of n points.
-int mix_threads(const std::vector<Radix>& radices, int n, int max_threads, int dtype) {
+// Threads of a mixed-radix tile of n points (alone: no other tile shares its SM).
+int mix_threads(const std::vector<Radix>& radices, int n, int max_threads, int dtype, bool alone = false) {
   int need = (n + kMixPoints - 1) / kMixPoints;
   bool sums = false;
   for (const Radix& r : radices) {
@@ -325,9 +325,18 @@ int mix_threads(const std::vector<Radix>& radices, int n, int max_threads, int d
   }
   need = (need + 31) / 32 * 32;
   if (dtype == PFFT_C64 || !sums) return need;
+  // level ones: the fewest turns, then the fewest threads
+  auto turns = [&](int t) {
+    int u = 0;
+    for (const Radix& r : radices)
+      if (r.direct) u += (n / r.R * (((r.R - 1) / 2 + kMixNarrow - 1) / kMixNarrow) + t - 1) / t;
+    return u;
+  };
   int best = need;
-  for (int t = need; t <= max_threads; t += 32)
-    if (direct_time(radices, n, t) <= direct_time(radices, n, best)) best = t;
+  for (int t = need; t <= max_threads; t += 32) {
+    const double a = direct_time(radices, n, t, alone), b = direct_time(radices, n, best, alone);
+    if (a < b || (a == b && turns(t) < turns(best))) best = t;
+  }
   return best;
 }
 
@@ -539,11 +548,11 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
     }
     a.st[i] = s;
   }
-  a.nthreads = mix_threads(rad, a.n, max_threads, P.dtype);
+  const i64 ctas = i64(a.groups) * (kind == MIX_WHOLE ? 1 : P.batch);
+  a.nthreads = mix_threads(rad, a.n, max_threads, P.dtype, !P.generic_only && ctas <= kSMs);
   // a launch that leaves the chip idle gets twice the threads that its stages ask
   // for, as long as all of it stays resident: half the turns of every load and store
   const int more = (a.n + kMixFewPoints - 1) / kMixFewPoints;
-  const i64 ctas = i64(a.groups) * (kind == MIX_WHOLE ? 1 : P.batch);
   if (!P.generic_only && more <= max_threads && ctas * more <= i64(kSMs) * max_threads)
     a.nthreads = std::max(a.nthreads, (more + 31) / 32 * 32);
   // each thread keeps one column (or, of a [element][row] tile, one row in turns of four elements)
@@ -590,7 +599,7 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
 // 243]] x 7, two columns of 3240 points in 544 threads: 3.60 and 3.24; a mix of 512
 // patterns: 2.14 and 2.11; but two of 3850 points in 704 threads lose 7%).
 // Complex128 tiles with direct sums hold another number of pencils, up to `most`
-// points, where that takes the launch at least 3% less by direct_time.
+// points, where the launch is at least 3% shorter for it.
 pfft_status mix_choose(pfft_plan_s& P, int kind, int cap, int budget, int most, int lanes, int ctas) {
   pfft_status st = mix_stages(P, kind);
   if (st != PFFT_OK) return st;
@@ -604,33 +613,36 @@ pfft_status mix_choose(pfft_plan_s& P, int kind, int cap, int budget, int most, 
     if (n > (2 * T <= lanes ? std::max(most, budget) : budget) || (few && 2 * T > lanes && n > 256)) break;
     T *= 2;
   }
-  const MixStages& S = P.stages[P.max2 == 16 ? 0 : 1][kind];
-  if (P.dtype == PFFT_C128 && S.ndirect) {
-    std::vector<Radix> rad;
-    for (int i = 0; i < int(S.st.size()); ++i) rad.push_back({S.st[i].R, i < S.ndirect});
-    auto time = [&](int x) {  // a pencil
-      return mix_configure(P, kind, x) == PFFT_OK ? direct_time(rad, x * L, P.mix[kind].nthreads) / x : 1e30;
-    };
-    // adjacent columns first as many as there may be, rows and signals as above
-    int best = T;
-    double least = lanes > 1 ? 1e30 : time(T);
-    for (int x = 16; x >= 1; x /= 2) {
-      if (x > cap || x > count || (x > 1 && (i64(x) * L > most || (count + x - 1) / x * signals < ctas))) continue;
-      const double c = time(x);
-      if (c < 0.97 * least) {
-        least = c;
-        best = x;
-      }
-    }
-    return mix_configure(P, kind, best);
-  }
   for (;; T /= 2) {
     st = mix_configure(P, kind, T);
     const int max = P.dtype == PFFT_C64 ? kMixThreadsC64 : kMixThreadsC128, t = P.mix[kind].nthreads, half = (t / 2 + 31) / 32 * 32;
-    if (T == 1) return st;
+    if (T == 1) break;
     if (st != PFFT_OK) continue;
-    if (t <= max / 2 || (T * elem_bytes(P.dtype) <= 16 && 4 * (max / half * half) < 5 * t)) return st;
+    if (t <= max / 2 || (T * elem_bytes(P.dtype) <= 16 && 4 * (max / half * half) < 5 * t)) break;
   }
+  const MixStages& S = P.stages[P.max2 == 16 ? 0 : 1][kind];
+  if (st != PFFT_OK || P.dtype == PFFT_C64 || !S.ndirect) return st;
+  std::vector<Radix> rad;
+  for (int i = 0; i < int(S.st.size()); ++i) rad.push_back({S.st[i].R, i < S.ndirect});
+  // Clocks of the launch on its busiest SM (grouped tiles: on average): 16 multiply-adds
+  // of a warp a step at half a lane a clock and scheduler, and 5000 that a tile takes
+  // besides ([[16336]] x 8: 0.67 ms a direction, 1.09 with pencils for a full chip).
+  auto time = [&](int x) {
+    if (mix_configure(P, kind, x) != PFFT_OK) return 1e30;
+    const double tiles = double((count + x - 1) / x) * signals / kSMs;
+    if (P.generic_only) return (1024 * direct_time(rad, x * L, P.mix[kind].nthreads) + 5000) * tiles;
+    return (1024 * direct_time(rad, x * L, P.mix[kind].nthreads, tiles <= 1) + 5000) * std::ceil(tiles);
+  };
+  double least = 0.97 * time(T);
+  for (int x = 16; x >= 1; x /= 2) {
+    if (x > cap || x > count || (x > 1 && i64(x) * L > most)) continue;
+    const double c = time(x);
+    if (c < least) {
+      least = c;
+      T = x;
+    }
+  }
+  return mix_configure(P, kind, T);
 }
 
 // Register-resident column pass over two pencil axes (fft_fast2.cuh): the
