@@ -889,7 +889,12 @@ pfft_status pfft::plan_host(pfft_plan_s& P, int d, const int64_t* Mv) {
       // pencils: above 2048 points eight adjacent pencils (64-byte accesses) no
       // longer leave room for a second tile on the SM, above 4096 the accesses
       // fall to 16 bytes, and fewer than eight rows lambda_a are not eight
-      // adjacent slots.  Weights measured with the passes' own times: 10800 =
+      // adjacent slots.  A long complex64 column costs three times what a long row
+      // does: its lanes are all the adjacent accesses it has on either side ([[4096,
+      // 1024], [0, 8192]] x 1, cycles 1024 and 32768, forward / inverse: 745 / 815 us with
+      // rows of 4096 and columns of 8192, 602 / 669 with 8192 and 4096, 780 / 742 before
+      // the mixed-radix tiles; in complex128 they are nearly level, [[1024, 256], [0,
+      // 4096]] x 1 with rows or columns of 4096: 630 and 650 us).  Weights measured with the passes' own times: 10800 =
       // 16 15 15 3 runs at 28 instructions a point and stage.
       double cr = 0, cc = 0;
       std::vector<int> pen(P.pen.begin(), P.pen.end());
@@ -897,7 +902,8 @@ pfft_status pfft::plan_host(pfft_plan_s& P, int d, const int64_t* Mv) {
       if (!mix_fits(P, {int(nb)}, int(nb), direct, &cr) || !mix_fits(P, pen, int(lb), direct, &cc)) continue;
       const int unit = P.dtype == PFFT_C64 ? 1024 : 512;
       auto long_tile = [&](i64 L) { return L > 8 * unit ? 60.0 : L > 4 * unit ? 30.0 : L > 2 * unit ? 12.0 : L > unit ? 3.0 : 0.0; };
-      const double c = cr + cc + long_tile(nb) + long_tile(lb) + 3.0 * std::max<i64>(0, 8 - na);
+      const double column = P.dtype == PFFT_C64 && lb > 4 * unit ? 3.0 : 1.0;
+      const double c = cr + cc + long_tile(nb) + column * long_tile(lb) + 3.0 * std::max<i64>(0, 8 - na);
       if (c < best_cost) {
         best_cost = c;
         best = int(nb);

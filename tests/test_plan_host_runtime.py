@@ -159,6 +159,18 @@ def test_bulk_copies_only_where_they_are_aligned(fake, n, inverse):
     fake.pfft_plan_destroy(h)
 
 
+@pytest.mark.gpu
+def test_long_cycle_beside_a_long_pencil():
+    """Cycles 1024 and 32768: rows of 8192, columns over axes of 1024 and 4."""
+    M = [[4096, 1024], [0, 8192]]
+    m = abs(L.det(M))
+    plan = pf.PatternFFT(M, 1)
+    c = SI.complex_normal(1, m, seed=67)
+    y = plan.forward(torch.from_numpy(c).cuda())
+    slots = SI.sample_slots(m, 16, seed=3)
+    assert rel_l2(y.cpu().numpy()[:, slots], oracle.pattern_fft(M, c, out_slots=slots)) <= TOL["c64"]
+    assert rel_l2(plan.inverse(y).cpu().numpy(), c) <= TOL["c64"]
+
 # matrix, signals, complex128, whole signals in one tile
 WHOLE = [([[512]], 4096, 0, True), ([[1024]], 304, 0, True), ([[1024]], 305, 0, False), ([[4096]], 1, 0, False),
          ([[16384]], 70, 0, False), ([[8192]], 1, 0, False), ([[4096]], 1, 1, True), ([[90, 0], [0, 90]], 1, 0, True),
