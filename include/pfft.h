@@ -261,8 +261,9 @@ enum {
  * Device memory owned by the plan: two workspaces of |det M| / 2 * batch
  * elements (more than one level), the phase tables, and, for complex64 plans
  * of four or more signals, the per-fibre symbols of every level (16 bytes
- * per point of G(N_l^T), about 16 |det M| bytes in all), which decompose
- * reads when it runs up to three levels in one launch.
+ * per point of G(N_l^T), about 16 |det M| bytes in all), which decompose,
+ * reconstruct and adjoint read when they run up to three levels in one launch
+ * (without them only decompose does).
  * Returns PFFT_ERR_NOT_INTEGRAL if some J_l^{-1} M_l is not integral. */
 pfft_status pwt_plan_create(pwt_plan* out, int d, const int64_t* M, int levels, const int64_t* J,
                             int symbol, double eta, int64_t batch, int dtype, unsigned flags);
@@ -362,10 +363,11 @@ enum {
    * split unit -- in ONE kernel launch whose CTAs take work units from a
    * device queue in dependency order; a column tile waits (bounded) until
    * its pattern's row tiles are done, a split unit until the pattern's
-   * coefficients are.  Results equal the grouped launches' up to rounding
-   * (the same tiles compiled into another kernel).  All units run with the
-   * largest tile's threads and shared memory (fewer CTAs per SM when one
-   * pattern needs a large tile). */
+   * coefficients are.  All units run with the largest tile's threads and
+   * shared memory, so the patterns are planned for tiles of at most half an
+   * SM's threads where they have such a plan: tiles, radices and the split of a
+   * long cycle may differ from the grouped launches', whose results these
+   * equal up to rounding. */
   PFFT_BATCH_ONE_LAUNCH = 8u
 };
 

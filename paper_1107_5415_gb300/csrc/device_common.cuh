@@ -43,9 +43,10 @@ template <typename C>
 __device__ __forceinline__ C csub(C a, C b) { return cmake<C>(a.x - b.x, a.y - b.y); }
 // Sums of the butterflies.  PK: one packed instruction per complex64 sum (the
 // same two IEEE sums), for the kernels bound by instruction issue (M = [[512,
-// 128], [0, 512]] x 16 there and back: 0.1024 -> 0.0977 ms); the pipelined passes,
-// bound by their memory phases, keep the plain ones, which the compiler may
-// contract with a preceding product (2.185 against 2.197 ms for the 2^24 x 8 step).
+// 128], [0, 512]] x 16 there and back: 0.1024 -> 0.0977 ms); the pipelined row
+// pass and the pipelined column pass of 1024 points, bound by their memory phases,
+// keep the plain ones, which the compiler may contract with a preceding product
+// (2.185 against 2.197 ms for the 2^24 x 8 step).
 template <bool PK, typename C>
 __device__ __forceinline__ C bsum(C a, C b) {
   if constexpr (PK && sizeof(C) == 8)

@@ -315,10 +315,10 @@ __device__ __noinline__ void run_direct_stage(C* sm, const PassArgs& a, const St
 // register allocation of each butterfly size separate (mixing sizes inside
 // one loop body makes the allocator spill).  POW2 kernels carry only the
 // power-of-two regions.
-template <typename C, int EPT, bool COLS, bool POW2, bool PAD, bool TCK>
+template <typename C, int EPT, bool COLS, bool POW2, bool PAD>
 __device__ void run_all_stages(C* sm, const PassArgs& a, const C* __restrict__ tw) {
   int i = 0;
-  constexpr bool kC64 = sizeof(C) == 8 && TCK;  // TCK = false: no tensor-core code in the kernel
+  constexpr bool kC64 = sizeof(C) == 8;
   if constexpr (!POW2) {
     _Pragma("unroll 1") for (int q = 0; q < a.cnt[kDirectRegion]; ++q, ++i)
         run_direct_stage<C, EPT, COLS, PAD>(sm, a, a.st[i], tw);
@@ -394,7 +394,7 @@ __device__ void run_all_stages(C* sm, const PassArgs& a, const C* __restrict__ t
 // The body takes the tile (blockIdx.x of a plain launch) and the signal index
 // (blockIdx.y) as arguments so that the grouped launches of many patterns
 // (batch_kernels.cu) run the same code on a per-CTA copy of the arguments.
-template <typename C, int EPT, bool POW2, bool PAD, bool TCK = true>
+template <typename C, int EPT, bool POW2, bool PAD>
 __device__ __forceinline__ void row_pass_body(const PassArgs& a, int tile, int sig, C* sm) {
   const C* __restrict__ tw = static_cast<const C*>(a.tw);
   const C* __restrict__ in = static_cast<const C*>(a.in) + (int64_t)sig * a.m;
@@ -439,7 +439,7 @@ __device__ __forceinline__ void row_pass_body(const PassArgs& a, int tile, int s
     if (sidx[k] >= 0) sm[phys<PAD>(sidx[k])] = (a.load_mode == MAP_WS) ? v[k] : maybe_conj(v[k], a.conj_in);
   }
   __syncthreads();
-  run_all_stages<C, EPT, false, POW2, PAD, TCK>(sm, a, tw);
+  run_all_stages<C, EPT, false, POW2, PAD>(sm, a, tw);
   using Rl = decltype(C::x);
   const Rl sc = Rl(a.scale);
 #pragma unroll
@@ -499,7 +499,7 @@ __device__ __forceinline__ int shear_index(const PassArgs& a, int j, const int* 
 // Column pass: all LB rows of T adjacent workspace columns per CTA, smem
 // layout [i][t].  The DFT runs over the (D-1) cycles inside the pencil.
 // Loads and stores are batched per thread as in the row pass.
-template <typename C, int EPT, bool POW2, bool PAD, bool TCK = true>
+template <typename C, int EPT, bool POW2, bool PAD>
 __device__ __forceinline__ void col_pass_body(const PassArgs& a, int tile, int sig, C* sm) {
   const C* __restrict__ tw = static_cast<const C*>(a.tw);
   const C* __restrict__ in = static_cast<const C*>(a.in) + (int64_t)sig * a.m;
@@ -547,7 +547,7 @@ __device__ __forceinline__ void col_pass_body(const PassArgs& a, int tile, int s
     if (sidx[k] >= 0) sm[phys<PAD>(sidx[k])] = maybe_conj(v[k], a.conj_in);
   }
   __syncthreads();
-  run_all_stages<C, EPT, true, POW2, PAD, TCK>(sm, a, tw);
+  run_all_stages<C, EPT, true, POW2, PAD>(sm, a, tw);
   using Rl = decltype(C::x);
   const Rl sc = Rl(a.scale);
   const bool ws_out = a.store_mode == MAP_WS;
@@ -583,13 +583,13 @@ __device__ __forceinline__ void col_pass_body(const PassArgs& a, int tile, int s
 template <typename C, int EPT, bool POW2, bool PAD, int MINB = 1>
 __global__ void __launch_bounds__(kMaxThreads, MINB) row_pass_kernel(PassArgs a) {
   extern __shared__ unsigned char smem_raw[];
-  row_pass_body<C, EPT, POW2, PAD, EPT == 32>(a, blockIdx.x, blockIdx.y, reinterpret_cast<C*>(smem_raw));
+  row_pass_body<C, EPT, POW2, PAD>(a, blockIdx.x, blockIdx.y, reinterpret_cast<C*>(smem_raw));
 }
 
 template <typename C, int EPT, bool POW2, bool PAD, int MINB = 1>
 __global__ void __launch_bounds__(kMaxThreads, MINB) col_pass_kernel(PassArgs a) {
   extern __shared__ unsigned char smem_raw[];
-  col_pass_body<C, EPT, POW2, PAD, EPT == 32>(a, blockIdx.x, blockIdx.y, reinterpret_cast<C*>(smem_raw));
+  col_pass_body<C, EPT, POW2, PAD>(a, blockIdx.x, blockIdx.y, reinterpret_cast<C*>(smem_raw));
 }
 
 // Allow the largest dynamic shared-memory size and prefer the maximum shared

@@ -13,21 +13,15 @@
 // instructions.  A thread holds at most 16 points and 64 registers, so 1024
 // threads are resident per SM, in one tile or several.
 //
-// Measured there and back (forward and inverse), before (one shared-memory
-// kernel over radices 16, 8, 4, 2, 3, 5, 7, indices from tables, 32 points per
-// thread) and now: [[1200, 240], [0, 1080]] x 8: 1.538 -> 0.448 ms (171 thread
-// instructions a point in the row pass, 450 before); [[2048, 8], [0, 2048]] x 8:
-// 1.993 -> 1.027 ms; [[64, 16], [-16, 64]] x 1: 0.089 -> 0.033 ms; a mix of 512
-// patterns: 3.65 -> 2.84 ms.  With the setups of a thread's loops trimmed (stage
-// tests by group, shears by multiply-high, one row per thread of a split tile):
-// 0.402, 0.964, 0.033 and, with the 32-bit splits, 2.33 ms.  With the padding of the
-// workspace side (pad_unit), eight points a thread in launches that leave the chip
-// idle and two or more tiles per SM wherever the pencils allow it: 0.388, 0.958,
-// 0.025 (0.029 with sixteen) and 2.20 ms.  Reading the workspace
-// straight into the first butterflies of a column tile and writing it from the last
-// ones saves instructions in such tiles but costs every other stage (0.415 ms for
-// the first), and so does a copy of the load and store loops without bounds checks
-// (0.393 against 0.389: the instruction cache).
+// There and back (forward and inverse), in one shared-memory kernel over radices 16,
+// 8, 4, 2, 3, 5, 7 with indices from tables and here: [[1200, 240], [0, 1080]] x 8: 1.538
+// and 0.39 ms (450 and 151 thread instructions a point in the row pass); [[2048, 8],
+// [0, 2048]] x 8: 1.99 and 0.96 ms; [[64, 16], [-16, 64]] x 1: 88 and 25 us; a mix of
+// 512 patterns, split once: 3.65 and 2.2 ms.  Reading the workspace straight into the
+// first butterflies of a column tile and writing it from the last ones saves
+// instructions in such tiles but costs every other stage (0.415 ms for the first), and
+// so does a copy of the load and store loops without bounds checks (0.393 against
+// 0.389: the instruction cache).
 #pragma once
 #include <cuda_runtime.h>
 

@@ -101,14 +101,6 @@ struct alignas(16) MixDesc {
 };
 static_assert(sizeof(MixDesc) % 16 == 0, "descriptors are copied in 16-byte pieces");
 
-// What a launch sets on top of a plan's descriptor.
-struct MixCall {
-  int load_mode, store_mode, conj_in, conj_out;
-  double scale;
-  const void* in;
-  void* out;
-};
-
 // Stage twiddles: entry (s, b, k) = exp(-2 pi i k 2^b / (Ns R)), or, for the
 // stages of fused_dft (fused), factor b of its levels: exp(-2 pi i (k + c Ns) /
 // (Ns 2^l)), b = fused_first(l) + c.

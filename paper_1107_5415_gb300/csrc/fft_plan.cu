@@ -488,10 +488,9 @@ pfft_status mix_stages(pfft_plan_s& P, int kind) {
 }
 
 // Points per thread of a launch that does not fill the chip.  [[64, 16], [-16,
-// 64]] x 1 there and back: 28.4 us with 16, 26.3 with 8, 29.7 with 5; [[300, 60],
+// 64]] x 1 there and back, called from Python: 28.7 us with 16, 24.6 with 8, 29.7 with 5; [[300, 60],
 // [0, 240]] x 1: 31.1 and 28.2 us; [[60, 24], [0, 72]] x 1 in complex128: 62 and 50.6 us.
 constexpr int kMixFewPoints = 8;
-constexpr int kSMs = 152;
 
 // The descriptor of a kind of tile with T pencils (T a power of two; any T for
 // row tiles in [row][element] order and whole tiles).
@@ -549,11 +548,11 @@ pfft_status mix_configure(pfft_plan_s& P, int kind, int T) {
     a.st[i] = s;
   }
   const i64 ctas = i64(a.groups) * (kind == MIX_WHOLE ? 1 : P.batch);
-  a.nthreads = mix_threads(rad, a.n, max_threads, P.dtype, !P.generic_only && ctas <= kSMs);
+  a.nthreads = mix_threads(rad, a.n, max_threads, P.dtype, !P.generic_only && ctas <= P.nsm);
   // a launch that leaves the chip idle gets twice the threads that its stages ask
   // for, as long as all of it stays resident: half the turns of every load and store
   const int more = (a.n + kMixFewPoints - 1) / kMixFewPoints;
-  if (!P.generic_only && more <= max_threads && ctas * more <= i64(kSMs) * max_threads)
+  if (!P.generic_only && more <= max_threads && ctas * more <= i64(P.nsm) * max_threads)
     a.nthreads = std::max(a.nthreads, (more + 31) / 32 * 32);
   // each thread keeps one column (or, of a [element][row] tile, one row in turns of four elements)
   const int keep = a.lay ? 4 * T : tstride;
@@ -629,7 +628,7 @@ pfft_status mix_choose(pfft_plan_s& P, int kind, int cap, int budget, int most, 
   // besides ([[16336]] x 8: 0.67 ms a direction, 1.09 with pencils for a full chip).
   auto time = [&](int x) {
     if (mix_configure(P, kind, x) != PFFT_OK) return 1e30;
-    const double tiles = double((count + x - 1) / x) * signals / kSMs;
+    const double tiles = double((count + x - 1) / x) * signals / P.nsm;
     if (P.generic_only) return (1024 * direct_time(rad, x * L, P.mix[kind].nthreads) + 5000) * tiles;
     return (1024 * direct_time(rad, x * L, P.mix[kind].nthreads, tiles <= 1) + 5000) * std::ceil(tiles);
   };
@@ -1283,7 +1282,7 @@ pfft_status pfft::plan_device(pfft_plan_s& P) {
       if (launch_whole_maps(a, P.rowp.PI, P.maps, P.maps + P.m, 0) != 0) return PFFT_ERR_CUDA;
     }
     // a launch of its own leaves at least two tiles per SM where the lanes of its accesses allow
-    const pfft_status st = mix_tile(P, kind, 2048, P.generic_only ? 0 : 304);
+    const pfft_status st = mix_tile(P, kind, 2048, P.generic_only ? 0 : 2 * P.nsm);
     if (st != PFFT_OK) return st;
   }
   // stage twiddle tables of the register-resident passes, gathered on the
