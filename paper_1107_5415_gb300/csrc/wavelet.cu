@@ -495,14 +495,16 @@ static int launch_fused_t(pwt_plan_s* P, int l, const void* coef, const void* sc
   // fibres of the last level over CTAs of kFuseThreads threads, about
   // kFuseWaves resident waves; the signals split into chunks only when the
   // fibres are too few, a synthesis keeping two signals a thread, whose loads are in
-  // flight together (seven levels of [[1024, 1024], [-1024, 1024]] x 4 back: 64.6 us
-  // with one, 60.7 with two, 63.3 in seven launches)
+  // flight together, where that leaves two CTAs an SM (seven levels of [[1024, 1024],
+  // [-1024, 1024]] x 4 back: 64.6 us with one, 60.7 with two, 63.3 in seven launches;
+  // without that limit the twelve levels x 16 take 168.6 us instead of 167.2)
   const long long mN = P->lv[l + F - 1].mN, cap = 152LL * kFuseWaves;
   long long x = (mN + kFuseThreads - 1) / kFuseThreads;
   if (x > cap) x = cap;
   long long y = (cap + x - 1) / x;
   if (y > P->batch) y = P->batch;
-  const int chunk = std::max(MODE && P->batch > 1 ? 2 : 1, int((P->batch + y - 1) / y));
+  const bool pairs = MODE != 0 && x * ((P->batch + 1) / 2) >= 2 * 152;
+  const int chunk = std::max(pairs ? 2 : 1, int((P->batch + y - 1) / y));
   const unsigned gy = unsigned((P->batch + chunk - 1) / chunk);
   auto p = [](const void* q) { return static_cast<float2*>(const_cast<void*>(q)); };
   float2* w[3] = {nullptr, nullptr, nullptr};
